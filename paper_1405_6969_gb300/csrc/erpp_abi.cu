@@ -260,9 +260,10 @@ erpp_status derive_ctx(const erpp_params* p, erpp_ctx* c) {
   double cpmin = std::min(kp.cp[0], std::min(kp.cp[1], kp.cp[2]));
   if (cpmin < 1.0) return ERPP_EINVAL;  // r_c must reach at least one grid spacing
   // A window starts at most floor(c') nodes below the particle's cell and holds
-  // at most floor(2 c') + 1 nodes (one more when 2 c' sits within rounding of
-  // an integer).
-  kp.hlo = (int)floor(cpmax);
+  // at most floor(2 c') + 1 nodes (one more when c', 2 c' sits within rounding
+  // of an integer: with c' = 3 - 2^-51 the window of a particle on a node still
+  // rounds to three nodes below it).
+  kp.hlo = (int)floor(cpmax + 1e-6);
   kp.xs = (int)floor(2.0 * cpmax + 1e-6) + 1;
   if (kp.hlo > 15 || kp.xs > 31) return ERPP_EINVAL;  // windows of at most 31 nodes
   kp.dV = kp.dx[0] * kp.dx[1] * kp.dx[2];
@@ -314,7 +315,7 @@ erpp_status derive_ctx(const erpp_params* p, erpp_ctx* c) {
   // in rows of 96 floats with an x-halo of xhlo nodes below and xhhi above
   // (the whole x-window of every particle whose home cell is in the tile);
   // 8 x 8 in y and z.
-  kp.xhlo = (int)floor(kp.cp[0]);
+  kp.xhlo = (int)floor(kp.cp[0] + 1e-6);
   kp.xhhi = kp.xhlo + 1;
   kp.xlmin = (int)floor(2.0 * kp.cp[0]);
   kp.xxs = (int)floor(2.0 * kp.cp[0] + 1e-6) + 1;
@@ -356,7 +357,7 @@ erpp_status derive_ctx(const erpp_params* p, erpp_ctx* c) {
   if (prec == ERPP_FP32 && kp.xxs <= 16 && yxs <= 16) {
     erpp_kparams k4 = kp;
     k4.design = 4;
-    k4.yhlo = (int)floor(kp.cp[1]);
+    k4.yhlo = (int)floor(kp.cp[1] + 1e-6);
     k4.yhhi = k4.yhlo + 1;
     const int hx = k4.xhlo + k4.xhhi, hy = k4.yhlo + k4.yhhi;
     // Tile widths: the requested size (x: 64), raised to the halo depth so
