@@ -43,6 +43,7 @@ erpp_status set_cuda_err(cudaError_t e) {
 }
 
 void free_scratch(erpp_ctx* c) {
+  erpp::bricks_free(c);
   cudaFree(c->geo_t);
   cudaFree(c->geo_c);
   cudaFree(c->xw);
@@ -127,6 +128,7 @@ erpp_status ensure_capacity(erpp_ctx* c, int64_t n) {
       e = cudaMalloc(&c->lap_part, sizeof(float4) * (size_t)ecap);
     if (e == cudaSuccess) e = cudaMalloc(&c->piece_slot, sizeof(int32_t) * (size_t)ecap);
     c->entries_cap = ecap;
+    if (e == cudaSuccess) e = bricks_alloc(c, cap);
   }
   if (e != cudaSuccess) {
     free_scratch(c);
@@ -152,6 +154,7 @@ erpp_status alloc_tile_tables(erpp_ctx* c) {
   if (e == cudaSuccess) e = cudaMalloc(&c->scan_tmp, sizeof(int32_t) * (nbins / 4096 + 1));
   const size_t hb = (size_t)kp.ntiles * (size_t)kp.halo_per_tile;
   if (e == cudaSuccess) e = cudaMalloc(&c->halo, sizeof(float) * hb);
+  if (e == cudaSuccess) e = erpp::bricks_alloc_tables(c);
   return set_cuda_err(e);
 }
 
@@ -162,6 +165,7 @@ void free_tile_tables(erpp_ctx* c) {
   cudaFree(c->halo);
   c->tile_cnt = c->tile_start = c->scan_tmp = nullptr;
   c->halo = nullptr;
+  erpp::bricks_free_tables(c);
 }
 
 // Cell-block tables of the other weights' particle sort (8 x 8 x 8-node blocks
@@ -596,6 +600,10 @@ erpp_status erpp_gather_backward(erpp_ctx* c, int64_t n, const double* const x[3
     if (s) return s;
     if (c->fp64) {
       e = erpp::launch_scatter_f64(c, n, x, g, c->kp.dV, (double*)du, st);
+    } else if (erpp::use_bricks(c, n)) {
+      e = erpp::brick_sort(c, n, x, st);
+      if (e == cudaSuccess) e = erpp::brick_forces(c, n, g, 1.0f, st);
+      if (e == cudaSuccess) e = erpp::brick_scatter(c, (float*)du, st);
     } else {
       e = erpp::bin_particles(c, n, x, false, st);
       if (e == cudaSuccess) e = erpp::launch_prep_fscat(c, n, g, 1.0f, st);
@@ -629,7 +637,14 @@ cudaError_t scatter_source(erpp_ctx* c, int64_t n, const double* const x[3],
   }
   if (c->fp64)
     return erpp::launch_scatter_f64(c, n, x, D, -1.0 / c->params.rho_f, (double*)S, st);
-  cudaError_t e = erpp::bin_particles(c, n, x, false, st);
+  cudaError_t e;
+  if (use_bricks(c, n)) {
+    e = brick_sort(c, n, x, st);
+    if (e == cudaSuccess) e = brick_forces(c, n, D, -c->kp.inv_rho_dV, st);
+    if (e == cudaSuccess) e = brick_scatter(c, (float*)S, st);
+    return e;
+  }
+  e = erpp::bin_particles(c, n, x, false, st);
   if (e == cudaSuccess) e = erpp::launch_prep_fscat(c, n, D, -c->kp.inv_rho_dV, st);
   if (e == cudaSuccess) e = erpp::launch_scatter_f32(c, (float*)S, st);
   return e;
@@ -734,7 +749,7 @@ erpp_status step_full_force(erpp_ctx* c, const void* u, const erpp_particles* P,
   }
   if (e == cudaSuccess) e = erpp::launch_advance_full(c, P, upc, first_step, st);
   if (e == cudaSuccess && after_advance) e = cudaEventRecord(after_advance, st);
-  if (e == cudaSuccess && tiles) {
+  if (e == cudaSuccess && tiles && !use_bricks(c, n)) {
     e = erpp::launch_prep_fscat(c, n, Dv, -c->kp.inv_rho_dV, st);
     if (e == cudaSuccess) e = erpp::launch_scatter_f32(c, (float*)S, st);
   } else if (e == cudaSuccess) {
@@ -791,7 +806,10 @@ erpp_status step_device(erpp_ctx* c, const void* u, const erpp_particles* P, voi
     if (e == cudaSuccess) e = erpp::launch_advance(c, P, nullptr, true, true, first_step, st);
     if (e == cudaSuccess && after_advance) e = cudaEventRecord(after_advance, st);
     if (ev) cudaEventRecord(ev[3], st);
-    if (e == cudaSuccess) e = erpp::launch_scatter_f32(c, (float*)S, st);
+    if (e == cudaSuccess && use_bricks(c, n))
+      e = scatter_source(c, n, xprev, Dv, S, st);
+    else if (e == cudaSuccess)
+      e = erpp::launch_scatter_f32(c, (float*)S, st);
     if (ev) cudaEventRecord(ev[4], st);
   }
   c->last_step_launches = c->launches;

@@ -1,0 +1,874 @@
+// erpp_bricks.cu -- particles sorted by 8 x 8 x 8-cell bricks, and the FP32
+// regularised source from them (Sec. 2.4, Eq. ns_regularized_filtered) as a
+// tensor-core contraction.
+//
+// Bricks.  A particle belongs to the brick of its home cell and is recorded
+// once (the x/y-halo tiles cut a stencil into pieces and record each).  Bricks
+// are numbered group by group of 2 x 2 x 2, so that the 16 x 16 x 16 cells of a
+// group, and the 16 x 16 x 8 of half of one, are one range of records.  The
+// sort is a counting sort by brick (k_brick_count, a scan, k_brick_place)
+// followed by k_brick_order, which puts the members of a brick in index
+// order: the order of the records, and with it every sum taken over them,
+// does not depend on the order in which the counting atomics arrived (bricks
+// of more than kOrderMax members keep the order of arrival).
+//
+// Source.  S_c(z, y, x) = sum_p (e_z e_y)(z, y; p) (f_c e_x)(x; p) over the
+// particles whose windows reach the region: a matrix product with the
+// particles as its inner dimension.  A block owns a region of 16 x 16 x 16
+// nodes; it lists the particles that touch it from the bricks around, and for
+// every batch of the list stages per particle the y- and z-weights (FP32) and
+// the products f_c e_x of the 16 columns.  Each of the 16 warps owns two
+// planes of eight rows, and accumulates 16 particles at a time in registers
+// with mma.m16n8k16 (rows: 2 planes x 8 rows; columns: 8 nodes of x; inner
+// dimension: the particles that reach the warp's rows, compacted).  Nothing is
+// added by atomics, the region needs no halo, and S is written once.
+//
+// Precision.  Both factors are split into two FP16 numbers, v = h + l (h the
+// rounded value, l the rounded rest: 22 bits and the sign of the rest, an error
+// of at most 2^-24 |v|), and the three products h h', h l', l h' are summed in
+// FP32, 16 particles at a time; the chunks' sums are added in FP32 with
+// rounding (the tensor core truncates: accumulating through it, 125 chunks of
+// a dense cluster left an error of 1.5e-5).  The factors are scaled by powers
+// of two so that a term of 2^-17 of the largest is still split without
+// underflow.  The dropped l l' is below 2^-24 of its term.
+#include <cuda_fp16.h>
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <vector>
+
+#include "erpp_internal.cuh"
+
+namespace {
+
+constexpr int kOrderMax = 4096;  // members of a brick put in index order, at most
+
+// Record of a particle: per axis the distance d0 from the particle to the first
+// node of its window (grid units), and a word with, in byte a, the first
+// node's position in the brick plus 8 (4 .. 15) and, in the upper half, the
+// window length.
+__device__ __forceinline__ int rec_lo(uint32_t w, int a) { return (int)((w >> (8 * a)) & 15u) - 8; }
+__device__ __forceinline__ int rec_nw(uint32_t w, int a) {
+  return (int)((w >> (8 * a + 4)) & 15u);
+}
+
+__device__ __forceinline__ int brick_id(const int ng[3], int bx, int by, int bz) {
+  const int g = ((bz >> 1) * ng[1] + (by >> 1)) * ng[0] + (bx >> 1);
+  return g * 8 + ((bz & 1) << 2) + ((by & 1) << 1) + (bx & 1);
+}
+
+// Window, home cell and brick of every particle; its place among the members
+// of the brick by order of arrival.  Invalid positions get brick -1.
+__global__ void __launch_bounds__(256) k_brick_count(erpp_kparams kp, erpp_brick_dims bd,
+                                                     int64_t n, const double* __restrict__ x0,
+                                                     const double* __restrict__ x1,
+                                                     const double* __restrict__ x2,
+                                                     float4* __restrict__ rec_in,
+                                                     int2* __restrict__ key,
+                                                     int32_t* __restrict__ cnt, uint32_t* err) {
+  erpp_pdl_enter();
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const double xv[3] = {x0[i], x1[i], x2[i]};
+  bool ok = true;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    // 0 <= x < L on the bit patterns (-0 is in range, NaN is not)
+    const unsigned long long bits = (unsigned long long)__double_as_longlong(xv[a]);
+    ok = ok && (bits < (unsigned long long)__double_as_longlong(kp.L[a]) || (bits << 1) == 0ull);
+  }
+  if (!ok) {
+    erpp_set_err(err, ERPP_ERRBIT_RANGE);
+    key[i] = make_int2(-1, 0);
+    return;
+  }
+  int c[3];
+  float d0[3];
+  uint32_t w = 0;
+  bool inb = true;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const erpp_axis_win aw =
+        erpp_axis_window_lean(xv[a], kp.inv_dx[a], kp.cp[a], kp.cp_int[a], kp.cp_frac[a]);
+    const int off = aw.lo - aw.ci, nw = aw.hi - aw.lo + 1;
+    inb = inb && off >= -kp.hlo && off <= 0 && nw >= 1 && nw <= kp.xs;
+    // s can round up to exactly N: the first cell of the next image
+    c[a] = aw.ci >= kp.n[a] ? aw.ci - kp.n[a] : aw.ci;
+    d0[a] = (float)off - aw.t;
+    w |= (uint32_t)((c[a] & 7) + off + 8) << (8 * a) | (uint32_t)nw << (8 * a + 4);
+  }
+  if (!inb) {
+    erpp_set_err(err, ERPP_ERRBIT_BOUNDS);
+    key[i] = make_int2(-1, 0);
+    return;
+  }
+  const int b = brick_id(bd.ng, c[0] >> 3, c[1] >> 3, c[2] >> 3);
+  rec_in[i] = make_float4(d0[0], d0[1], d0[2], __uint_as_float(w));
+  key[i] = make_int2(b, atomicAdd(&cnt[b], 1));
+}
+
+// Exclusive scan of the brick counts in one launch, 4096 counts a block: each
+// block also adds up all the counts before its own (2 MB of L2 reads in all for
+// 65536 bricks), so that no block waits for another.  Up to kBrickScanOne
+// bricks; beyond, where those reads grow, the three-kernel scan.
+constexpr int kBrickScanOne = 131072;
+__global__ void __launch_bounds__(1024) k_brick_scan(const int32_t* __restrict__ cnt,
+                                                     int32_t* __restrict__ start, int nb) {
+  __shared__ int32_t ws[32], wp[32];
+  erpp_pdl_enter();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int base = blockIdx.x * 4096;
+  int32_t before = 0;
+#pragma unroll 8
+  for (int k = threadIdx.x * 4; k < base; k += 4096) {
+    const int4 v = *reinterpret_cast<const int4*>(cnt + k);
+    before += v.x + v.y + v.z + v.w;
+  }
+  const int at = base + threadIdx.x * 4;  // nb is a multiple of 8
+  const int4 v = at < nb ? *reinterpret_cast<const int4*>(cnt + at) : make_int4(0, 0, 0, 0);
+  const int32_t s = v.x + v.y + v.z + v.w;
+  int32_t incl = s;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int32_t u = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += u;
+    before += __shfl_xor_sync(0xffffffffu, before, o);
+  }
+  if (lane == 31) ws[warp] = incl;
+  if (lane == 0) wp[warp] = before;
+  __syncthreads();
+  int32_t wi = ws[lane], all = wp[lane];
+  const int32_t own = wi;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int32_t u = __shfl_up_sync(0xffffffffu, wi, o);
+    if (lane >= o) wi += u;
+    all += __shfl_xor_sync(0xffffffffu, all, o);
+  }
+  const int32_t pre = __shfl_sync(0xffffffffu, wi - own, warp);
+  const int32_t tot = __shfl_sync(0xffffffffu, wi, 31);
+  if (at < nb) {
+    int4 o;
+    o.x = all + pre + incl - s;
+    o.y = o.x + v.x;
+    o.z = o.y + v.y;
+    o.w = o.z + v.z;
+    *reinterpret_cast<int4*>(start + at) = o;
+  }
+  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) start[nb] = all + tot;
+}
+
+__global__ void __launch_bounds__(256) k_brick_place(int64_t n, const int2* __restrict__ key,
+                                                     const float4* __restrict__ rec_in,
+                                                     const int32_t* __restrict__ start,
+                                                     float4* __restrict__ rec_tmp,
+                                                     int32_t* __restrict__ pidx,
+                                                     int32_t* __restrict__ pbrick,
+                                                     int32_t* __restrict__ slot) {
+  erpp_pdl_enter();
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const int2 k = key[i];
+  if (k.x < 0) {
+    slot[i] = -1;
+    return;
+  }
+  const int pos = start[k.x] + k.y;
+  rec_tmp[pos] = rec_in[i];
+  pidx[pos] = (int)i;
+  pbrick[pos] = k.x;
+}
+
+// Position j's particle moves to its rank (by index) among its brick's members.
+// The threads of a warp mostly share a brick, so its indices are read as
+// broadcasts, 16 bytes at a time (a dense cluster's bricks hold a thousand
+// members: 95 us one index at a time for 100k particles in such bricks).
+__global__ void __launch_bounds__(256) k_brick_order(int64_t n, int nb,
+                                                     const int32_t* __restrict__ pidx,
+                                                     const int32_t* __restrict__ pbrick,
+                                                     const float4* __restrict__ rec_tmp,
+                                                     const int32_t* __restrict__ start,
+                                                     float4* __restrict__ rec,
+                                                     uint32_t* __restrict__ win,
+                                                     int32_t* __restrict__ slot) {
+  erpp_pdl_enter();
+  const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (j >= n || j >= start[nb]) return;
+  const int me = pidx[j], b = pbrick[j];
+  const float4 v = rec_tmp[j];
+  const int s = start[b], e = start[b + 1];
+  int r = 0;
+  if (e - s <= kOrderMax) {
+    int k = s;
+    const int body = min((s + 3) & ~3, e), tail = max(e & ~3, body);
+    for (; k < body; ++k) r += pidx[k] < me ? 1 : 0;
+#pragma unroll 4
+    for (; k < tail; k += 4) {
+      const int4 q = *reinterpret_cast<const int4*>(pidx + k);
+      r += (q.x < me ? 1 : 0) + (q.y < me ? 1 : 0) + (q.z < me ? 1 : 0) + (q.w < me ? 1 : 0);
+    }
+    for (; k < e; ++k) r += pidx[k] < me ? 1 : 0;
+  } else {
+    r = (int)j - s;
+  }
+  rec[s + r] = v;
+  win[s + r] = __float_as_uint(v.w);
+  slot[me] = s + r;
+}
+
+// The source's force of a particle, scale * norm * D (a component that is not
+// finite gives no force), stored at its record's place, and the brick's
+// largest |component| (as the bits of a non-negative float).
+__device__ __forceinline__ void put_force(float4* __restrict__ fs, int32_t* __restrict__ bmax,
+                                          int slot, int brick, float f0, float f1, float f2) {
+  f0 = isfinite(f0) ? f0 : 0.f;
+  f1 = isfinite(f1) ? f1 : 0.f;
+  f2 = isfinite(f2) ? f2 : 0.f;
+  fs[slot] = make_float4(f0, f1, f2, 0.f);
+  const int m = __float_as_int(fmaxf(fabsf(f0), fmaxf(fabsf(f1), fabsf(f2))));
+  if (m > bmax[brick]) atomicMax(&bmax[brick], m);
+}
+
+// Normalisation of a particle's weights (erpp_norm's arithmetic on its record).
+__device__ __forceinline__ float rec_norm(const erpp_kparams& kp, float4 r) {
+  if (!kp.normalize) return (float)(kp.dV * kp.raw_norm3);
+  const uint32_t w = __float_as_uint(r.w);
+  const float d0[3] = {r.x, r.y, r.z};
+  float prod = 1.f;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const int nw = rec_nw(w, a);
+    float sum = 0.f;
+    for (int k = 0; k < nw; ++k) {
+      const float d = d0[a] + (float)k;
+      sum += exp2f(-kp.beta[a] * d * d);
+    }
+    prod *= sum;
+  }
+  return 1.f / prod;
+}
+
+__global__ void __launch_bounds__(256) k_brick_forces(erpp_kparams kp, int64_t n,
+                                                      const double* __restrict__ D0,
+                                                      const double* __restrict__ D1,
+                                                      const double* __restrict__ D2, float scale,
+                                                      const float4* __restrict__ rec,
+                                                      const int2* __restrict__ key,
+                                                      const int32_t* __restrict__ slot,
+                                                      float4* __restrict__ fs,
+                                                      int32_t* __restrict__ bmax) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const int sl = slot[i];
+  if (sl < 0) return;
+  const float s = rec_norm(kp, rec[sl]) * scale;
+  put_force(fs, bmax, sl, key[i].x, s * (float)D0[i], s * (float)D1[i], s * (float)D2[i]);
+}
+
+// ---- the source ----
+constexpr int kRegion = 16;      // nodes of a region per axis
+constexpr int kListBatch = 296;  // particles staged at a time, at most
+constexpr int kScatThreads = 512;
+constexpr int kScatWarps = kScatThreads / 32;
+constexpr int kQueue = (kListBatch + 16) / 4;  // members a warp queues before staging them
+// Staged row of a particle: 3 components x (h, l) x 16 columns of FP16, 16 y-
+// and 16 z-weights (FP32).  The pitch puts the rows that an ldmatrix (eight consecutive particles) or a
+// fragment load (four, every other one) reads together in different banks.
+constexpr int kRowW = 192;
+constexpr int kPitch = 336;
+constexpr int kMaxAxisSegs = 8;  // at most 6 are used
+constexpr int kMaxSegs = 352;
+
+__device__ __forceinline__ void mma_f16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0,
+                                        uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+      "{%0,%1,%2,%3};\n"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// The same with a zero addend.
+__device__ __forceinline__ void mma_f16_zero(float (&d)[4], const uint32_t (&a)[4], uint32_t b0,
+                                             uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+      "{%10,%10,%10,%10};\n"
+      : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.f));
+}
+__device__ __forceinline__ void ldmatrix_x4_trans(uint32_t (&r)[4], unsigned addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr));
+}
+// v = h + l in FP16 for a pair of values.
+__device__ __forceinline__ void split_pair(float v0, float v1, uint32_t& h, uint32_t& l) {
+  const __half2 hh = __floats2half2_rn(v0, v1);
+  const float2 hf = __half22float2(hh);
+  const __half2 ll = __floats2half2_rn(v0 - hf.x, v1 - hf.y);
+  h = *reinterpret_cast<const uint32_t*>(&hh);
+  l = *reinterpret_cast<const uint32_t*>(&ll);
+}
+
+struct ScatShared {
+  int cnt[kScatWarps];  // members each warp found that touch the region
+  int maxbits;          // largest |force component| of the bricks around
+  int pre[kMaxSegs + 1];// dense regions: touching members before each segment
+};
+
+// A particle's window relative to a region, all axes at once in the bytes of
+// a word: first node + 64.
+__device__ __forceinline__ uint32_t window_lo(uint32_t w, uint32_t org) {
+  return (w & 0x0f0f0fu) + org;
+}
+// Whether the window reaches nodes [0, ext) on every axis; ext1 holds 63 + ext
+// per byte, with the top bits set: lo < ext leaves the top bit of ext1 - (lo +
+// 64), and lo + length > 0 carries (lo + 64) + length + 63 into the top bit.
+__device__ __forceinline__ bool touches(uint32_t w, uint32_t org, uint32_t ext1) {
+  const uint32_t lo = window_lo(w, org);
+  const uint32_t hi = lo + ((w >> 4) & 0x0f0f0fu) + 0x3f3f3fu;
+  return (((ext1 - lo) & hi) & 0x808080u) == 0x808080u;
+}
+
+__device__ __forceinline__ float ex2_approx(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;\n" : "=f"(y) : "f"(x));
+  return y;
+}
+
+// LP: lanes that stage a particle, each two neighbouring nodes per axis: 4 for
+// windows of at most 7 nodes (at most 4 aligned pairs of nodes), else 8.
+// axis: per axis a and group g the stretches of bricks that hold the home
+// cells of the particles reaching the group's nodes (brick, first cell
+// relative to the group); the last entry of the eight holds their number and
+// 65536 / number, rounded up.
+template <int LP>
+__global__ void __launch_bounds__(kScatThreads, 2) k_brick_scatter(
+    erpp_kparams kp, erpp_brick_dims bd, const int2* __restrict__ axis,
+    const float4* __restrict__ rec, const uint32_t* __restrict__ win,
+    const float4* __restrict__ fs, const int32_t* __restrict__ bstart,
+    const int32_t* __restrict__ bmax, float* __restrict__ S) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  __shared__ ScatShared sh;
+  unsigned char* const row0 = smem;  // [kListBatch + 1][kPitch]
+  uint32_t* const mask = reinterpret_cast<uint32_t*>(row0 + (kListBatch + 1) * kPitch);
+  uint16_t* const wl = reinterpret_cast<uint16_t*>(mask + kListBatch);  // [warps][batch + 16]
+
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int b[3] = {(int)blockIdx.x * kRegion, (int)blockIdx.y * kRegion,
+                    (int)blockIdx.z * kRegion};
+  int ext[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) ext[a] = min(kRegion, kp.n[a] - b[a]);
+  const uint32_t ext1 = 0x808080u | (uint32_t)(63 + ext[0]) | (uint32_t)(63 + ext[1]) << 8 |
+                        (uint32_t)(63 + ext[2]) << 16;
+  const int2* axx = axis + (size_t)blockIdx.x * kMaxAxisSegs;
+  const int2* axy = axis + (size_t)(bd.ng[0] + blockIdx.y) * kMaxAxisSegs;
+  const int2* axz = axis + (size_t)(bd.ng[0] + bd.ng[1] + blockIdx.z) * kMaxAxisSegs;
+  const int2 nsx = axx[kMaxAxisSegs - 1], nsy = axy[kMaxAxisSegs - 1],
+             nsz = axz[kMaxAxisSegs - 1];
+  const int ns = min(nsx.x * nsy.x * nsz.x, kMaxSegs);
+  const int K = (ns + kScatWarps - 1) / kScatWarps;  // segments per warp, at most 22
+
+  if (tid == 0) sh.maxbits = 0;
+  if (tid < kPitch / 16)
+    reinterpret_cast<uint4*>(row0 + kListBatch * kPitch)[tid] = make_uint4(0u, 0u, 0u, 0u);
+  // Segment q: its brick's records, its first cell; returns the brick's
+  // largest force component.
+  auto describe = [&](int q, int& start, int& count, uint32_t& org) {
+    const int r = (q * nsx.y) >> 16, rz = (r * nsy.y) >> 16;  // q / nsx, q / (nsx nsy)
+    const int2 ex_ = axx[q - r * nsx.x], ey_ = axy[r - rz * nsy.x], ez_ = axz[rz];
+    const int id = brick_id(bd.ng, ex_.x, ey_.x, ez_.x);
+    start = bstart[id];
+    count = bstart[id + 1] - start;
+    org = (uint32_t)(ex_.y + 56) | (uint32_t)(ey_.y + 56) << 8 | (uint32_t)(ez_.y + 56) << 16;
+    return bmax[id];
+  };
+  // Lane k describes the warp's k-th segment (the warps take turns, shifted
+  // from turn to turn, so that each gets inner and outer bricks)
+  int seg_s = 0, seg_c = 0, mx = 0;
+  uint32_t seg_o = 0u;
+  const int myq = lane * kScatWarps + ((warp + 5 * lane) & (kScatWarps - 1));
+  if (lane < K && myq < ns) mx = describe(myq, seg_s, seg_c, seg_o);
+  uint16_t* const mylist = wl + warp * (kListBatch + 16);
+  uint2* const queue = reinterpret_cast<uint2*>(mylist);  // until the warp's list is made
+
+  // The members of the warp's segments, four segments at a time as one range,
+  // 32 members a step; those that touch go into the warp's queue (while they
+  // fit).
+  int mine = 0;
+  {
+    for (int k = 0; k < K; k += 4) {
+      int s0[4], e[4];
+      uint32_t o[4];
+      int tot = 0;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        // the member at position idx of the range is record idx + s0[i]
+        s0[i] = __shfl_sync(0xffffffffu, seg_s, k + i) - tot;
+        tot += __shfl_sync(0xffffffffu, seg_c, k + i);
+        o[i] = __shfl_sync(0xffffffffu, seg_o, k + i);
+        e[i] = tot;
+      }
+      for (int m0 = 0; m0 < tot; m0 += 32) {
+        const int idx = m0 + lane;
+        int j = s0[0];
+        uint32_t og = o[0];
+#pragma unroll
+        for (int i = 1; i < 4; ++i) {
+          j = idx >= e[i - 1] ? s0[i] : j;
+          og = idx >= e[i - 1] ? o[i] : og;
+        }
+        j += idx;
+        const uint32_t w = idx < tot ? __ldg(&win[j]) : 0u;
+        const bool t = idx < tot && touches(w, og, ext1);
+        const uint32_t bal = __ballot_sync(0xffffffffu, t);
+        const int at = mine + __popc(bal & ((1u << lane) - 1u));
+        if (t && at < kQueue) queue[at] = make_uint2((uint32_t)j, window_lo(w, og));
+        mine += __popc(bal);
+      }
+    }
+  }
+  mx = __reduce_max_sync(0xffffffffu, (unsigned)mx);
+  __syncthreads();  // maxbits is cleared
+  if (lane == 0) {
+    sh.cnt[warp] = mine;
+    if (mx > 0) atomicMax(&sh.maxbits, mx);
+  }
+  __syncthreads();
+  // the list: warp by warp, segment by segment, in record order
+  int total, at0;
+  bool dense;
+  {
+    const int v = lane < kScatWarps ? sh.cnt[lane] : 0;
+    int incl = v;
+#pragma unroll
+    for (int o = 1; o < kScatWarps; o <<= 1) {
+      const int u = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += u;
+    }
+    total = __shfl_sync(0xffffffffu, incl, kScatWarps - 1);
+    at0 = __shfl_sync(0xffffffffu, incl - v, warp);
+    dense = total > kListBatch || __any_sync(0xffffffffu, v > kQueue);
+  }
+  if (dense) {
+    // more than one batch, or more than a warp can queue: the list is instead
+    // in segment order, and every warp stages an equal share of each batch
+    for (int k = 0; k < K; ++k) {
+      const int s0 = __shfl_sync(0xffffffffu, seg_s, k), c = __shfl_sync(0xffffffffu, seg_c, k);
+      const uint32_t o = __shfl_sync(0xffffffffu, seg_o, k);
+      const int q = __shfl_sync(0xffffffffu, myq, k);
+      int m = 0;
+      for (int m0 = 0; m0 < c; m0 += 32) {
+        const bool t = m0 + lane < c && touches(__ldg(&win[s0 + m0 + lane]), o, ext1);
+        m += __popc(__ballot_sync(0xffffffffu, t));
+      }
+      if (lane == 0 && q < ns) sh.pre[q] = m;
+    }
+    __syncthreads();
+    if (warp == 0) {
+      int carry = 0;
+      for (int q0 = 0; q0 < ns; q0 += 32) {
+        const int v = q0 + lane < ns ? sh.pre[q0 + lane] : 0;
+        int incl = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int u = __shfl_up_sync(0xffffffffu, incl, o);
+          if (lane >= o) incl += u;
+        }
+        if (q0 + lane < ns) sh.pre[q0 + lane] = carry + incl - v;
+        carry += __shfl_sync(0xffffffffu, incl, 31);
+      }
+      if (lane == 0) sh.pre[ns] = carry;
+    }
+    __syncthreads();
+  }
+
+  // factors scaled into the FP16 range: weights by 2^14 (at most 2^14), forces
+  // by 2^(14 - ex) with the largest component below 2^ex
+  const float fmx = __int_as_float(sh.maxbits);
+  int ex = 0;
+  frexpf(fmx, &ex);
+  ex = max(ex, -100);
+  const float sB = ldexpf(1.f, 14 - ex);
+
+  const int zp = warp & 7, yh = warp >> 3;  // planes 2 zp, 2 zp + 1; rows 8 yh ..
+  const int gr = lane >> 2, tq = lane & 3;
+  float acc[3][2][4];
+#pragma unroll
+  for (int c = 0; c < 3; ++c)
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int k = 0; k < 4; ++k) acc[c][h][k] = 0.f;
+
+  // batches of equal size, so that none leaves the warps a nearly empty chunk
+  const int nbatch = (total + kListBatch - 1) / kListBatch;
+  const int bsize = nbatch > 0 ? (total + nbatch - 1) / nbatch : 1;
+
+  // Stages the queue's nq members as rows p0, p0 + 1, ...: LP lanes a particle,
+  // a pair of neighbouring nodes per axis each; the row cleared, then the
+  // weights at the region's nodes.
+  auto stage = [&](int p0, int nq) {
+    const int ql = lane & (LP - 1);
+    for (int i0 = 0; i0 < nq; i0 += 32 / LP) {
+      const int i = i0 + lane / LP;
+      const bool live = i < nq;
+      const uint2 e = queue[live ? i : i0];
+      const float4 r = __ldg(&rec[e.x]);
+      const float4 f = __ldg(&fs[e.x]);
+      unsigned char* const row = row0 + (p0 + i) * kPitch;
+      if (live) {
+#pragma unroll
+        for (int k = 0; k < (20 + LP - 1) / LP; ++k)
+          if (LP == 4 || ql + k * LP < 20)
+            *reinterpret_cast<uint4*>(row + 16 * (ql + k * LP)) = make_uint4(0u, 0u, 0u, 0u);
+      }
+      __syncwarp();
+      const uint32_t w = __float_as_uint(r.w);
+      const float d0[3] = {r.x, r.y, r.z};
+      float v[3][2];
+      bool in[3];
+      int at[3], lo[3];
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        // the pair's first node in the region (even), and its window position
+        lo[a] = (int)((e.y >> (8 * a)) & 255u) - 64;
+        at[a] = (lo[a] & ~1) + 2 * ql;
+        const int q = at[a] - lo[a];  // -1 at the least
+        const int nw = rec_nw(w, a);
+        const float d = d0[a] + (float)q, dn = d0[a] + (float)(q + 1);
+        v[a][0] = q >= 0 && q < nw ? ex2_approx(-kp.beta[a] * d * d) : 0.f;
+        v[a][1] = q + 1 < nw ? ex2_approx(-kp.beta[a] * dn * dn) : 0.f;
+        in[a] = live && q < nw && (unsigned)at[a] < 16u;
+      }
+      const float x0 = v[0][0] * sB, x1 = v[0][1] * sB;
+      uint32_t h[3], l[3];
+      split_pair(f.x * x0, f.x * x1, h[0], l[0]);
+      split_pair(f.y * x0, f.y * x1, h[1], l[1]);
+      split_pair(f.z * x0, f.z * x1, h[2], l[2]);
+      if (in[0]) {
+        uint32_t* col = reinterpret_cast<uint32_t*>(row + 2 * at[0]);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          col[16 * c] = h[c];
+          col[16 * c + 8] = l[c];
+        }
+      }
+      float* const wt = reinterpret_cast<float*>(row + kRowW);
+      if (in[1])
+        *reinterpret_cast<float2*>(wt + at[1]) =
+            make_float2(v[1][0] * 16384.f, v[1][1] * 16384.f);
+      if (in[2]) *reinterpret_cast<float2*>(wt + 16 + at[2]) = make_float2(v[2][0], v[2][1]);
+      if (live && ql == 0) {
+        // the warps whose rows and planes the window reaches: bit 8 yh + zp
+        const int y1 = lo[1] + rec_nw(w, 1) - 1;
+        const int za = max(lo[2], 0) >> 1, zb = min(lo[2] + rec_nw(w, 2) - 1, 15) >> 1;
+        const uint32_t zm = (2u << zb) - (1u << za);
+        mask[p0 + i] = (lo[1] < 8 ? zm : 0u) | (y1 >= 8 ? zm << 8 : 0u);
+      }
+    }
+  };
+
+  for (int l0 = 0; l0 < total; l0 += bsize) {
+    const int np = min(bsize, total - l0);
+    // the warp's members of the batch
+    if (!dense) {
+      __syncwarp();
+      stage(at0, mine);
+    } else {
+      // the warp's share: list positions [ra, rb)
+      const int share = (np + kScatWarps - 1) / kScatWarps;
+      const int ra = l0 + min(warp * share, np), rb = l0 + min((warp + 1) * share, np);
+      for (int q0 = 0; q0 < ns && ra < rb; q0 += 32) {
+        const int q = q0 + lane;
+        const bool over = q < ns && sh.pre[q] < rb && sh.pre[q + 1] > ra;
+        uint32_t todo = __ballot_sync(0xffffffffu, over);
+        int ds = 0, dc = 0;
+        uint32_t dorg = 0u;
+        if (over) describe(q, ds, dc, dorg);
+        while (todo) {
+          const int k = __ffs(todo) - 1;
+          todo &= todo - 1u;
+          const int s0 = __shfl_sync(0xffffffffu, ds, k), c = __shfl_sync(0xffffffffu, dc, k);
+          const uint32_t o = __shfl_sync(0xffffffffu, dorg, k);
+          int at = sh.pre[q0 + k];
+          for (int m0 = 0; m0 < c && at < rb; m0 += 32) {
+            uint32_t w = 0u;
+            bool t = false;
+            if (m0 + lane < c) {
+              w = __ldg(&win[s0 + m0 + lane]);
+              t = touches(w, o, ext1);
+            }
+            const uint32_t bal = __ballot_sync(0xffffffffu, t);
+            const int p = at + __popc(bal & ((1u << lane) - 1u));
+            if (t && p >= ra && p < rb)
+              queue[p - ra] = make_uint2((uint32_t)(s0 + m0 + lane), window_lo(w, o));
+            at += __popc(bal);
+          }
+        }
+      }
+      __syncwarp();
+      stage(ra - l0, rb - ra);
+    }
+    __syncthreads();
+    // the warp's own particles, those that reach its rows and planes: their
+    // rows' offsets in units of 16 bytes
+    int cw = 0;
+    for (int p0 = 0; p0 < np; p0 += 32) {
+      const uint32_t m = p0 + lane < np ? mask[p0 + lane] : 0u;
+      const bool t = (m >> warp) & 1u;
+      const unsigned bal = __ballot_sync(0xffffffffu, t);
+      if (t)
+        mylist[cw + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)((p0 + lane) * (kPitch / 16));
+      cw += __popc(bal);
+    }
+    if (lane < 16) mylist[cw + lane] = (uint16_t)(kListBatch * (kPitch / 16));  // the zero row
+    __syncwarp();
+    const unsigned char* const wty = row0 + kRowW + 4 * (8 * yh + gr);
+    const unsigned char* const wtz = row0 + kRowW + 4 * (16 + 2 * zp);
+    const unsigned btab = (unsigned)__cvta_generic_to_shared(row0) + ((lane >> 4) << 4);
+    for (int c0 = 0; c0 < cw; c0 += 16) {
+      const uint32_t pa = *reinterpret_cast<const uint32_t*>(mylist + c0 + 2 * tq);
+      const uint32_t pb = *reinterpret_cast<const uint32_t*>(mylist + c0 + 8 + 2 * tq);
+      const unsigned pk[4] = {(pa & 0xffffu) * 16u, (pa >> 16) * 16u, (pb & 0xffffu) * 16u,
+                              (pb >> 16) * 16u};
+      float w0[4], w1[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const float y = *reinterpret_cast<const float*>(wty + pk[k]);
+        const float2 z = *reinterpret_cast<const float2*>(wtz + pk[k]);
+        w0[k] = y * z.x;
+        w1[k] = y * z.y;
+      }
+      uint32_t ah[4], al[4];
+      split_pair(w0[0], w0[1], ah[0], al[0]);
+      split_pair(w1[0], w1[1], ah[1], al[1]);
+      split_pair(w0[2], w0[3], ah[2], al[2]);
+      split_pair(w1[2], w1[3], ah[3], al[3]);
+      const unsigned addr = btab + 16u * mylist[c0 + (lane & 15)];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        uint32_t bh[4], bl[4];
+        ldmatrix_x4_trans(bh, addr + (2 * c) * 32);
+        ldmatrix_x4_trans(bl, addr + (2 * c + 1) * 32);
+        // the chunk's own sums first (the tensor core truncates its sums; the
+        // small products go first), then one rounded FP32 addition
+        float d0[4], d1[4];
+        mma_f16_zero(d0, al, bh[0], bh[1]);
+        mma_f16_zero(d1, al, bh[2], bh[3]);
+        mma_f16(d0, ah, bl[0], bl[1]);
+        mma_f16(d1, ah, bl[2], bl[3]);
+        mma_f16(d0, ah, bh[0], bh[1]);
+        mma_f16(d1, ah, bh[2], bh[3]);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          acc[c][0][k] += d0[k];
+          acc[c][1][k] += d1[k];
+        }
+      }
+    }
+    if (l0 + bsize < total) __syncthreads();  // the rows are staged again
+  }
+
+  // a lane holds nodes (x, x + 1) of row gr of both planes
+  const float inv = ldexpf(1.f, ex - 28);
+  const size_t nxy = (size_t)kp.n[0] * kp.n[1], nn = nxy * kp.n[2];
+  const int y = 8 * yh + gr;
+  const bool pair = (kp.n[0] & 1) == 0 && (((uintptr_t)S) & 7) == 0;
+  if (y < ext[1]) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int x = 8 * h + 2 * tq;
+#pragma unroll
+      for (int z = 0; z < 2; ++z) {
+        if (2 * zp + z >= ext[2] || x >= ext[0]) continue;
+        float* d = S + (size_t)(b[2] + 2 * zp + z) * nxy + (size_t)(b[1] + y) * kp.n[0] + b[0] + x;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          const float v0 = acc[c][h][2 * z] * inv, v1 = acc[c][h][2 * z + 1] * inv;
+          if (pair) {
+            *reinterpret_cast<float2*>(d + c * nn) = make_float2(v0, v1);
+          } else {
+            d[c * nn] = v0;
+            if (x + 1 < ext[0]) d[c * nn + 1] = v1;
+          }
+        }
+      }
+    }
+  }
+}
+
+size_t scatter_smem() {
+  return (size_t)(kListBatch + 1) * kPitch + (size_t)kListBatch * 4 +
+         (size_t)kScatWarps * (kListBatch + 16) * 2;
+}
+
+// The stretches of bricks along an axis of n cells whose particles (windows
+// starting at most hlo nodes below the home cell and ending at most hlo + 1
+// above) can reach the nodes of group g: each stretch's brick and its first
+// cell relative to the group's first node, periodic images included; the last
+// entry holds their number.
+void axis_segments(int n, int hlo, int g, int2* out) {
+  const int b = g * kRegion, last = std::min(b + kRegion, n) - 1 + hlo;
+  int k = 0;
+  for (int j = b - hlo - 1; j <= last && k < kMaxAxisSegs - 1;) {
+    const int m = j >= 0 ? j / n : -((-j + n - 1) / n);
+    const int br = (j - m * n) >> 3;
+    out[k].x = br;
+    out[k].y = 8 * br + m * n - b;
+    ++k;
+    j = std::min(8 * br + 8, n) + m * n;
+  }
+  for (int i = k; i < kMaxAxisSegs - 1; ++i) out[i] = make_int2(-1, 0);
+  out[kMaxAxisSegs - 1] = make_int2(k, 65536 / k + 1);
+}
+
+}  // namespace
+
+namespace erpp {
+
+// Whether the context's windows and options allow the brick kernels (windows
+// of at most 10 nodes that start at most 4 below the cell: the record's
+// fields; FP32, Gaussian source).
+bool bricks_possible(const erpp_ctx* c) {
+  return !c->fp64 && c->kp.design == 4 && c->kp.weights != ERPP_W_PIC && !c->kp.kahan &&
+         c->kp.xs <= 10 && c->kp.hlo <= 4;
+}
+
+// The brick kernels serve a call when the context's scatter mode is the
+// default and the box gives every SM a region to work on (152 regions of
+// 16^3 nodes), or its particles are dense (a quarter of a particle per node,
+// 16384 at least: the x/y-halo tiles then hold thousands of pieces each).  Smaller boxes keep
+// the tile kernels, whose smaller blocks finish earlier there.
+bool use_bricks(const erpp_ctx* c, int64_t n) {
+  if (!c->bk.rec || c->scatter_mode != ERPP_SCATTER_MERGE || n <= 0) return false;
+  const int64_t regions = c->bk.nbricks / 8;
+  const double nodes = (double)c->kp.n[0] * c->kp.n[1] * c->kp.n[2];
+  return regions >= 152 || (n >= 16384 && (double)n >= 0.25 * nodes);
+}
+
+cudaError_t bricks_alloc_tables(erpp_ctx* c) {
+  erpp_bricks& k = c->bk;
+  if (!bricks_possible(c)) return cudaSuccess;
+  int64_t ng = 1;
+  for (int a = 0; a < 3; ++a) {
+    k.dims.ng[a] = (c->kp.n[a] + kRegion - 1) / kRegion;
+    ng *= k.dims.ng[a];
+  }
+  if (ng > (1 << 24) || k.dims.ng[1] > 65535 || k.dims.ng[2] > 65535) return cudaSuccess;
+  k.nbricks = (int)(8 * ng);
+  // counts and force maxima, cleared together
+  cudaError_t e = cudaMalloc(&k.cnt, sizeof(int32_t) * 2 * (size_t)k.nbricks);
+  if (e == cudaSuccess) e = cudaMalloc(&k.start, sizeof(int32_t) * ((size_t)k.nbricks + 4));
+  if (e == cudaSuccess) e = cudaMalloc(&k.scan_tmp, sizeof(int32_t) * (k.nbricks / 4096 + 1));
+  k.bmax = k.cnt ? k.cnt + k.nbricks : nullptr;
+  std::vector<int2> ax;
+  for (int a = 0; a < 3; ++a)
+    for (int g = 0; g < k.dims.ng[a]; ++g) {
+      ax.resize(ax.size() + kMaxAxisSegs);
+      axis_segments(c->kp.n[a], c->kp.hlo, g, ax.data() + ax.size() - kMaxAxisSegs);
+    }
+  if (e == cudaSuccess) e = cudaMalloc(&k.axis, sizeof(int2) * ax.size());
+  if (e == cudaSuccess)
+    e = cudaMemcpy(k.axis, ax.data(), sizeof(int2) * ax.size(), cudaMemcpyHostToDevice);
+  return e;
+}
+
+void bricks_free_tables(erpp_ctx* c) {
+  erpp_bricks& k = c->bk;
+  cudaFree(k.cnt);
+  cudaFree(k.start);
+  cudaFree(k.scan_tmp);
+  cudaFree(k.axis);
+  k.axis = nullptr;
+  k.cnt = k.start = k.scan_tmp = k.bmax = nullptr;
+}
+
+cudaError_t bricks_alloc(erpp_ctx* c, int64_t cap) {
+  erpp_bricks& k = c->bk;
+  if (!k.cnt) return cudaSuccess;
+  const size_t n = (size_t)cap;
+  cudaError_t e = cudaMalloc(&k.key, sizeof(int2) * n);
+  if (e == cudaSuccess) e = cudaMalloc(&k.pidx, sizeof(int32_t) * n);
+  if (e == cudaSuccess) e = cudaMalloc(&k.pbrick, sizeof(int32_t) * n);
+  if (e == cudaSuccess) e = cudaMalloc(&k.slot, sizeof(int32_t) * n);
+  if (e == cudaSuccess) e = cudaMalloc(&k.up, sizeof(float4) * n);
+  if (e == cudaSuccess) e = cudaMalloc(&k.fs, sizeof(float4) * n);
+  if (e == cudaSuccess) e = cudaMalloc(&k.rec, sizeof(float4) * n);
+  if (e == cudaSuccess) e = cudaMalloc(&k.win, sizeof(uint32_t) * n);
+  return e;
+}
+
+void bricks_free(erpp_ctx* c) {
+  erpp_bricks& k = c->bk;
+  cudaFree(k.key);
+  cudaFree(k.pidx);
+  cudaFree(k.pbrick);
+  cudaFree(k.slot);
+  cudaFree(k.up);
+  cudaFree(k.fs);
+  cudaFree(k.rec);
+  cudaFree(k.win);
+  k.win = nullptr;
+  k.key = nullptr;
+  k.pidx = k.pbrick = k.slot = nullptr;
+  k.up = k.fs = k.rec = nullptr;
+}
+
+// Sorts n particles at x into bricks: bk.rec in order, bk.slot each particle's
+// place (-1: invalid position), bk.start the bricks' ranges.
+cudaError_t brick_sort(erpp_ctx* c, int64_t n, const double* const x[3], cudaStream_t st) {
+  erpp_bricks& k = c->bk;
+  const int nb = k.nbricks;
+  cudaError_t e = cudaMemsetAsync(k.cnt, 0, sizeof(int32_t) * 2 * (size_t)nb, st);
+  if (e != cudaSuccess) return e;
+  const unsigned blocks = (unsigned)((n + 255) / 256);
+  // between the kernels of the sort: the windows in input order (where the
+  // gathered velocities go later) and in order of arrival (the forces)
+  float4* rec_in = k.up;
+  float4* rec_tmp = k.fs;
+  ++c->launches;
+  e = erpp_launch_pdl(k_brick_count, dim3(blocks), dim3(256), 0, st, 0u, c->kp, k.dims, n, x[0],
+                      x[1], x[2], rec_in, k.key, k.cnt, c->err);
+  if (e != cudaSuccess) return e;
+  if (nb <= kBrickScanOne) {
+    ++c->launches;
+    e = erpp_launch_pdl(k_brick_scan, dim3((unsigned)((nb + 4095) / 4096)), dim3(1024), 0, st, 0u, (const int32_t*)k.cnt,
+                        k.start, nb);
+  } else {
+    e = launch_scan(c, k.cnt, k.start, k.scan_tmp, nb, st);
+  }
+  if (e != cudaSuccess) return e;
+  c->launches += 2;
+  e = erpp_launch_pdl(k_brick_place, dim3(blocks), dim3(256), 0, st, 0u, n, (const int2*)k.key,
+                      (const float4*)rec_in, (const int32_t*)k.start, rec_tmp, k.pidx, k.pbrick,
+                      k.slot);
+  if (e != cudaSuccess) return e;
+  return erpp_launch_pdl(k_brick_order, dim3(blocks), dim3(256), 0, st, 0u, n, nb,
+                         (const int32_t*)k.pidx, (const int32_t*)k.pbrick, (const float4*)rec_tmp,
+                         (const int32_t*)k.start, k.rec,
+                         k.win, k.slot);
+}
+
+cudaError_t brick_forces(erpp_ctx* c, int64_t n, const double* const D[3], float scale,
+                         cudaStream_t st) {
+  erpp_bricks& k = c->bk;
+  ++c->launches;
+  k_brick_forces<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(c->kp, n, D[0], D[1], D[2], scale,
+                                                              k.rec, k.key, k.slot, k.fs, k.bmax);
+  return cudaGetLastError();
+}
+
+cudaError_t brick_scatter(erpp_ctx* c, float* S, cudaStream_t st) {
+  erpp_bricks& k = c->bk;
+  const size_t sm = scatter_smem();
+  auto kern = c->kp.xs <= 7 ? k_brick_scatter<4> : k_brick_scatter<8>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  if (e != cudaSuccess) return e;
+  ++c->launches;
+  const dim3 grid((unsigned)k.dims.ng[0], (unsigned)k.dims.ng[1], (unsigned)k.dims.ng[2]);
+  kern<<<grid, kScatThreads, sm, st>>>(c->kp, k.dims, k.axis, k.rec, k.win, k.fs, k.start,
+                                                k.bmax, S);
+  return cudaGetLastError();
+}
+
+}  // namespace erpp

@@ -119,6 +119,31 @@ struct erpp_kparams {
   int64_t wrap_lo_bits[3], wrap_hi_bits[3];
 };
 
+// Groups of 2 x 2 x 2 bricks per axis (bricks of 8 x 8 x 8 cells).
+struct erpp_brick_dims {
+  int32_t ng[3];
+};
+
+// Particles sorted by brick (erpp_bricks.cu); every pointer null where the
+// context's windows or options rule the brick kernels out.
+struct erpp_bricks {
+  erpp_brick_dims dims;
+  int32_t nbricks;
+  int32_t* cnt;     // [nbricks] members; cleared with bmax
+  int32_t* bmax;    // [nbricks] largest |force component| (float bits), after cnt
+  int32_t* start;   // [nbricks + 1]
+  int32_t* scan_tmp;
+  int2* axis;       // per axis and group: the stretches of bricks around it
+  int2* key;        // [cap] per particle: brick (-1: invalid position), place by arrival
+  int32_t* pidx;    // [cap] in order of arrival: particle
+  int32_t* pbrick;  // [cap] in order of arrival: brick
+  int32_t* slot;    // [cap] per particle: place in the order of the records
+  float4* rec;      // [cap] records in order: distances to the window's first nodes, window word
+  uint32_t* win;    // [cap] the window words alone
+  float4* up;       // [cap] in order: gathered velocity (scratch of the sort before)
+  float4* fs;       // [cap] in order: scaled force (scratch of the sort before)
+};
+
 struct erpp_ctx {
   erpp_params params;
   erpp_kparams kp;
@@ -170,6 +195,7 @@ struct erpp_ctx {
   int32_t* tile_start;    // [32 ntiles + 1]
   int32_t* piece_slot;    // [maxseg product][cap]: each piece's place in its bin
   int32_t* scan_tmp;      // [ceil(32 ntiles / 4096)] chunk totals of the scan
+  erpp_bricks bk;         // particles sorted by brick
   uint32_t* err;          // device error word
   double* red;            // reduction scratch
   int red_cap;
@@ -232,6 +258,19 @@ cudaError_t launch_bin_multi(const erpp_box_dev* boxes, int nbox, const int2* pi
                              int npitems, cudaStream_t st);
 cudaError_t launch_advance_multi(const erpp_box_dev* boxes, const int2* pitems, int npitems,
                                  int first_step, cudaStream_t st);
+
+// Particles sorted by brick (erpp_bricks.cu): scratch, the sort, the forces at
+// their records' places (scale * norm * D), and the source from them.
+bool bricks_possible(const erpp_ctx* c);
+bool use_bricks(const erpp_ctx* c, int64_t n);
+cudaError_t bricks_alloc_tables(erpp_ctx* c);
+void bricks_free_tables(erpp_ctx* c);
+cudaError_t bricks_alloc(erpp_ctx* c, int64_t cap);
+void bricks_free(erpp_ctx* c);
+cudaError_t brick_sort(erpp_ctx* c, int64_t n, const double* const x[3], cudaStream_t st);
+cudaError_t brick_forces(erpp_ctx* c, int64_t n, const double* const D[3], float scale,
+                         cudaStream_t st);
+cudaError_t brick_scatter(erpp_ctx* c, float* S, cudaStream_t st);
 
 erpp_status derive_ctx(const erpp_params* p, erpp_ctx* c);
 erpp_status ensure_capacity(erpp_ctx* c, int64_t n);  // may allocate (synchronous)
