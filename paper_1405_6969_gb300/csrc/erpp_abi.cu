@@ -59,6 +59,8 @@ void free_scratch(erpp_ctx* c) {
   cudaFree(c->fscat);
   cudaFree(c->entries);
   cudaFree(c->piece_slot);
+  cudaFree(c->gather_items);
+  c->gather_items = nullptr;
   cudaFree(c->up64);
   cudaFree(c->w_key);
   cudaFree(c->w_slot);
@@ -127,6 +129,8 @@ erpp_status ensure_capacity(erpp_ctx* c, int64_t n) {
     if (e == cudaSuccess && c->kp.design == 4 && c->kp.full_force)
       e = cudaMalloc(&c->lap_part, sizeof(float4) * (size_t)ecap);
     if (e == cudaSuccess) e = cudaMalloc(&c->piece_slot, sizeof(int32_t) * (size_t)ecap);
+    if (e == cudaSuccess && c->kp.design == 4)
+      e = cudaMalloc(&c->gather_items, sizeof(int2) * (size_t)(ecap / ERPP_GATHER_CHUNK + 1));
     c->entries_cap = ecap;
     if (e == cudaSuccess) e = bricks_alloc(c, cap);
   }
@@ -149,7 +153,7 @@ erpp_status alloc_tile_tables(erpp_ctx* c) {
   if (c->fp64) return ERPP_OK;
   const erpp_kparams& kp = c->kp;
   const size_t nbins = (size_t)erpp::nbins(kp);
-  cudaError_t e = cudaMalloc(&c->tile_cnt, sizeof(int32_t) * nbins);
+  cudaError_t e = cudaMalloc(&c->tile_cnt, sizeof(int32_t) * (nbins + 1));
   if (e == cudaSuccess) e = cudaMalloc(&c->tile_start, sizeof(int32_t) * (nbins + 1));
   if (e == cudaSuccess) e = cudaMalloc(&c->scan_tmp, sizeof(int32_t) * (nbins / 4096 + 1));
   const size_t hb = (size_t)kp.ntiles * (size_t)kp.halo_per_tile;
@@ -742,7 +746,7 @@ erpp_status step_full_force(erpp_ctx* c, const void* u, const erpp_particles* P,
   cudaError_t e = cudaSuccess;
   if (tiles) {
     e = erpp::bin_particles(c, n, xin, true, st);
-    if (e == cudaSuccess) e = erpp::launch_gather_lap_f32_4(c, (const float*)u, st);
+    if (e == cudaSuccess) e = erpp::launch_gather_lap_f32_4(c, (const float*)u, n, st);
     if (e == cudaSuccess) e = erpp::launch_finalize_full(c, n, xin, up, c->ff_lap, c->cap, st);
   } else {
     e = erpp::launch_gather_faxen(c, u, n, xin, up, st);
@@ -799,17 +803,18 @@ erpp_status step_device(erpp_ctx* c, const void* u, const erpp_particles* P, voi
     cudaEvent_t* ev = nullptr;
     if (c->prof_on) ev = c->prof_ev + 5 * (c->prof_n++ % kProfSets);
     if (ev) cudaEventRecord(ev[0], st);
-    e = erpp::bin_particles(c, n, xin, true, st);
+    const bool bricks = use_bricks(c, n);
+    e = bricks ? brick_sort(c, n, xin, st) : cudaSuccess;
+    if (e == cudaSuccess) e = erpp::bin_particles(c, n, xin, true, st);
     if (ev) cudaEventRecord(ev[1], st);
     if (e == cudaSuccess) e = erpp::launch_gather_f32(c, (const float*)u, n, st);
     if (ev) cudaEventRecord(ev[2], st);
-    if (e == cudaSuccess) e = erpp::launch_advance(c, P, nullptr, true, true, first_step, st);
+    if (e == cudaSuccess)
+      e = erpp::launch_advance(c, P, nullptr, true, true, first_step, st, nullptr, nullptr, bricks);
     if (e == cudaSuccess && after_advance) e = cudaEventRecord(after_advance, st);
     if (ev) cudaEventRecord(ev[3], st);
-    if (e == cudaSuccess && use_bricks(c, n))
-      e = scatter_source(c, n, xprev, Dv, S, st);
-    else if (e == cudaSuccess)
-      e = erpp::launch_scatter_f32(c, (float*)S, st);
+    if (e == cudaSuccess)
+      e = bricks ? brick_scatter(c, (float*)S, st) : erpp::launch_scatter_f32(c, (float*)S, st);
     if (ev) cudaEventRecord(ev[4], st);
   }
   c->last_step_launches = c->launches;

@@ -290,7 +290,8 @@ __device__ __forceinline__ void bin_fill_one(const erpp_kparams& kp, int64_t i, 
                                              const int32_t* __restrict__ start,
                                              int32_t* __restrict__ slot, int ms,
                                              int4* __restrict__ entries, int64_t cap,
-                                             uint32_t* err) {
+                                             int32_t* __restrict__ nitems,
+                                             int2* __restrict__ items, uint32_t* err) {
   const int4 g = geo_c[i];
   const uint32_t pack = (uint32_t)g.w;
   if (!(pack & ERPP_GEO_VALID)) return;
@@ -331,10 +332,15 @@ __device__ __forceinline__ void bin_fill_one(const erpp_kparams& kp, int64_t i, 
                           ((uint32_t)(ez - jz + 1) << 15) | ((uint32_t)qa << 18) |
                           ((uint32_t)lx << 22);
       const int64_t pos = place(tile);
-      if (pos < cap)
+      if (pos < cap) {
         entries[pos] = make_int4((int)i, (int)pk, __float_as_int(d0y), __float_as_int(d0z));
-      else
+        // the first piece of a further chunk of the gather's tile
+        const int off = (int)pos - start[tile];
+        if (items && off > 0 && off % ERPP_GATHER_CHUNK == 0)
+          items[atomicAdd(nitems, 1)] = make_int2(tile, (int)pos);
+      } else {
         erpp_set_err(err, ERPP_ERRBIT_BOUNDS);
+      }
     });
     return;
   }
@@ -359,11 +365,13 @@ __device__ __forceinline__ void bin_fill_one(const erpp_kparams& kp, int64_t i, 
 __global__ void k_bin_fill(erpp_kparams kp, int64_t n, const float4* __restrict__ geo_t,
                            const int4* __restrict__ geo_c, const int32_t* __restrict__ start,
                            int32_t* __restrict__ slot, int ms,
-                           int4* __restrict__ entries, int64_t cap, uint32_t* err) {
+                           int4* __restrict__ entries, int64_t cap,
+                           int32_t* __restrict__ nitems, int2* __restrict__ items,
+                           uint32_t* err) {
   erpp_pdl_enter();
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  bin_fill_one(kp, i, n, geo_t, geo_c, start, slot, ms, entries, cap, err);
+  bin_fill_one(kp, i, n, geo_t, geo_c, start, slot, ms, entries, cap, nitems, items, err);
 }
 
 // Exclusive scan of the per-bin counts: k_scan_local scans chunks of
@@ -554,7 +562,7 @@ __global__ void __launch_bounds__(256) k_bin_fill_multi(const erpp_box_dev* __re
   const int64_t i = (int64_t)it.y + threadIdx.x;
   if (i >= B.n) return;
   bin_fill_one(B.kp, i, B.n, B.geo_t, B.geo_c, B.tile_start, B.piece_slot, B.ms, B.entries,
-               B.ecap, B.err);
+               B.ecap, nullptr, nullptr, B.err);
 }
 
 }  // namespace
@@ -576,7 +584,9 @@ cudaError_t bin_particles(erpp_ctx* ctx, int64_t n, const double* const x[3], bo
   const erpp_kparams& kp = ctx->kp;
   const int nbins = erpp::nbins(kp);
   const int ms = ctx->maxseg[0] * ctx->maxseg[1] * ctx->maxseg[2];
-  cudaError_t e = cudaMemsetAsync(ctx->tile_cnt, 0, sizeof(int32_t) * nbins, st);
+  // with the number of the gather's further chunks after the counts
+  cudaError_t e = cudaMemsetAsync(ctx->tile_cnt, 0,
+                                  sizeof(int32_t) * (nbins + (ctx->gather_items ? 1 : 0)), st);
   if (e != cudaSuccess) return e;
   if (n > 0 && kp.design == 4 && !kp.full_force && nbins <= kHistBins && ms <= kHistPieces) {
     // few tiles (a small box): count through block histograms
@@ -616,7 +626,7 @@ cudaError_t bin_particles(erpp_ctx* ctx, int64_t n, const double* const x[3], bo
     e = erpp_launch_pdl(k_bin_fill, dim3(blocks), dim3(256), 0, st, 0u, kp, n,
                         (const float4*)ctx->geo_t, (const int4*)ctx->geo_c,
                         (const int32_t*)ctx->tile_start, ctx->piece_slot, ms, ctx->entries,
-                        ctx->entries_cap, ctx->err);
+                        ctx->entries_cap, ctx->tile_cnt + nbins, ctx->gather_items, ctx->err);
     if (e != cudaSuccess) return e;
   }
   return cudaGetLastError();

@@ -43,15 +43,6 @@ namespace {
 
 constexpr int kOrderMax = 4096;  // members of a brick put in index order, at most
 
-// Record of a particle: per axis the distance d0 from the particle to the first
-// node of its window (grid units), and a word with, in byte a, the first
-// node's position in the brick plus 8 (4 .. 15) and, in the upper half, the
-// window length.
-__device__ __forceinline__ int rec_lo(uint32_t w, int a) { return (int)((w >> (8 * a)) & 15u) - 8; }
-__device__ __forceinline__ int rec_nw(uint32_t w, int a) {
-  return (int)((w >> (8 * a + 4)) & 15u);
-}
-
 __device__ __forceinline__ int brick_id(const int ng[3], int bx, int by, int bz) {
   const int g = ((bz >> 1) * ng[1] + (by >> 1)) * ng[0] + (bx >> 1);
   return g * 8 + ((bz & 1) << 2) + ((by & 1) << 1) + (bx & 1);
@@ -83,7 +74,7 @@ __global__ void __launch_bounds__(256) k_brick_count(erpp_kparams kp, erpp_brick
     return;
   }
   int c[3];
-  float d0[3];
+  float t[3];
   uint32_t w = 0;
   bool inb = true;
 #pragma unroll
@@ -94,8 +85,12 @@ __global__ void __launch_bounds__(256) k_brick_count(erpp_kparams kp, erpp_brick
     inb = inb && off >= -kp.hlo && off <= 0 && nw >= 1 && nw <= kp.xs;
     // s can round up to exactly N: the first cell of the next image
     c[a] = aw.ci >= kp.n[a] ? aw.ci - kp.n[a] : aw.ci;
-    d0[a] = (float)off - aw.t;
-    w |= (uint32_t)((c[a] & 7) + off + 8) << (8 * a) | (uint32_t)nw << (8 * a + 4);
+    t[a] = aw.t;
+    // off is -ck - 1, -ck or -ck + 1 (ck = floor(c'), the first by rounding)
+    const int so = off + kp.cp_int[a] + 1;
+    inb = inb && so >= 0 && so <= 3;
+    w |= (uint32_t)((c[a] & 7) + off + 8) << (8 * a) | (uint32_t)nw << (8 * a + 4) |
+         (uint32_t)so << (24 + 2 * a);
   }
   if (!inb) {
     erpp_set_err(err, ERPP_ERRBIT_BOUNDS);
@@ -103,7 +98,7 @@ __global__ void __launch_bounds__(256) k_brick_count(erpp_kparams kp, erpp_brick
     return;
   }
   const int b = brick_id(bd.ng, c[0] >> 3, c[1] >> 3, c[2] >> 3);
-  rec_in[i] = make_float4(d0[0], d0[1], d0[2], __uint_as_float(w));
+  rec_in[i] = make_float4(t[0], t[1], t[2], __uint_as_float(w));
   key[i] = make_int2(b, atomicAdd(&cnt[b], 1));
 }
 
@@ -216,32 +211,19 @@ __global__ void __launch_bounds__(256) k_brick_order(int64_t n, int nb,
   slot[me] = s + r;
 }
 
-// The source's force of a particle, scale * norm * D (a component that is not
-// finite gives no force), stored at its record's place, and the brick's
-// largest |component| (as the bits of a non-negative float).
-__device__ __forceinline__ void put_force(float4* __restrict__ fs, int32_t* __restrict__ bmax,
-                                          int slot, int brick, float f0, float f1, float f2) {
-  f0 = isfinite(f0) ? f0 : 0.f;
-  f1 = isfinite(f1) ? f1 : 0.f;
-  f2 = isfinite(f2) ? f2 : 0.f;
-  fs[slot] = make_float4(f0, f1, f2, 0.f);
-  const int m = __float_as_int(fmaxf(fabsf(f0), fmaxf(fabsf(f1), fabsf(f2))));
-  if (m > bmax[brick]) atomicMax(&bmax[brick], m);
-}
-
 // Normalisation of a particle's weights (erpp_norm's arithmetic on its record).
 __device__ __forceinline__ float rec_norm(const erpp_kparams& kp, float4 r) {
   if (!kp.normalize) return (float)(kp.dV * kp.raw_norm3);
   const uint32_t w = __float_as_uint(r.w);
-  const float d0[3] = {r.x, r.y, r.z};
+  const float t[3] = {r.x, r.y, r.z};
   float prod = 1.f;
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    const int nw = rec_nw(w, a);
+    const int nw = erpp_rec_nw(w, a), off = erpp_rec_off(kp, w, a);
     float sum = 0.f;
     for (int k = 0; k < nw; ++k) {
-      const float d = d0[a] + (float)k;
-      sum += exp2f(-kp.beta[a] * d * d);
+      const float d = (float)(off + k) - t[a];
+      sum += erpp_ex2(-kp.beta[a] * d * d);
     }
     prod *= sum;
   }
@@ -262,7 +244,7 @@ __global__ void __launch_bounds__(256) k_brick_forces(erpp_kparams kp, int64_t n
   const int sl = slot[i];
   if (sl < 0) return;
   const float s = rec_norm(kp, rec[sl]) * scale;
-  put_force(fs, bmax, sl, key[i].x, s * (float)D0[i], s * (float)D1[i], s * (float)D2[i]);
+  erpp_put_force(fs, bmax, sl, key[i].x, s * (float)D0[i], s * (float)D1[i], s * (float)D2[i]);
 }
 
 // ---- the source ----
@@ -326,12 +308,6 @@ __device__ __forceinline__ bool touches(uint32_t w, uint32_t org, uint32_t ext1)
   const uint32_t lo = window_lo(w, org);
   const uint32_t hi = lo + ((w >> 4) & 0x0f0f0fu) + 0x3f3f3fu;
   return (((ext1 - lo) & hi) & 0x808080u) == 0x808080u;
-}
-
-__device__ __forceinline__ float ex2_approx(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;\n" : "=f"(y) : "f"(x));
-  return y;
 }
 
 // LP: lanes that stage a particle, each two neighbouring nodes per axis: 4 for
@@ -524,7 +500,7 @@ __global__ void __launch_bounds__(kScatThreads, 2) k_brick_scatter(
       }
       __syncwarp();
       const uint32_t w = __float_as_uint(r.w);
-      const float d0[3] = {r.x, r.y, r.z};
+      const float t[3] = {r.x, r.y, r.z};
       float v[3][2];
       bool in[3];
       int at[3], lo[3];
@@ -534,10 +510,11 @@ __global__ void __launch_bounds__(kScatThreads, 2) k_brick_scatter(
         lo[a] = (int)((e.y >> (8 * a)) & 255u) - 64;
         at[a] = (lo[a] & ~1) + 2 * ql;
         const int q = at[a] - lo[a];  // -1 at the least
-        const int nw = rec_nw(w, a);
-        const float d = d0[a] + (float)q, dn = d0[a] + (float)(q + 1);
-        v[a][0] = q >= 0 && q < nw ? ex2_approx(-kp.beta[a] * d * d) : 0.f;
-        v[a][1] = q + 1 < nw ? ex2_approx(-kp.beta[a] * dn * dn) : 0.f;
+        const int nw = erpp_rec_nw(w, a);
+        const float k = (float)(erpp_rec_off(kp, w, a) + q);
+        const float d = k - t[a], dn = (k + 1.f) - t[a];
+        v[a][0] = q >= 0 && q < nw ? erpp_ex2(-kp.beta[a] * d * d) : 0.f;
+        v[a][1] = q + 1 < nw ? erpp_ex2(-kp.beta[a] * dn * dn) : 0.f;
         in[a] = live && q < nw && (unsigned)at[a] < 16u;
       }
       const float x0 = v[0][0] * sB, x1 = v[0][1] * sB;
@@ -560,8 +537,8 @@ __global__ void __launch_bounds__(kScatThreads, 2) k_brick_scatter(
       if (in[2]) *reinterpret_cast<float2*>(wt + 16 + at[2]) = make_float2(v[2][0], v[2][1]);
       if (live && ql == 0) {
         // the warps whose rows and planes the window reaches: bit 8 yh + zp
-        const int y1 = lo[1] + rec_nw(w, 1) - 1;
-        const int za = max(lo[2], 0) >> 1, zb = min(lo[2] + rec_nw(w, 2) - 1, 15) >> 1;
+        const int y1 = lo[1] + erpp_rec_nw(w, 1) - 1;
+        const int za = max(lo[2], 0) >> 1, zb = min(lo[2] + erpp_rec_nw(w, 2) - 1, 15) >> 1;
         const uint32_t zm = (2u << zb) - (1u << za);
         mask[p0 + i] = (lo[1] < 8 ? zm : 0u) | (y1 >= 8 ? zm << 8 : 0u);
       }
@@ -791,7 +768,7 @@ cudaError_t bricks_alloc(erpp_ctx* c, int64_t cap) {
   if (e == cudaSuccess) e = cudaMalloc(&k.pidx, sizeof(int32_t) * n);
   if (e == cudaSuccess) e = cudaMalloc(&k.pbrick, sizeof(int32_t) * n);
   if (e == cudaSuccess) e = cudaMalloc(&k.slot, sizeof(int32_t) * n);
-  if (e == cudaSuccess) e = cudaMalloc(&k.up, sizeof(float4) * n);
+  if (e == cudaSuccess) e = cudaMalloc(&k.rec_in, sizeof(float4) * n);
   if (e == cudaSuccess) e = cudaMalloc(&k.fs, sizeof(float4) * n);
   if (e == cudaSuccess) e = cudaMalloc(&k.rec, sizeof(float4) * n);
   if (e == cudaSuccess) e = cudaMalloc(&k.win, sizeof(uint32_t) * n);
@@ -804,14 +781,14 @@ void bricks_free(erpp_ctx* c) {
   cudaFree(k.pidx);
   cudaFree(k.pbrick);
   cudaFree(k.slot);
-  cudaFree(k.up);
+  cudaFree(k.rec_in);
   cudaFree(k.fs);
   cudaFree(k.rec);
   cudaFree(k.win);
   k.win = nullptr;
   k.key = nullptr;
   k.pidx = k.pbrick = k.slot = nullptr;
-  k.up = k.fs = k.rec = nullptr;
+  k.rec_in = k.fs = k.rec = nullptr;
 }
 
 // Sorts n particles at x into bricks: bk.rec in order, bk.slot each particle's
@@ -822,13 +799,11 @@ cudaError_t brick_sort(erpp_ctx* c, int64_t n, const double* const x[3], cudaStr
   cudaError_t e = cudaMemsetAsync(k.cnt, 0, sizeof(int32_t) * 2 * (size_t)nb, st);
   if (e != cudaSuccess) return e;
   const unsigned blocks = (unsigned)((n + 255) / 256);
-  // between the kernels of the sort: the windows in input order (where the
-  // gathered velocities go later) and in order of arrival (the forces)
-  float4* rec_in = k.up;
+  // the records in order of arrival: where the forces go later
   float4* rec_tmp = k.fs;
   ++c->launches;
   e = erpp_launch_pdl(k_brick_count, dim3(blocks), dim3(256), 0, st, 0u, c->kp, k.dims, n, x[0],
-                      x[1], x[2], rec_in, k.key, k.cnt, c->err);
+                      x[1], x[2], k.rec_in, k.key, k.cnt, c->err);
   if (e != cudaSuccess) return e;
   if (nb <= kBrickScanOne) {
     ++c->launches;
@@ -840,7 +815,7 @@ cudaError_t brick_sort(erpp_ctx* c, int64_t n, const double* const x[3], cudaStr
   if (e != cudaSuccess) return e;
   c->launches += 2;
   e = erpp_launch_pdl(k_brick_place, dim3(blocks), dim3(256), 0, st, 0u, n, (const int2*)k.key,
-                      (const float4*)rec_in, (const int32_t*)k.start, rec_tmp, k.pidx, k.pbrick,
+                      (const float4*)k.rec_in, (const int32_t*)k.start, rec_tmp, k.pidx, k.pbrick,
                       k.slot);
   if (e != cudaSuccess) return e;
   return erpp_launch_pdl(k_brick_order, dim3(blocks), dim3(256), 0, st, 0u, n, nb,
@@ -853,8 +828,8 @@ cudaError_t brick_forces(erpp_ctx* c, int64_t n, const double* const D[3], float
                          cudaStream_t st) {
   erpp_bricks& k = c->bk;
   ++c->launches;
-  k_brick_forces<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(c->kp, n, D[0], D[1], D[2], scale,
-                                                              k.rec, k.key, k.slot, k.fs, k.bmax);
+  k_brick_forces<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(
+      c->kp, n, D[0], D[1], D[2], scale, k.rec, k.key, k.slot, k.fs, k.bmax);
   return cudaGetLastError();
 }
 

@@ -53,6 +53,10 @@
 // 22-26 = window length on x / y / z, bit 31 = valid.
 #define ERPP_GEO_VALID 0x80000000u
 
+// Pieces of a tile that one block of the x/y-halo tile gather takes; a denser
+// tile's further chunks are listed by the binning.
+#define ERPP_GATHER_CHUNK 1024
+
 // Particle indices are 31-bit; the packed piece base is 17 bits.
 #define ERPP_MAX_PARTICLES ((int64_t)0x7fffffff)
 #define ERPP_BASE_BITS 17
@@ -138,9 +142,9 @@ struct erpp_bricks {
   int32_t* pidx;    // [cap] in order of arrival: particle
   int32_t* pbrick;  // [cap] in order of arrival: brick
   int32_t* slot;    // [cap] per particle: place in the order of the records
-  float4* rec;      // [cap] records in order: distances to the window's first nodes, window word
+  float4* rec;      // [cap] records in order: fractional position, window word
   uint32_t* win;    // [cap] the window words alone
-  float4* up;       // [cap] in order: gathered velocity (scratch of the sort before)
+  float4* rec_in;   // [cap] records in input order (scratch of the sort)
   float4* fs;       // [cap] in order: scaled force (scratch of the sort before)
 };
 
@@ -190,8 +194,11 @@ struct erpp_ctx {
   int64_t ff_n;           // particle count since the last first step (-1: none)
   int4* entries;
   int64_t entries_cap;
+  int2* gather_items;     // [entries_cap / ERPP_GATHER_CHUNK + 1] x/y-halo tiles: further
+                          // chunks of dense tiles (tile, first record); their number
+                          // follows tile_cnt and is cleared with it
   float* halo;            // scatter x-halo columns, [ntiles][3][T_z][T_y][xhlo + xhhi]
-  int32_t* tile_cnt;      // [32 ntiles]: pieces per (tile, bucket) bin
+  int32_t* tile_cnt;      // [32 ntiles + 1]: pieces per (tile, bucket) bin; gather_items' number
   int32_t* tile_start;    // [32 ntiles + 1]
   int32_t* piece_slot;    // [maxseg product][cap]: each piece's place in its bin
   int32_t* scan_tmp;      // [ceil(32 ntiles / 4096)] chunk totals of the scan
@@ -217,6 +224,12 @@ struct erpp_acc {
   const float4* up_part;    // x/y-halo tiles: per piece
   const int32_t* piece_slot;// [k][n]: place of particle i's k-th piece
   int64_t n;
+  // source from brick-sorted particles (bfs not null): their forces go to their
+  // records' places, with the bricks' force maxima
+  const int32_t* bslot;
+  const int2* bkey;
+  float4* bfs;
+  int32_t* bmax;
 };
 
 // One box of the multi-box launches (batched boxes): its kernel parameters,
@@ -272,6 +285,7 @@ cudaError_t brick_forces(erpp_ctx* c, int64_t n, const double* const D[3], float
                          cudaStream_t st);
 cudaError_t brick_scatter(erpp_ctx* c, float* S, cudaStream_t st);
 
+
 erpp_status derive_ctx(const erpp_params* p, erpp_ctx* c);
 erpp_status ensure_capacity(erpp_ctx* c, int64_t n);  // may allocate (synchronous)
 int xw_len(const erpp_kparams& kp);
@@ -290,11 +304,11 @@ cudaError_t bin_particles(erpp_ctx* ctx, int64_t n, const double* const x[3], bo
                           cudaStream_t st);
 cudaError_t launch_gather_f32(erpp_ctx* ctx, const float* u, int64_t n, cudaStream_t st);
 cudaError_t launch_scatter_f32(erpp_ctx* ctx, float* S, cudaStream_t st);  // + x-halo merge
-cudaError_t launch_gather_f32_4(erpp_ctx* ctx, const float* u, cudaStream_t st);
+cudaError_t launch_gather_f32_4(erpp_ctx* ctx, const float* u, int64_t n, cudaStream_t st);
 // General force on x/y-halo tiles: the gather of the velocity and of its
 // Laplacian (per-piece sums in up_part and lap_part), and their per-particle
 // totals: up = norm * sum + shear y (x component), lap = norm * sum.
-cudaError_t launch_gather_lap_f32_4(erpp_ctx* ctx, const float* u, cudaStream_t st);
+cudaError_t launch_gather_lap_f32_4(erpp_ctx* ctx, const float* u, int64_t n, cudaStream_t st);
 cudaError_t launch_finalize_full(erpp_ctx* ctx, int64_t n, const double* const x[3],
                                  double* const up[3], double* lap, int64_t lap_stride,
                                  cudaStream_t st);
@@ -328,7 +342,7 @@ cudaError_t launch_prep_fscat(erpp_ctx* ctx, int64_t n, const double* const D[3]
 cudaError_t launch_advance(erpp_ctx* ctx, const erpp_particles* P, const double* const up[3],
                            bool from_acc, bool write_fscat, int first_step, cudaStream_t st,
                            const double* const xs[3] = nullptr,
-                           const double* const Ds[3] = nullptr);
+                           const double* const Ds[3] = nullptr, bool bricks = false);
 // ERPP_FULL_FORCE: gathered velocity (plus the mean shear) and its Laplacian in
 // the particle position, into up and ctx->ff_lap; then the general-force
 // advance from them (ctx->ff_prev holds u~ and lap u~ of the previous step).
@@ -481,6 +495,42 @@ __device__ __forceinline__ int erpp_geo_nw(uint32_t pack, int a) {
 
 __device__ __forceinline__ void erpp_set_err(uint32_t* err, uint32_t bit) {
   if (err) atomicOr(err, bit);
+}
+
+// Record of a brick-sorted particle: its fractional position in the home cell
+// (the distance of window position q is then off + q - t, with one rounding) and
+// a word: byte a holds the window's first node's position in the brick on axis
+// a plus 8 (4 .. 15) and, in its upper half, the window's length; bits 24 + 2a
+// hold off + floor(c') + 1, off the first node relative to the home cell.
+__device__ __forceinline__ int erpp_rec_lo(uint32_t w, int a) {
+  return (int)((w >> (8 * a)) & 15u) - 8;
+}
+__device__ __forceinline__ int erpp_rec_nw(uint32_t w, int a) {
+  return (int)((w >> (8 * a + 4)) & 15u);
+}
+__device__ __forceinline__ int erpp_rec_off(const erpp_kparams& kp, uint32_t w, int a) {
+  return (int)((w >> (24 + 2 * a)) & 3u) - kp.cp_int[a] - 1;
+}
+
+// A particle's force for the source from sorted particles, stored at its
+// record's place (a component that is not finite gives no force), and the
+// brick's largest |component| (as the bits of a non-negative float).
+__device__ __forceinline__ void erpp_put_force(float4* __restrict__ fs,
+                                               int32_t* __restrict__ bmax, int slot, int brick,
+                                               float f0, float f1, float f2) {
+  f0 = isfinite(f0) ? f0 : 0.f;
+  f1 = isfinite(f1) ? f1 : 0.f;
+  f2 = isfinite(f2) ? f2 : 0.f;
+  fs[slot] = make_float4(f0, f1, f2, 0.f);
+  const int m = __float_as_int(fmaxf(fabsf(f0), fmaxf(fabsf(f1), fabsf(f2))));
+  if (m > bmax[brick]) atomicMax(&bmax[brick], m);
+}
+
+// 2^x by the special-function unit (exp2f for x >= -126; smaller powers give 0).
+__device__ __forceinline__ float erpp_ex2(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;\n" : "=f"(y) : "f"(x));
+  return y;
 }
 
 // Programmatic dependent launch between the kernels of a step.  Each such

@@ -382,7 +382,12 @@ __device__ __forceinline__ void advance_one(const erpp_kparams& kp, int64_t i, c
       P.D[a][i] = Dn[a];
     }
   }
-  if (fscat) {
+  if (FROM_ACC && acc.bfs) {
+    const int slot = acc.bslot[i];
+    const float s = -norm * kp.inv_rho_dV;
+    if (slot >= 0)
+      erpp_put_force(acc.bfs, acc.bmax, slot, acc.bkey[i].x, s * Dnf[0], s * Dnf[1], s * Dnf[2]);
+  } else if (fscat) {
     const float s = -norm * kp.inv_rho_dV;
     const float f0 = s * Dnf[0], f1 = s * Dnf[1], f2 = s * Dnf[2];
     fscat[i] = make_float4(f0, f1, f2, fmaxf(fabsf(f0), fmaxf(fabsf(f1), fabsf(f2))));
@@ -423,8 +428,7 @@ __global__ void __launch_bounds__(256) k_advance_multi(const erpp_box_dev* __res
   P.radius = B.radius;
   P.rho_p = B.rho_p;
   UpPtrs U = {{nullptr, nullptr, nullptr}};
-  erpp_acc acc;
-  acc.up_acc = nullptr;
+  erpp_acc acc = {};
   acc.stride = B.cap;
   acc.up_part = B.up_part;
   acc.piece_slot = B.piece_slot;
@@ -478,7 +482,7 @@ __global__ void k_finalize_full(erpp_kparams kp, int64_t n, erpp_acc acc,
 }
 
 erpp_acc acc_of(const erpp_ctx* ctx, int64_t n) {
-  erpp_acc a;
+  erpp_acc a = {};
   a.up_acc = ctx->up_acc;
   a.stride = ctx->cap;
   a.up_part = ctx->up_part;
@@ -622,7 +626,7 @@ static PartPtrs part_ptrs(const erpp_particles* P) {
 
 cudaError_t launch_advance(erpp_ctx* ctx, const erpp_particles* P, const double* const up[3],
                            bool from_acc, bool write_fscat, int first_step, cudaStream_t st,
-                           const double* const xs[3], const double* const Ds[3]) {
+                           const double* const xs[3], const double* const Ds[3], bool bricks) {
   const int64_t n = P->n;
   if (n <= 0) return cudaSuccess;
   PartPtrs q = part_ptrs(P);
@@ -638,7 +642,14 @@ cudaError_t launch_advance(erpp_ctx* ctx, const erpp_particles* P, const double*
   const bool f32 = !ctx->fp64;
   ++ctx->launches;
   if (from_acc) {
-    k_advance<true, true><<<blocks, 256, 0, st>>>(ctx->kp, n, q, U, acc_of(ctx, n), ctx->geo_t,
+    erpp_acc a = acc_of(ctx, n);
+    if (write_fscat && bricks) {
+      a.bslot = ctx->bk.slot;
+      a.bkey = ctx->bk.key;
+      a.bfs = ctx->bk.fs;
+      a.bmax = ctx->bk.bmax;
+    }
+    k_advance<true, true><<<blocks, 256, 0, st>>>(ctx->kp, n, q, U, a, ctx->geo_t,
                                                   ctx->geo_c, fs, first_step);
   } else if (f32) {
     k_advance<false, true><<<blocks, 256, 0, st>>>(ctx->kp, n, q, U, erpp_acc{}, nullptr,

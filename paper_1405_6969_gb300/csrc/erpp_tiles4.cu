@@ -71,6 +71,7 @@
 #include <cudaTypedefs.h>
 #include <cuda_runtime.h>
 
+#include <math.h>
 #include <string.h>
 
 #include <algorithm>
@@ -132,7 +133,7 @@ __device__ __forceinline__ void make_ex(const Piece4& pc, float d0x, float bx, f
 #pragma unroll
   for (int q = 0; q < XM; ++q) {
     const float d = d0x + (float)(pc.qa + q);
-    ex[q] = q < pc.lx ? exp2f(-bx * d * d) : 0.f;
+    ex[q] = q < pc.lx ? erpp_ex2(-bx * d * d) : 0.f;
   }
 }
 
@@ -307,13 +308,18 @@ struct Carve {
 // slots may reach past the last staged row.
 constexpr int kFieldPad = 16;
 
+// Schedule entries of up to NU units: whole rounds of 256, 384 or 512 threads.
+__host__ __device__ constexpr int sched_slots(int NU) {
+  return (NU + 511) / 512 * 512 > (NU + 383) / 384 * 384 ? (NU + 511) / 512 * 512
+                                                         : (NU + 383) / 384 * 384;
+}
+
 // The unit words, the schedule and the gather's piece accumulators are sized
-// for the tile's tz planes (a piece has at most tz units); the schedule holds
-// whole rounds of up to 512 threads.
+// for the tile's tz planes (a piece has at most tz units).
 template <int PB>
 __host__ __device__ inline size_t carve_bytes(int plane, int tz, int copies, bool gather,
                                               bool lap = false) {
-  const int NU = PB * tz, NS = (NU + 511) & ~511;
+  const int NU = PB * tz, NS = sched_slots(NU);
   size_t b = ((size_t)copies * plane + kFieldPad) * 4;
   b += (size_t)PB * 16;          // rec
   if (!gather) b += (size_t)PB * 16;  // fsb
@@ -330,7 +336,7 @@ __host__ __device__ inline size_t carve_bytes(int plane, int tz, int copies, boo
 template <int PB>
 __device__ inline Carve<PB> carve(unsigned char* base, int plane, int tz, int copies, bool gather,
                                   bool lap = false) {
-  const int NU = PB * tz, NS = (NU + 511) & ~511;
+  const int NU = PB * tz, NS = sched_slots(NU);
   Carve<PB> c;
   size_t o = 0;
   c.field = reinterpret_cast<float*>(base);
@@ -584,8 +590,8 @@ struct UnitRows {
   float d0y, ezz;
 };
 
-// The gather of one tile, called by the whole block (the body of k_gather4
-// and of the multi-box gather).  XM: longest x-window; LMIN: shortest (slots
+// The gather of the pieces [e0, e1) of one tile, called by the whole block (the
+// body of k_gather4 and of the multi-box gather).  XM: longest x-window; LMIN: shortest (slots
 // q >= LMIN are tested); XW: 8 for windows of at most 7 nodes, else 16 (sets
 // the pieces per batch).  LAP: also the Laplacian of the gathered velocity
 // (general force, Eq. force_particle): per row, the same loaded values
@@ -596,13 +602,11 @@ struct UnitRows {
 template <int XM, int LMIN, int XW, int NT, bool LAP, int PB>
 __device__ __forceinline__ int gather_tile4(
     const erpp_kparams& kp, int tile, const float* __restrict__ u, const CUtensorMap* tmap,
-    int use_tma, const int32_t* __restrict__ start, const int4* __restrict__ entries,
-    int64_t ecap, const float* __restrict__ d0x, const float4* __restrict__ lapc,
+    int use_tma, int e0, int e1, const int4* __restrict__ entries,
+    const float* __restrict__ d0x, const float4* __restrict__ lapc,
     float4* __restrict__ up_part, float4* __restrict__ lap_part, uint32_t* err,
     unsigned char* smem_raw, SchedState& ss, uint64_t& tma_bar, uint64_t& stall_bar) {
   static_assert(PB <= 1024, "unit words hold the piece index in 10 bits");
-  const int e0 = start[tile];
-  const int e1 = (int)min((int64_t)start[tile + 1], ecap);
   if (e0 >= e1) return 0;
   const int tzs = kp.T[2];  // planes per tile: units per piece, at most
   const Carve<PB> cv = carve<PB>(smem_raw, kp.plane, tzs, 3, true, LAP);
@@ -742,7 +746,7 @@ __device__ __forceinline__ int gather_tile4(
         float dy = ur.d0y + (float)ur.rot;
 #pragma unroll 1
         for (int t = 0; t < rows; ++t) {
-          const float e = exp2f(-fmaf(by * dy, dy, ur.ezz));
+          const float e = erpp_ex2(-fmaf(by * dy, dy, ur.ezz));
           const bool in = t < ur.ly;
           const float wr = in ? e : 0.f;
           float x0 = 0.f, x1 = 0.f, x2 = 0.f;
@@ -828,19 +832,38 @@ __device__ __forceinline__ int gather_tile4(
   return (tma || rows) ? 2 : 0;
 }
 
+// The first nextra blocks take the further chunks of dense tiles in turn (the
+// binning lists the pieces kGatherChunk, 2 kGatherChunk, ... of every tile), the
+// others a tile's first chunk each: a tile that holds a cluster is gathered by
+// many blocks (100k particles in 50 clusters: 700 us in one block per tile).
 template <int XM, int LMIN, int XW, int NT, bool LAP, int PB>
 __global__ void __launch_bounds__(NT, LAP ? 2 : 768 / NT) k_gather4(
     erpp_kparams kp, const float* __restrict__ u, const __grid_constant__ CUtensorMap tmap,
     int use_tma, const int32_t* __restrict__ start, const int4* __restrict__ entries,
     int64_t ecap, const float* __restrict__ d0x, const float4* __restrict__ lapc,
-    float4* __restrict__ up_part, float4* __restrict__ lap_part, uint32_t* err) {
+    float4* __restrict__ up_part, float4* __restrict__ lap_part, int nextra,
+    const int32_t* __restrict__ nitems, const int2* __restrict__ items, uint32_t* err) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ SchedState ss;
   __shared__ __align__(8) uint64_t tma_bar;
   __shared__ __align__(8) uint64_t stall_bar;  // debug_stall only: never completed
-  gather_tile4<XM, LMIN, XW, NT, LAP, PB>(kp, blockIdx.x, u, &tmap, use_tma, start, entries,
-                                          ecap, d0x, lapc, up_part, lap_part, err, smem_raw, ss,
-                                          tma_bar, stall_bar);
+  const bool extra = (int)blockIdx.x < nextra;
+  const int nit = extra ? *nitems : 1;
+  for (int it = extra ? (int)blockIdx.x : 0; it < nit; it += nextra) {
+    const int tile = extra ? items[it].x : (int)blockIdx.x - nextra;
+    const int e0 = extra ? items[it].y : start[tile];
+    int e1 = (int)min((int64_t)start[tile + 1], ecap);
+    if (nextra > 0) e1 = min(e1, e0 + ERPP_GATHER_CHUNK);
+    const int r = gather_tile4<XM, LMIN, XW, NT, LAP, PB>(kp, tile, u, &tmap, use_tma, e0, e1,
+                                                          entries, d0x, lapc, up_part, lap_part,
+                                                          err, smem_raw, ss, tma_bar, stall_bar);
+    if (!extra || (r & 1)) break;
+    __syncthreads();  // every thread is done with the tile and its barriers
+    if (threadIdx.x == 0 && (r & 2)) {
+      mbar_inval(&tma_bar);
+      if (kp.debug_stall) mbar_inval(&stall_bar);
+    }
+  }
 }
 
 // MODE 0: 32-bit fixed point (FP32 atomics on dense tiles); MODE 1: split
@@ -985,7 +1008,7 @@ __device__ __forceinline__ TileAcc scatter_tile(const erpp_kparams& kp, int tile
           ur.rot = (int)(w >> 31);
           ur.d0y = pc.d0y;
           const float dz = pc.d0z + (float)z;
-          const float wz = exp2f(-bz * dz * dz);
+          const float wz = erpp_ex2(-bz * dz * dz);
           const float4 fv = cv.fsb[k];
           f0 = fv.x * wz;
           f1 = fv.y * wz;
@@ -1015,7 +1038,7 @@ __device__ __forceinline__ TileAcc scatter_tile(const erpp_kparams& kp, int tile
             const unsigned lo = 3u * pl4;  // the low sums follow the three components
 #pragma unroll 1
             for (int t = 0; t < rows; ++t) {
-              const float e = exp2f(-by * dy * dy);
+              const float e = erpp_ex2(-by * dy * dy);
               const int W = t < ur.ly ? __float2int_rn(e * 2147483648.f) : 0;
               row_red_split<0, XM, LMIN, NQ>(ar, ar + pl4, ar + 2 * pl4, lo, G0, G1, G2, W, ur.lx);
               ar += px4;
@@ -1027,7 +1050,7 @@ __device__ __forceinline__ TileAcc scatter_tile(const erpp_kparams& kp, int tile
           } else if (fixedp) {
 #pragma unroll 1
             for (int t = 0; t < rows; ++t) {
-              const float e = exp2f(-by * dy * dy);
+              const float e = erpp_ex2(-by * dy * dy);
               const int W = t < ur.ly ? __float2int_rn(e * 2147483648.f) : 0;
               row_red_fixed<0, XM, LMIN, NQ>(ar, ar + pl4, ar + 2 * pl4, G0, G1, G2, W, ur.lx);
               ar += px4;
@@ -1039,7 +1062,7 @@ __device__ __forceinline__ TileAcc scatter_tile(const erpp_kparams& kp, int tile
           } else {
 #pragma unroll 1
             for (int t = 0; t < rows; ++t) {
-              const float e = exp2f(-by * dy * dy);
+              const float e = erpp_ex2(-by * dy * dy);
               const float wy = t < ur.ly ? e : 0.f;
               row_red_f32<0, XM, LMIN, NQ>(ar, ar + pl4, ar + 2 * pl4, ex, f0, f1, f2, wy, ur.lx);
               ar += px4;
@@ -1447,9 +1470,12 @@ cudaError_t gather4_nt(erpp_ctx* ctx, const float* u, cudaStream_t st) {
   memset(&map, 0, sizeof(map));
   const int use_tma = field_tensor_map(kp, u, &map) ? 1 : 0;
   ++ctx->launches;
-  kern<<<kp.ntiles, NT, sm, st>>>(kp, u, map, use_tma, ctx->tile_start, ctx->entries,
-                                  ctx->entries_cap, ctx->d0x, ctx->lapc, ctx->up_part,
-                                  ctx->lap_part, ctx->err);
+  const int nextra =
+      ctx->gather_items ? (int)std::min<int64_t>(ctx->entries_cap / ERPP_GATHER_CHUNK, 608) : 0;
+  kern<<<kp.ntiles + nextra, NT, sm, st>>>(kp, u, map, use_tma, ctx->tile_start, ctx->entries,
+                                           ctx->entries_cap, ctx->d0x, ctx->lapc, ctx->up_part,
+                                           ctx->lap_part, nextra, ctx->tile_cnt + kp.ntiles,
+                                           ctx->gather_items, ctx->err);
   return cudaGetLastError();
 }
 
@@ -1465,9 +1491,20 @@ inline bool gather_big_batch(size_t small, size_t big) {
   return std::min(gather_blocks_per_sm(big), 3) >= std::min(gather_blocks_per_sm(small), 3);
 }
 
+// Lanes that a tile's batches occupy with blocks of NT threads, per unit: whole
+// rounds of NT lanes for the units of a batch of a tile of average density
+// (a piece has xs planes cut at the tile's).
+inline double gather_lanes(const erpp_kparams& kp, int64_t n, int PB, int NT) {
+  const double lz = 2.0 * kp.cp[2];
+  const double units = (double)n * lz / ((double)kp.nt[0] * kp.nt[1] * kp.n[2]) * kp.T[2];
+  const double pieces = (double)n * (1.0 + (lz - 1.0) / kp.T[2]) / kp.ntiles;
+  const double nb = std::max(1.0, ceil(pieces / PB));
+  return ceil(units / nb / NT) * NT;
+}
+
 // LAP (the general force's gather) always runs 256-thread blocks.
 template <int XM, int LMIN, int XW, bool LAP = false>
-cudaError_t gather4(erpp_ctx* ctx, const float* u, cudaStream_t st) {
+cudaError_t gather4(erpp_ctx* ctx, const float* u, int64_t n, cudaStream_t st) {
   constexpr int PB = Batch<XW>::kPB;
   if constexpr (LAP) {
     return gather4_nt<XM, LMIN, XW, 256, true, PB>(ctx, u, st);
@@ -1477,6 +1514,13 @@ cudaError_t gather4(erpp_ctx* ctx, const float* u, cudaStream_t st) {
     if (gather_big_batch(carve_bytes<PB>(kp.plane, kp.T[2], 3, true),
                          carve_bytes<2 * PB>(kp.plane, kp.T[2], 3, true)))
       return gather4_nt<XM, LMIN, XW, 256, false, 2 * PB>(ctx, u, st);
+    // Shared memory for two blocks per SM only: 384 threads each where that
+    // leaves fewer lanes idle in a batch's last round (512x256x256, 1M
+    // particles, 64x16x4 tiles: 366 units a batch, 346 -> 329 us; 256^3, 1M:
+    // 490 units, 306 us with 256 threads, 334 us with 384).
+    if (gather_blocks_per_sm(carve_bytes<PB>(kp.plane, kp.T[2], 3, true)) <= 2 &&
+        gather_lanes(kp, n, PB, 384) < gather_lanes(kp, n, PB, 256))
+      return gather4_nt<XM, LMIN, XW, 384, false, PB>(ctx, u, st);
     return gather4_nt<XM, LMIN, XW, 256, false, PB>(ctx, u, st);
   }
 }
@@ -1600,8 +1644,8 @@ __global__ void __launch_bounds__(256, 3) k_gather4_multi(const BoxTiles* __rest
     const int2 bt = items[it];
     const BoxTiles& B = boxes[bt.x];
     const int r = gather_tile4<XM, LMIN, XW, 256, false, Batch<XW>::kPB>(
-        B.kp, bt.y, B.u, &B.tmap, B.use_tma, B.start, B.entries, B.ecap, B.d0x, nullptr,
-        B.up_part, nullptr, B.err, smem_raw, ss, tma_bar, stall_bar);
+        B.kp, bt.y, B.u, &B.tmap, B.use_tma, B.start[bt.y],
+        (int)min((int64_t)B.start[bt.y + 1], B.ecap), B.entries, B.d0x, nullptr, B.up_part, nullptr, B.err, smem_raw, ss, tma_bar, stall_bar);
     // every thread is done with the tile, its barriers and `item`
     __syncthreads();
     if (r & 1) break;  // a bounded wait ran out (recorded): the block stops
@@ -1688,24 +1732,24 @@ size_t smem_bytes4(const erpp_kparams& kp, int copies, bool gather) {
 }
 
 template <bool LAP>
-cudaError_t gather4_variant(erpp_ctx* ctx, const float* u, cudaStream_t st) {
+cudaError_t gather4_variant(erpp_ctx* ctx, const float* u, int64_t n, cudaStream_t st) {
   switch (variant4(ctx->kp)) {
-    case 0: return gather4<7, 6, 8, LAP>(ctx, u, st);
-    case 1: return gather4<7, 5, 8, LAP>(ctx, u, st);
-    case 2: return gather4<10, 9, 16, LAP>(ctx, u, st);
-    case 3: return gather4<10, 8, 16, LAP>(ctx, u, st);
-    case 5: return gather4<7, 1, 8, LAP>(ctx, u, st);
-    case 6: return gather4<10, 1, 16, LAP>(ctx, u, st);
-    default: return gather4<16, 1, 16, LAP>(ctx, u, st);
+    case 0: return gather4<7, 6, 8, LAP>(ctx, u, n, st);
+    case 1: return gather4<7, 5, 8, LAP>(ctx, u, n, st);
+    case 2: return gather4<10, 9, 16, LAP>(ctx, u, n, st);
+    case 3: return gather4<10, 8, 16, LAP>(ctx, u, n, st);
+    case 5: return gather4<7, 1, 8, LAP>(ctx, u, n, st);
+    case 6: return gather4<10, 1, 16, LAP>(ctx, u, n, st);
+    default: return gather4<16, 1, 16, LAP>(ctx, u, n, st);
   }
 }
 
-cudaError_t launch_gather_f32_4(erpp_ctx* ctx, const float* u, cudaStream_t st) {
-  return gather4_variant<false>(ctx, u, st);
+cudaError_t launch_gather_f32_4(erpp_ctx* ctx, const float* u, int64_t n, cudaStream_t st) {
+  return gather4_variant<false>(ctx, u, n, st);
 }
 
-cudaError_t launch_gather_lap_f32_4(erpp_ctx* ctx, const float* u, cudaStream_t st) {
-  return gather4_variant<true>(ctx, u, st);
+cudaError_t launch_gather_lap_f32_4(erpp_ctx* ctx, const float* u, int64_t n, cudaStream_t st) {
+  return gather4_variant<true>(ctx, u, n, st);
 }
 
 cudaError_t launch_scatter_f32_4(erpp_ctx* ctx, float* S, cudaStream_t st) {

@@ -148,3 +148,23 @@ def test_invalid_particles_and_forces(erpp, oracle_lib):
     ctx.scatter_source(cuda(x), cuda(np.zeros_like(D)), S=S)
     ctx.check()
     assert not S.any()
+
+
+def test_gather_of_dense_tiles(erpp, oracle_lib):
+    """Tiles of more than 1024 pieces are gathered by several blocks: every
+    particle of a cluster inside one tile, next to sparse tiles, equals the
+    oracle's and, bit for bit, the gather of the same particle in a sparse
+    cloud (its sums do not depend on its neighbours)."""
+    import torch
+    w = work((72, 40, 24), 6000, 1.0, "clusters", 0.08)
+    x = I.make_particles(w, None).x
+    grid, _ = I.make_grid(w)
+    u = cuda(grid, torch.float32)
+    ctx = erpp.Context(w.params(), precision="fp32")
+    up = ctx.interpolate(u, cuda(x))
+    ctx.check()
+    assert rel(up.cpu().numpy(), oracle_lib.gather(w.params(), x, grid)) < TOL
+    few = np.ascontiguousarray(x[:, ::60])
+    alone = ctx.interpolate(u, cuda(few))
+    ctx.check()
+    assert torch.equal(alone, up[:, ::60])
