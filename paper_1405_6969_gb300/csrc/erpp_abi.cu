@@ -187,6 +187,23 @@ erpp_status alloc_weight_tables(erpp_ctx* c) {
   return set_cuda_err(e);
 }
 
+// Whether an adjoint, which needs no scratch otherwise, takes the brick kernels:
+// where their scratch is there, or can be made without losing a step history
+// and outside a stream capture.
+bool adjoint_bricks(erpp_ctx* c, int64_t n, cudaStream_t st) {
+  if (c->fp64 || n <= 0 || !erpp::bricks_possible(c)) return false;
+  if (n > c->cap) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (c->kp.lag > 0 || c->kp.full_force ||
+        cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone ||
+        erpp::ensure_capacity(c, n) != ERPP_OK) {
+      cudaGetLastError();
+      return false;
+    }
+  }
+  return erpp::use_bricks(c, n);
+}
+
 erpp_status check_n(int64_t n) {
   if (n < 0 || n > ERPP_MAX_PARTICLES) return ERPP_EINVAL;
   return ERPP_OK;
@@ -583,8 +600,16 @@ erpp_status erpp_scatter_backward(erpp_ctx* c, int64_t n, const double* const x[
   if (n == 0) return ERPP_OK;
   if (!valid_vec(x) || !valid_vec(D) || !dx || !dx[0] || !dx[1] || !dx[2]) return ERPP_EINVAL;
   if (dD && (!dD[0] || !dD[1] || !dD[2])) return ERPP_EINVAL;
-  cudaError_t e = erpp::launch_adjoint(c, n, x, R, D, -1.0 / c->params.rho_f, 0.0, dD, dx,
-                                       (cudaStream_t)stream);
+  cudaStream_t st = (cudaStream_t)stream;
+  cudaError_t e;
+  if (adjoint_bricks(c, n, st)) {
+    e = erpp::brick_sort(c, n, x, true, st);
+    if (e == cudaSuccess)
+      e = erpp::brick_adjoint(c, n, x, (const float*)R, D, -1.0 / c->params.rho_f, 0.0, dD, dx,
+                              st);
+  } else {
+    e = erpp::launch_adjoint(c, n, x, R, D, -1.0 / c->params.rho_f, 0.0, dD, dx, st);
+  }
   return set_cuda_err(e);
 }
 
@@ -597,15 +622,21 @@ erpp_status erpp_gather_backward(erpp_ctx* c, int64_t n, const double* const x[3
   if (!du && !dx) return ERPP_EINVAL;
   cudaStream_t st = (cudaStream_t)stream;
   cudaError_t e = cudaSuccess;
-  if (dx && n > 0)
-    e = erpp::launch_adjoint(c, n, x, u, g, c->kp.dV, c->params.shear_rate, nullptr, dx, st);
+  // one sort serves both parts
+  const bool adj = dx && adjoint_bricks(c, n, st);
+  if (adj) e = erpp::brick_sort(c, n, x, true, st);
+  if (e == cudaSuccess && dx && n > 0)
+    e = adj ? erpp::brick_adjoint(c, n, x, (const float*)u, g, c->kp.dV, c->params.shear_rate,
+                                  nullptr, dx, st)
+            : erpp::launch_adjoint(c, n, x, u, g, c->kp.dV, c->params.shear_rate, nullptr, dx,
+                                   st);
   if (e == cudaSuccess && du) {
     erpp_status s = erpp::ensure_capacity(c, n);
     if (s) return s;
     if (c->fp64) {
       e = erpp::launch_scatter_f64(c, n, x, g, c->kp.dV, (double*)du, st);
     } else if (erpp::use_bricks(c, n)) {
-      e = erpp::brick_sort(c, n, x, st);
+      if (!adj) e = erpp::brick_sort(c, n, x, false, st);
       if (e == cudaSuccess) e = erpp::brick_forces(c, n, g, 1.0f, st);
       if (e == cudaSuccess) e = erpp::brick_scatter(c, (float*)du, st);
     } else {
@@ -643,7 +674,7 @@ cudaError_t scatter_source(erpp_ctx* c, int64_t n, const double* const x[3],
     return erpp::launch_scatter_f64(c, n, x, D, -1.0 / c->params.rho_f, (double*)S, st);
   cudaError_t e;
   if (use_bricks(c, n)) {
-    e = brick_sort(c, n, x, st);
+    e = brick_sort(c, n, x, false, st);
     if (e == cudaSuccess) e = brick_forces(c, n, D, -c->kp.inv_rho_dV, st);
     if (e == cudaSuccess) e = brick_scatter(c, (float*)S, st);
     return e;
@@ -804,7 +835,7 @@ erpp_status step_device(erpp_ctx* c, const void* u, const erpp_particles* P, voi
     if (c->prof_on) ev = c->prof_ev + 5 * (c->prof_n++ % kProfSets);
     if (ev) cudaEventRecord(ev[0], st);
     const bool bricks = use_bricks(c, n);
-    e = bricks ? brick_sort(c, n, xin, st) : cudaSuccess;
+    e = bricks ? brick_sort(c, n, xin, false, st) : cudaSuccess;
     if (e == cudaSuccess) e = erpp::bin_particles(c, n, xin, true, st);
     if (ev) cudaEventRecord(ev[1], st);
     if (e == cudaSuccess) e = erpp::launch_gather_f32(c, (const float*)u, n, st);

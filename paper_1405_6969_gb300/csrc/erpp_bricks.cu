@@ -185,7 +185,10 @@ __global__ void __launch_bounds__(256) k_brick_order(int64_t n, int nb,
                                                      const int32_t* __restrict__ start,
                                                      float4* __restrict__ rec,
                                                      uint32_t* __restrict__ win,
-                                                     int32_t* __restrict__ slot) {
+                                                     int32_t* __restrict__ slot,
+                                                     int32_t* __restrict__ ord, int tile_bricks,
+                                                     int chunk, int32_t* __restrict__ nitems,
+                                                     int2* __restrict__ items) {
   erpp_pdl_enter();
   const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= n || j >= start[nb]) return;
@@ -209,6 +212,14 @@ __global__ void __launch_bounds__(256) k_brick_order(int64_t n, int nb,
   rec[s + r] = v;
   win[s + r] = __float_as_uint(v.w);
   slot[me] = s + r;
+  if (ord) {
+    ord[s + r] = me;
+    // the further chunks of an adjoint tile of more than `chunk` particles
+    const int tile = b / tile_bricks;
+    const int off = s + r - start[tile * tile_bricks];
+    if (off >= chunk && off % chunk == 0)
+      items[atomicAdd(nitems, 1)] = make_int2(tile, s + r);
+  }
 }
 
 // Normalisation of a particle's weights (erpp_norm's arithmetic on its record).
@@ -733,11 +744,12 @@ cudaError_t bricks_alloc_tables(erpp_ctx* c) {
   }
   if (ng > (1 << 24) || k.dims.ng[1] > 65535 || k.dims.ng[2] > 65535) return cudaSuccess;
   k.nbricks = (int)(8 * ng);
-  // counts and force maxima, cleared together
-  cudaError_t e = cudaMalloc(&k.cnt, sizeof(int32_t) * 2 * (size_t)k.nbricks);
+  // counts, force maxima and the number of further adjoint chunks, cleared together
+  cudaError_t e = cudaMalloc(&k.cnt, sizeof(int32_t) * (2 * (size_t)k.nbricks + 1));
   if (e == cudaSuccess) e = cudaMalloc(&k.start, sizeof(int32_t) * ((size_t)k.nbricks + 4));
   if (e == cudaSuccess) e = cudaMalloc(&k.scan_tmp, sizeof(int32_t) * (k.nbricks / 4096 + 1));
   k.bmax = k.cnt ? k.cnt + k.nbricks : nullptr;
+  k.nitems = k.cnt ? k.cnt + 2 * (size_t)k.nbricks : nullptr;
   std::vector<int2> ax;
   for (int a = 0; a < 3; ++a)
     for (int g = 0; g < k.dims.ng[a]; ++g) {
@@ -757,7 +769,7 @@ void bricks_free_tables(erpp_ctx* c) {
   cudaFree(k.scan_tmp);
   cudaFree(k.axis);
   k.axis = nullptr;
-  k.cnt = k.start = k.scan_tmp = k.bmax = nullptr;
+  k.cnt = k.start = k.scan_tmp = k.bmax = k.nitems = nullptr;
 }
 
 cudaError_t bricks_alloc(erpp_ctx* c, int64_t cap) {
@@ -768,6 +780,8 @@ cudaError_t bricks_alloc(erpp_ctx* c, int64_t cap) {
   if (e == cudaSuccess) e = cudaMalloc(&k.pidx, sizeof(int32_t) * n);
   if (e == cudaSuccess) e = cudaMalloc(&k.pbrick, sizeof(int32_t) * n);
   if (e == cudaSuccess) e = cudaMalloc(&k.slot, sizeof(int32_t) * n);
+  if (e == cudaSuccess) e = cudaMalloc(&k.ord, sizeof(int32_t) * n);
+  if (e == cudaSuccess) e = cudaMalloc(&k.items, sizeof(int2) * (n / brick_chunk(c) + 1));
   if (e == cudaSuccess) e = cudaMalloc(&k.rec_in, sizeof(float4) * n);
   if (e == cudaSuccess) e = cudaMalloc(&k.fs, sizeof(float4) * n);
   if (e == cudaSuccess) e = cudaMalloc(&k.rec, sizeof(float4) * n);
@@ -781,22 +795,26 @@ void bricks_free(erpp_ctx* c) {
   cudaFree(k.pidx);
   cudaFree(k.pbrick);
   cudaFree(k.slot);
+  cudaFree(k.ord);
+  cudaFree(k.items);
+  k.items = nullptr;
   cudaFree(k.rec_in);
   cudaFree(k.fs);
   cudaFree(k.rec);
   cudaFree(k.win);
   k.win = nullptr;
   k.key = nullptr;
-  k.pidx = k.pbrick = k.slot = nullptr;
+  k.pidx = k.pbrick = k.slot = k.ord = nullptr;
   k.rec_in = k.fs = k.rec = nullptr;
 }
 
 // Sorts n particles at x into bricks: bk.rec in order, bk.slot each particle's
 // place (-1: invalid position), bk.start the bricks' ranges.
-cudaError_t brick_sort(erpp_ctx* c, int64_t n, const double* const x[3], cudaStream_t st) {
+cudaError_t brick_sort(erpp_ctx* c, int64_t n, const double* const x[3], bool for_adjoint,
+                       cudaStream_t st) {
   erpp_bricks& k = c->bk;
   const int nb = k.nbricks;
-  cudaError_t e = cudaMemsetAsync(k.cnt, 0, sizeof(int32_t) * 2 * (size_t)nb, st);
+  cudaError_t e = cudaMemsetAsync(k.cnt, 0, sizeof(int32_t) * (2 * (size_t)nb + 1), st);
   if (e != cudaSuccess) return e;
   const unsigned blocks = (unsigned)((n + 255) / 256);
   // the records in order of arrival: where the forces go later
@@ -821,7 +839,8 @@ cudaError_t brick_sort(erpp_ctx* c, int64_t n, const double* const x[3], cudaStr
   return erpp_launch_pdl(k_brick_order, dim3(blocks), dim3(256), 0, st, 0u, n, nb,
                          (const int32_t*)k.pidx, (const int32_t*)k.pbrick, (const float4*)rec_tmp,
                          (const int32_t*)k.start, k.rec,
-                         k.win, k.slot);
+                         k.win, k.slot, for_adjoint ? k.ord : nullptr, brick_tile(c),
+                         brick_chunk(c), k.nitems, k.items);
 }
 
 cudaError_t brick_forces(erpp_ctx* c, int64_t n, const double* const D[3], float scale,

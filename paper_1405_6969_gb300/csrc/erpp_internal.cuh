@@ -142,6 +142,9 @@ struct erpp_bricks {
   int32_t* pidx;    // [cap] in order of arrival: particle
   int32_t* pbrick;  // [cap] in order of arrival: brick
   int32_t* slot;    // [cap] per particle: place in the order of the records
+  int32_t* ord;     // [cap] in order: particle (sorts for the adjoint)
+  int2* items;      // further chunks of dense adjoint tiles: tile, first record
+  int32_t* nitems;  // their number (after bmax, cleared with it)
   float4* rec;      // [cap] records in order: fractional position, window word
   uint32_t* win;    // [cap] the window words alone
   float4* rec_in;   // [cap] records in input order (scratch of the sort)
@@ -280,11 +283,21 @@ cudaError_t bricks_alloc_tables(erpp_ctx* c);
 void bricks_free_tables(erpp_ctx* c);
 cudaError_t bricks_alloc(erpp_ctx* c, int64_t cap);
 void bricks_free(erpp_ctx* c);
-cudaError_t brick_sort(erpp_ctx* c, int64_t n, const double* const x[3], cudaStream_t st);
+cudaError_t brick_sort(erpp_ctx* c, int64_t n, const double* const x[3], bool for_adjoint,
+                       cudaStream_t st);
 cudaError_t brick_forces(erpp_ctx* c, int64_t n, const double* const D[3], float scale,
                          cudaStream_t st);
 cudaError_t brick_scatter(erpp_ctx* c, float* S, cudaStream_t st);
-
+// launch_adjoint's contractions on an FP32 grid from particles sorted for the
+// adjoint (erpp_bricks_adjoint.cu), bit for bit the same.
+int brick_tile(const erpp_ctx* c);   // bricks of an adjoint tile
+int brick_chunk(const erpp_ctx* c);  // its particles per block
+cudaError_t brick_adjoint(erpp_ctx* c, int64_t n, const double* const x[3], const float* F,
+                          const double* const v[3], double alpha, double shear_coef,
+                          double* const outv[3], double* const outx[3], cudaStream_t st);
+// TMA map (a CUtensorMap) of the FP32 field u for a staged box of box[0] x box[1] x
+// box[2] nodes and 3 components; false where the alignment does not allow it.
+bool field_box_map(const erpp_kparams& kp, const float* u, const int box[3], void* map);
 
 erpp_status derive_ctx(const erpp_params* p, erpp_ctx* c);
 erpp_status ensure_capacity(erpp_ctx* c, int64_t n);  // may allocate (synchronous)

@@ -1443,20 +1443,35 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
 // alignment does not allow it (the kernels then stage with cp.async).
 bool field_tensor_map(const erpp_kparams& kp, const float* u, CUtensorMap* map) {
   const int ny_st = kp.T[1] + kp.yhlo + kp.yhhi;
-  if ((kp.n[0] & 3) || (kp.T[0] & 3) || (kp.xoff & 3) || kp.pxy != kp.px * ny_st ||
-      (((uintptr_t)u) & 15) || kp.px > 256 || ny_st > 256 || kp.T[2] > 256)
+  if ((kp.T[0] & 3) || (kp.xoff & 3) || kp.pxy != kp.px * ny_st) return false;
+  const int box[3] = {kp.px, ny_st, kp.T[2]};
+  return erpp::field_box_map(kp, u, box, map);
+}
+
+}  // namespace
+
+namespace erpp {
+
+bool field_box_map(const erpp_kparams& kp, const float* u, const int box[3], void* map) {
+  if ((kp.n[0] & 3) || (((uintptr_t)u) & 15) || (box[0] & 3) || box[0] > 256 || box[1] > 256 ||
+      box[2] > 256)
     return false;
   PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
   if (!enc) return false;
   const cuuint64_t dims[4] = {(cuuint64_t)kp.n[0], (cuuint64_t)kp.n[1], (cuuint64_t)kp.n[2], 3};
   const cuuint64_t strides[3] = {(cuuint64_t)kp.n[0] * 4, (cuuint64_t)kp.n[0] * kp.n[1] * 4,
                                  (cuuint64_t)kp.n[0] * kp.n[1] * kp.n[2] * 4};
-  const cuuint32_t box[4] = {(cuuint32_t)kp.px, (cuuint32_t)ny_st, (cuuint32_t)kp.T[2], 3};
+  const cuuint32_t ext[4] = {(cuuint32_t)box[0], (cuuint32_t)box[1], (cuuint32_t)box[2], 3};
   const cuuint32_t estr[4] = {1, 1, 1, 1};
-  return enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, const_cast<float*>(u), dims, strides, box,
-             estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  return enc(static_cast<CUtensorMap*>(map), CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4,
+             const_cast<float*>(u), dims, strides, ext, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+             CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
+
+}  // namespace erpp
+
+namespace {
 
 template <int XM, int LMIN, int XW, int NT, bool LAP, int PB>
 cudaError_t gather4_nt(erpp_ctx* ctx, const float* u, cudaStream_t st) {

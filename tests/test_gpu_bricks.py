@@ -168,3 +168,72 @@ def test_gather_of_dense_tiles(erpp, oracle_lib):
     alone = ctx.interpolate(u, cuda(few))
     ctx.check()
     assert torch.equal(alone, up[:, ::60])
+
+
+ADJOINT = ["ragged_90x83x85", "even_96x96x80_raw", "rows_of_odd_length_91x97x81",
+           "thin_x_9x300x170", "one_past_a_region_17x289x81", "shorter_than_a_brick_7x160x257",
+           "windows_of_two_88x88x81", "windows_of_ten_88x90x85", "stretched_81x96x90",
+           "dense_24x20x18", "dense_wide_33x31x30", "one_brick_of_many_16x16x16"]
+
+
+@pytest.mark.parametrize("name", ADJOINT)
+def test_adjoints(erpp, oracle_lib, name):
+    """The adjoints from sorted particles: the bits of the warp-per-particle
+    kernel (which contexts in another halo mode keep) and the oracle's values."""
+    import torch
+    w, opts = CASES[name]
+    p = w.params(**opts)
+    x = positions(w)
+    rng = np.random.default_rng(6)
+    D = rng.standard_normal(x.shape)
+    R = rng.standard_normal((3,) + tuple(w.n)[::-1]).astype(np.float32)
+    got = []
+    for mode in ("merge", "cluster"):
+        ctx = erpp.Context(w.params(), precision="fp32", **opts)
+        ctx.set_scatter_mode(mode)
+        dD, dxs = ctx.scatter_backward(cuda(x), cuda(D), cuda(R, torch.float32))
+        _, dxg = ctx.gather_backward(cuda(x), cuda(R, torch.float32), cuda(D), need_du=False)
+        ctx.check()
+        got.append((dD, dxs, dxg))
+    for a, b in zip(*got):
+        assert torch.equal(a, b)
+    rdD, rdx = oracle_lib.scatter_backward(p, x, D, R.astype(np.float64))
+    assert rel(got[0][0].cpu().numpy(), rdD) < TOL and rel(got[0][1].cpu().numpy(), rdx) < TOL
+    rdx = oracle_lib.gather_backward(p, x, R.astype(np.float64), D)[1]
+    assert rel(got[0][2].cpu().numpy(), rdx) < TOL
+
+
+def test_adjoint_of_invalid_particles(erpp, oracle_lib):
+    """A position outside the box is reported; its gradients are zeros."""
+    w, _ = CASES["ragged_90x83x85"]
+    x = positions(w)
+    x[1, 33] = np.nan
+    D = np.random.default_rng(7).standard_normal(x.shape)
+    R = np.random.default_rng(8).standard_normal((3,) + tuple(w.n)[::-1]).astype(np.float32)
+    import torch
+    ctx = erpp.Context(w.params(), precision="fp32")
+    dD, dx = ctx.scatter_backward(cuda(x), cuda(D), cuda(R, torch.float32))
+    with pytest.raises(erpp.ErppError):
+        ctx.check()
+    assert not dD[:, 33].any() and not dx[:, 33].any()
+    assert dD.isfinite().all() and (dD[:, 34:] != 0).all()
+
+
+def test_adjoint_wait_runs_out(erpp):
+    """The bounded wait for the staged field gives up with a status, and the
+    next call works."""
+    import torch
+    w, _ = CASES["even_96x96x80_raw"]
+    x = positions(w)
+    D = np.ones(x.shape)
+    R = torch.ones((3,) + tuple(w.n)[::-1], dtype=torch.float32, device="cuda")
+    ctx = erpp.Context(w.params(), precision="fp32")
+    ctx.debug_set_wait(limit_ns=2_000_000, stall=True)
+    ctx.scatter_backward(cuda(x), cuda(D), R)
+    with pytest.raises(erpp.ErppError) as ei:
+        ctx.check()
+    assert ei.value.status == 6  # ERPP_ETIMEOUT
+    ctx.debug_set_wait(0, False)
+    dD, _ = ctx.scatter_backward(cuda(x), cuda(D), R)
+    ctx.check()
+    assert dD.isfinite().all()
