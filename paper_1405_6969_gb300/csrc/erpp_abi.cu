@@ -62,6 +62,8 @@ void free_scratch(erpp_ctx* c) {
   cudaFree(c->gather_items);
   c->gather_items = nullptr;
   cudaFree(c->up64);
+  cudaFree(c->w64);
+  c->w64 = nullptr;
   cudaFree(c->w_key);
   cudaFree(c->w_slot);
   cudaFree(c->w_perm);
@@ -100,6 +102,9 @@ erpp_status ensure_capacity(erpp_ctx* c, int64_t n) {
   cudaError_t e = cudaSuccess;
   if (c->fp64 || c->kp.weights != ERPP_W_GAUSS)
     e = cudaMalloc(&c->up64, sizeof(double) * 3 * (size_t)cap);
+  if (c->fp64 && c->kp.weights == ERPP_W_GAUSS && !c->kp.full_force && c->kp.lag == 0 &&
+      e == cudaSuccess)
+    e = cudaMalloc(&c->w64, w64_bytes(c->kp, cap));
   if (c->kp.full_force && e == cudaSuccess) {
     e = cudaMalloc(&c->ff_lap, sizeof(double) * 3 * (size_t)cap);
     if (e == cudaSuccess) e = cudaMalloc(&c->ff_prev, sizeof(double) * 6 * (size_t)cap);
@@ -300,6 +305,8 @@ erpp_status derive_ctx(const erpp_params* p, erpp_ctx* c) {
   for (int a = 0; a < 3; ++a) kp.gravity[a] = p->gravity[a];
   kp.shear_rate = p->shear_rate;
   kp.sig2 = sig2;
+  kp.gauss_hi = -1.0 / (2.0 * sig2);
+  kp.gauss_lo = -fma(kp.gauss_hi, 2.0 * sig2, 1.0) / (2.0 * sig2);
   kp.raw_norm3 = pow(2.0 * kPi * sig2, -1.5);
   kp.lag = (p->flags & ERPP_LAG) ? std::max(1, (int)lround(p->eps_R / p->dt)) : 0;
   kp.full_force = (p->flags & ERPP_FULL_FORCE) ? 1 : 0;
@@ -311,6 +318,7 @@ erpp_status derive_ctx(const erpp_params* p, erpp_ctx* c) {
   // matching kernel's own sigma_R^2 (none for a point-value gather).
   kp.self_s2 = (2.0 * p->nu) * (p->eps_R + p->dt) +
                (kp.weights == ERPP_W_POINT ? 0.0 : (2.0 * p->nu) * p->eps_R);
+  kp.self_inv_2s2 = 1.0 / (2.0 * kp.self_s2);
   kp.self_pref64 = -(p->dt / p->rho_f) / pow(2.0 * kPi * kp.self_s2, 1.5);
   kp.self_pref = (float)kp.self_pref64;
   kp.raw_norm1 = 1.0 / sqrt(2.0 * kPi * sig2);
@@ -563,7 +571,7 @@ erpp_status erpp_interpolate(erpp_ctx* c, const void* u, int64_t n, const double
     e = erpp::sort_by_cell_block(c, n, x, st);
     if (e == cudaSuccess) e = erpp::launch_gather_weights(c, u, n, x, up, st);
   } else if (c->fp64) {
-    e = erpp::launch_gather_f64(c, (const double*)u, n, x, up, st);
+    e = erpp::launch_gather_f64(c, (const double*)u, n, x, up, false, st);
   } else {
     e = erpp::bin_particles(c, n, x, true, st);
     if (e == cudaSuccess) e = erpp::launch_gather_f32(c, (const float*)u, n, st);
@@ -634,7 +642,7 @@ erpp_status erpp_gather_backward(erpp_ctx* c, int64_t n, const double* const x[3
     erpp_status s = erpp::ensure_capacity(c, n);
     if (s) return s;
     if (c->fp64) {
-      e = erpp::launch_scatter_f64(c, n, x, g, c->kp.dV, (double*)du, st);
+      e = erpp::launch_scatter_f64(c, n, x, g, c->kp.dV, (double*)du, false, st);
     } else if (erpp::use_bricks(c, n)) {
       if (!adj) e = erpp::brick_sort(c, n, x, false, st);
       if (e == cudaSuccess) e = erpp::brick_forces(c, n, g, 1.0f, st);
@@ -671,7 +679,7 @@ cudaError_t scatter_source(erpp_ctx* c, int64_t n, const double* const x[3],
     return erpp::launch_scatter_pic(c, n, x, D, -1.0 / c->params.rho_f, S, st);
   }
   if (c->fp64)
-    return erpp::launch_scatter_f64(c, n, x, D, -1.0 / c->params.rho_f, (double*)S, st);
+    return erpp::launch_scatter_f64(c, n, x, D, -1.0 / c->params.rho_f, (double*)S, false, st);
   cudaError_t e;
   if (use_bricks(c, n)) {
     e = brick_sort(c, n, x, false, st);
@@ -724,7 +732,7 @@ erpp_status step_lagged(erpp_ctx* c, const void* u, const erpp_particles* P, voi
   c->launches = 0;
   if (c->fp64) {
     double* up[3] = {c->up64, c->up64 + c->cap, c->up64 + 2 * c->cap};
-    e = erpp::launch_gather_f64(c, (const double*)u, n, xin, up, st);
+    e = erpp::launch_gather_f64(c, (const double*)u, n, xin, up, false, st);
     const double* const upc[3] = {up[0], up[1], up[2]};
     if (e == cudaSuccess)
       e = erpp::launch_advance(c, P, upc, false, false, no_removal, st, remove ? xs : nullptr,
@@ -824,12 +832,12 @@ erpp_status step_device(erpp_ctx* c, const void* u, const erpp_particles* P, voi
     }
   } else if (c->fp64) {
     double* up[3] = {c->up64, c->up64 + c->cap, c->up64 + 2 * c->cap};
-    e = erpp::launch_gather_f64(c, (const double*)u, n, xin, up, st);
+    e = erpp::launch_gather_f64(c, (const double*)u, n, xin, up, true, st);
     const double* const upc[3] = {up[0], up[1], up[2]};
     if (e == cudaSuccess) e = erpp::launch_advance(c, P, upc, false, false, first_step, st);
     if (e == cudaSuccess && after_advance) e = cudaEventRecord(after_advance, st);
     if (e == cudaSuccess)
-      e = erpp::launch_scatter_f64(c, n, xprev, Dv, -1.0 / c->params.rho_f, (double*)S, st);
+      e = erpp::launch_scatter_f64(c, n, xprev, Dv, -1.0 / c->params.rho_f, (double*)S, true, st);
   } else {
     cudaEvent_t* ev = nullptr;
     if (c->prof_on) ev = c->prof_ev + 5 * (c->prof_n++ % kProfSets);

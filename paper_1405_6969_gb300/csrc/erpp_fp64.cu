@@ -1,10 +1,10 @@
 // erpp_fp64.cu -- the plain FP64 form of the gather and the scatter, and the
 // gather of the velocity with its Laplacian for the general force.
 //
-// One warp per particle, particles in index order, no binning: the lanes
-// evaluate the per-axis weights of Sec. 2.4's truncated Gaussian in double
-// precision, then walk the flattened window.  The gather reads the grid from
-// global memory; the scatter adds fscale * D_p W_p(j) (fscale = -1/rho_f for
+// Particles in index order, no binning: a block evaluates the per-axis weights
+// of Sec. 2.4's truncated Gaussian of its particles in double precision, a
+// thread per particle and axis, then a warp walks each particle's window.  The
+// gather reads the grid from global memory; the scatter adds fscale * D_p W_p(j) (fscale = -1/rho_f for
 // the source) into the zeroed grid with FP64 global atomics.  This is the
 // straightforward double-precision implementation the FP32 tile kernels are
 // measured against.
@@ -21,88 +21,188 @@ namespace {
 
 constexpr int kWarps = 8;
 constexpr int kMaxW = 32;
+constexpr int kRowBuf = 64;  // row weights a warp keeps at a time
 
-// Weights of one axis (raw or normalised) into w[0..nw); returns nw (0 on an
-// invalid position).
-__device__ int axis_weights_f64(const erpp_kparams& kp, int a, double x, double* w, int64_t* jlo,
-                                uint32_t* err) {
-  const int lane = threadIdx.x & 31;
+// Weights of one axis of a particle (raw or normalised), one thread: w[0..nw)
+// stored with stride ws, the rest of the xs slots not written; returns nw (0 on
+// an invalid position).
+__device__ int axis_weights_f64(const erpp_kparams& kp, int a, double x, double* w, int ws,
+                                int* jlo, uint32_t* err) {
   if (!(x >= 0.0 && x < kp.L[a])) {
-    if (lane == 0) erpp_set_err(err, ERPP_ERRBIT_RANGE);
+    erpp_set_err(err, ERPP_ERRBIT_RANGE);
     return 0;
   }
-  double s, lo, hi;
-  erpp_axis_window(x, kp.inv_dx[a], kp.cp[a], &s, &lo, &hi);
-  int nw = (int)(hi - lo) + 1;
-  if (nw > kMaxW || nw < 1) {
-    if (lane == 0) erpp_set_err(err, ERPP_ERRBIT_BOUNDS);
+  const erpp_axis_win aw =
+      erpp_axis_window_lean(x, kp.inv_dx[a], kp.cp[a], kp.cp_int[a], kp.cp_frac[a]);
+  const int nw = aw.hi - aw.lo + 1;
+  if (nw > kp.xs || nw < 1) {
+    erpp_set_err(err, ERPP_ERRBIT_BOUNDS);
     return 0;
   }
-  const double raw1 = 1.0 / sqrt(2.0 * 3.141592653589793238462643 * kp.sig2);
-  double wv = 0.0;
-  if (lane < nw) {
-    double d = ((lo + (double)lane) - s) * kp.dx[a];
-    wv = raw1 * exp(-(d * d) / (2.0 * kp.sig2));
+  const double s = __dmul_rn(x, kp.inv_dx[a]);
+  double sum = 0.0;
+  for (int k = 0; k < nw; ++k) {
+    const double d = ((double)(aw.lo + k) - s) * kp.dx[a];
+    const double q = d * d;
+    // -q / (2 sigma_R^2) by the reciprocal's high and low parts
+    const double e = exp(fma(q, kp.gauss_hi, q * kp.gauss_lo));
+    w[k * ws] = e;
+    sum += e;
   }
-  if (kp.normalize) {
-    double sum = wv;
-    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-    wv = wv / (kp.dx[a] * sum);
-  }
-  w[lane] = wv;
-  *jlo = (int64_t)lo;
+  const double scale = kp.normalize ? 1.0 / (kp.dx[a] * sum) : kp.raw_norm1;
+  for (int k = 0; k < nw; ++k) w[k * ws] *= scale;
+  *jlo = aw.lo;
   return nw;
 }
 
-__device__ __forceinline__ int64_t wrap_idx(int64_t j, int64_t n) {
-  int64_t r = j % n;
-  return r < 0 ? r + n : r;
+// Particles of a block of the plain kernels.
+constexpr int kPlainP = 32;
+constexpr int kPlainS = kPlainP + 1;  // stride of a weight's particles
+
+// Doubles that keep a block's weights and windows between the gather and the
+// source of one step.
+__host__ __device__ constexpr size_t kept_doubles(int xs) { return (size_t)3 * (xs + 1) * kPlainP; }
+
+// The weights of a block's particles into shared memory, a thread per particle
+// and axis: w[axis][k][particle], window starts and lengths beside (length 0:
+// invalid).
+__device__ __forceinline__ void plain_weights(const erpp_kparams& kp, int64_t p0, int np,
+                                              const double* __restrict__ x0,
+                                              const double* __restrict__ x1,
+                                              const double* __restrict__ x2, double* w,
+                                              int (*jlo)[kPlainP], int (*nw)[kPlainP],
+                                              const double* __restrict__ kept, uint32_t* err) {
+  if (kept) {
+    // evaluated by the step's gather at the same positions
+    const double* src = kept + (size_t)blockIdx.x * kept_doubles(kp.xs);
+    for (int i = threadIdx.x; i < 3 * kp.xs * kPlainP; i += blockDim.x)
+      w[(i / kPlainP) * kPlainS + (i & (kPlainP - 1))] = src[i];
+    const int2* win = reinterpret_cast<const int2*>(src + 3 * kp.xs * kPlainP);
+    for (int i = threadIdx.x; i < 3 * kPlainP; i += blockDim.x) {
+      const int a = i / kPlainP, p = i & (kPlainP - 1);
+      const int2 v = win[i];
+      jlo[a][p] = v.x;
+      nw[a][p] = v.y;
+    }
+    return;
+  }
+  for (int i = threadIdx.x; i < 3 * kPlainP; i += blockDim.x) {
+    const int a = i / kPlainP, p = i & (kPlainP - 1);
+    if (p >= np) continue;
+    const double x = a == 0 ? x0[p0 + p] : (a == 1 ? x1[p0 + p] : x2[p0 + p]);
+    int lo = 0;
+    nw[a][p] =
+        axis_weights_f64(kp, a, x, w + a * kp.xs * kPlainS + p, kPlainS, &lo, err);
+    jlo[a][p] = lo;
+  }
 }
 
+__device__ __forceinline__ int wrap_idx(int j, int n) {
+  return j < 0 ? j + n : (j >= n ? j - n : j);
+}
+
+// A warp's walk over the window of one particle: lanes (kx, row), nwx lanes a
+// row and 32 / nwx rows at a time; wyz[] holds the products of the rows'
+// weights (written here), f(lane's weight e_x, row weight, node) sees every node
+// of the window once.
+template <typename F>
+__device__ __forceinline__ void plain_walk(const erpp_kparams& kp, const double* w,
+                                           const int (*jlo)[kPlainP], const int (*nw)[kPlainP],
+                                           int p, double* wyz, F f) {
+  const int lane = threadIdx.x & 31;
+  const int nx = nw[0][p], ny = nw[1][p], nz = nw[2][p], rows = ny * nz;
+  const double* wy = w + kp.xs * kPlainS + p;
+  const double* wz = wy + kp.xs * kPlainS;
+  const int R = nx <= 32 ? 32 / nx : 1;
+  const int kx = lane % nx, r0 = lane / nx;
+  const bool on = r0 < R;
+  const double wx = w[kx * kPlainS + p];
+  const int jx = wrap_idx(jlo[0][p] + kx, kp.n[0]);
+  // row products in passes of as many rows as the buffer holds
+  for (int c0 = 0; c0 < rows; c0 += kRowBuf) {
+    const int nr = min(kRowBuf, rows - c0);
+    __syncwarp();
+    for (int r = lane; r < nr; r += 32) {
+      const int z = (c0 + r) / ny, y = (c0 + r) - z * ny;
+      wyz[r] = wy[y * kPlainS] * wz[z * kPlainS];
+    }
+    __syncwarp();
+    int z = (c0 + r0) / ny, y = (c0 + r0) - z * ny;
+    for (int r = r0; r < nr && on; r += R) {
+      const size_t node = ((size_t)wrap_idx(jlo[2][p] + z, kp.n[2]) * kp.n[1] +
+                           (size_t)wrap_idx(jlo[1][p] + y, kp.n[1])) * kp.n[0] + jx;
+      f(wx, wyz[r], node);
+      y += R;
+      while (y >= ny) {
+        y -= ny;
+        ++z;
+      }
+    }
+  }
+}
+
+// A block takes kPlainP particles: their weights first, a thread per particle
+// and axis, then a warp per particle.  The FP64 pipe bounds both kernels (2
+// lanes a clock on an SM, whatever the number of active lanes of an
+// instruction): per particle the exponentials are evaluated once per node and
+// axis instead of by all 32 lanes of a warp, the row weights once per row, and
+// a node costs one operation per component.  100k particles, 216 nodes each, on
+// 128^3: gather 1585 -> 302 us (100 us of it the weights), source 1480 -> 210 us
+// with the weights that the step's gather leaves in w64, 290 us without.
 __global__ void __launch_bounds__(kWarps * 32) k_gather_f64(erpp_kparams kp, int64_t n,
                                                             const double* __restrict__ x0,
                                                             const double* __restrict__ x1,
                                                             const double* __restrict__ x2,
                                                             const double* __restrict__ u,
                                                             double* up0, double* up1, double* up2,
+                                                            double* __restrict__ keep,
                                                             uint32_t* err) {
-  __shared__ double w[kWarps][3][kMaxW];
+  extern __shared__ double plain_smem[];
+  __shared__ int jlo[3][kPlainP], nw[3][kPlainP];
+  double* const w = plain_smem;  // [3][xs][kPlainS]
+  double* const rowbuf = w + 3 * kp.xs * kPlainS;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t p = (int64_t)blockIdx.x * kWarps + warp;
-  if (p >= n) return;
-  const double xv[3] = {x0[p], x1[p], x2[p]};
-  int nw[3];
-  int64_t jlo[3];
-  bool ok = true;
-  for (int a = 0; a < 3; ++a) {
-    nw[a] = axis_weights_f64(kp, a, xv[a], w[warp][a], &jlo[a], err);
-    ok = ok && nw[a] > 0;
+  const int64_t p0 = (int64_t)blockIdx.x * kPlainP;
+  const int np = (int)min((int64_t)kPlainP, n - p0);
+  plain_weights(kp, p0, np, x0, x1, x2, w, jlo, nw, nullptr, err);
+  __syncthreads();
+  if (keep) {
+    double* dst = keep + (size_t)blockIdx.x * kept_doubles(kp.xs);
+    for (int i = threadIdx.x; i < 3 * kp.xs * kPlainP; i += blockDim.x)
+      dst[i] = w[(i / kPlainP) * kPlainS + (i & (kPlainP - 1))];
+    int2* win = reinterpret_cast<int2*>(dst + 3 * kp.xs * kPlainP);
+    for (int i = threadIdx.x; i < 3 * kPlainP; i += blockDim.x)
+      win[i] = make_int2(jlo[i / kPlainP][i & (kPlainP - 1)], nw[i / kPlainP][i & (kPlainP - 1)]);
   }
-  __syncwarp();
-  double acc[3] = {0.0, 0.0, 0.0};
   const size_t nn = (size_t)kp.n[0] * kp.n[1] * kp.n[2];
-  if (ok) {
-    const int total = nw[0] * nw[1] * nw[2];
-    for (int f = lane; f < total; f += 32) {
-      int kx = f % nw[0];
-      int t = f / nw[0];
-      int ky = t % nw[1];
-      int kz = t / nw[1];
-      size_t node = ((size_t)wrap_idx(jlo[2] + kz, kp.n[2]) * kp.n[1] +
-                     (size_t)wrap_idx(jlo[1] + ky, kp.n[1])) * kp.n[0] +
-                    (size_t)wrap_idx(jlo[0] + kx, kp.n[0]);
-      double W = kp.dV * (w[warp][0][kx] * w[warp][1][ky] * w[warp][2][kz]);
-      acc[0] += W * u[node];
-      acc[1] += W * u[nn + node];
-      acc[2] += W * u[2 * nn + node];
+  for (int p = warp; p < np; p += kWarps) {
+    double a0 = 0.0, a1 = 0.0, a2 = 0.0;
+    if (nw[0][p] > 0 && nw[1][p] > 0 && nw[2][p] > 0) {
+      double wx = 0.0;
+      plain_walk(kp, w, jlo, nw, p, rowbuf + warp * kRowBuf,
+                 [&](double wl, double wr, size_t node) {
+                   wx = wl;
+                   a0 = fma(wr, __ldg(u + node), a0);
+                   a1 = fma(wr, __ldg(u + nn + node), a1);
+                   a2 = fma(wr, __ldg(u + 2 * nn + node), a2);
+                 });
+      wx *= kp.dV;
+      a0 *= wx;
+      a1 *= wx;
+      a2 *= wx;
     }
-  }
-  for (int c = 0; c < 3; ++c)
-    for (int o = 16; o > 0; o >>= 1) acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], o);
-  if (lane == 0) {
-    up0[p] = acc[0] + kp.shear_rate * xv[1];
-    up1[p] = acc[1];
-    up2[p] = acc[2];
+    // sums over the lanes: two values change hands, then one
+    const bool h16 = lane & 16, h8 = lane & 8;
+    const double s0 = (h16 ? a2 : a0) + __shfl_xor_sync(0xffffffffu, h16 ? a0 : a2, 16);
+    const double b1 = __shfl_xor_sync(0xffffffffu, a1, 16);
+    const double s1 = a1 + b1;  // in both halves
+    // lanes below 16: s0 = component 0; above: component 2; s1 everywhere
+    double v = (h8 ? s1 : s0) + __shfl_xor_sync(0xffffffffu, h8 ? s0 : s1, 8);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane == 0) up0[p0 + p] = v + kp.shear_rate * x1[p0 + p];
+    if (lane == 8) up1[p0 + p] = v;
+    if (lane == 16) up2[p0 + p] = v;
   }
 }
 
@@ -114,37 +214,33 @@ __global__ void __launch_bounds__(kWarps * 32) k_scatter_f64(erpp_kparams kp, in
                                                              const double* __restrict__ D1,
                                                              const double* __restrict__ D2,
                                                              double fscale, double* S,
+                                                             const double* __restrict__ kept,
                                                              uint32_t* err) {
-  __shared__ double w[kWarps][3][kMaxW];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t p = (int64_t)blockIdx.x * kWarps + warp;
-  if (p >= n) return;
-  const double xv[3] = {x0[p], x1[p], x2[p]};
-  int nw[3];
-  int64_t jlo[3];
-  bool ok = true;
-  for (int a = 0; a < 3; ++a) {
-    nw[a] = axis_weights_f64(kp, a, xv[a], w[warp][a], &jlo[a], err);
-    ok = ok && nw[a] > 0;
-  }
-  __syncwarp();
-  if (!ok) return;
-  const double f[3] = {fscale * D0[p], fscale * D1[p], fscale * D2[p]};
+  extern __shared__ double plain_smem[];
+  __shared__ int jlo[3][kPlainP], nw[3][kPlainP];
+  double* const w = plain_smem;  // [3][xs][kPlainS]
+  double* const rowbuf = w + 3 * kp.xs * kPlainS;
+  const int warp = threadIdx.x >> 5;
+  const int64_t p0 = (int64_t)blockIdx.x * kPlainP;
+  const int np = (int)min((int64_t)kPlainP, n - p0);
+  plain_weights(kp, p0, np, x0, x1, x2, w, jlo, nw, kept, err);
+  __syncthreads();
   const size_t nn = (size_t)kp.n[0] * kp.n[1] * kp.n[2];
-  const int total = nw[0] * nw[1] * nw[2];
-  for (int fi = lane; fi < total; fi += 32) {
-    int kx = fi % nw[0];
-    int t = fi / nw[0];
-    int ky = t % nw[1];
-    int kz = t / nw[1];
-    size_t node = ((size_t)wrap_idx(jlo[2] + kz, kp.n[2]) * kp.n[1] +
-                   (size_t)wrap_idx(jlo[1] + ky, kp.n[1])) * kp.n[0] +
-                  (size_t)wrap_idx(jlo[0] + kx, kp.n[0]);
-    double W = w[warp][0][kx] * w[warp][1][ky] * w[warp][2][kz];
-    atomicAdd(S + node, f[0] * W);
-    atomicAdd(S + nn + node, f[1] * W);
-    atomicAdd(S + 2 * nn + node, f[2] * W);
+  for (int p = warp; p < np; p += kWarps) {
+    if (!(nw[0][p] > 0 && nw[1][p] > 0 && nw[2][p] > 0)) continue;
+    const double wl = w[((threadIdx.x & 31) % nw[0][p]) * kPlainS + p];
+    const double f0 = fscale * D0[p0 + p] * wl, f1 = fscale * D1[p0 + p] * wl,
+                 f2 = fscale * D2[p0 + p] * wl;
+    plain_walk(kp, w, jlo, nw, p, rowbuf + warp * kRowBuf, [&](double, double wr, size_t node) {
+      atomicAdd(S + node, f0 * wr);
+      atomicAdd(S + nn + node, f1 * wr);
+      atomicAdd(S + 2 * nn + node, f2 * wr);
+    });
   }
+}
+
+size_t plain_smem_bytes(const erpp_kparams& kp) {
+  return sizeof(double) * ((size_t)3 * kp.xs * kPlainS + (size_t)kWarps * kRowBuf);
 }
 
 // Weights of one axis and their second derivatives in the particle
@@ -442,27 +538,32 @@ cudaError_t launch_gather_faxen(erpp_ctx* ctx, const void* u, int64_t n,
 }
 
 cudaError_t launch_gather_f64(erpp_ctx* ctx, const double* u, int64_t n,
-                              const double* const x[3], double* const up[3], cudaStream_t st) {
+                              const double* const x[3], double* const up[3], bool keep,
+                              cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  int blocks = (int)((n + kWarps - 1) / kWarps);
+  const unsigned blocks = (unsigned)((n + kPlainP - 1) / kPlainP);
   ++ctx->launches;
-  k_gather_f64<<<blocks, kWarps * 32, 0, st>>>(ctx->kp, n, x[0], x[1], x[2], u, up[0], up[1],
-                                               up[2], ctx->err);
+  k_gather_f64<<<blocks, kWarps * 32, plain_smem_bytes(ctx->kp), st>>>(
+      ctx->kp, n, x[0], x[1], x[2], u, up[0], up[1], up[2], keep ? ctx->w64 : nullptr, ctx->err);
   return cudaGetLastError();
 }
 
+size_t w64_bytes(const erpp_kparams& kp, int64_t cap) {
+  return sizeof(double) * kept_doubles(kp.xs) * (size_t)((cap + kPlainP - 1) / kPlainP);
+}
+
 cudaError_t launch_scatter_f64(erpp_ctx* ctx, int64_t n, const double* const x[3],
-                               const double* const D[3], double fscale, double* S,
+                               const double* const D[3], double fscale, double* S, bool kept,
                                cudaStream_t st) {
   const erpp_kparams& kp = ctx->kp;
   size_t nn = (size_t)kp.n[0] * kp.n[1] * kp.n[2];
   cudaError_t e = cudaMemsetAsync(S, 0, sizeof(double) * 3 * nn, st);
   if (e != cudaSuccess) return e;
   if (n <= 0) return cudaSuccess;
-  int blocks = (int)((n + kWarps - 1) / kWarps);
+  const unsigned blocks = (unsigned)((n + kPlainP - 1) / kPlainP);
   ++ctx->launches;
-  k_scatter_f64<<<blocks, kWarps * 32, 0, st>>>(kp, n, x[0], x[1], x[2], D[0], D[1], D[2],
-                                                fscale, S, ctx->err);
+  k_scatter_f64<<<blocks, kWarps * 32, plain_smem_bytes(kp), st>>>(
+      kp, n, x[0], x[1], x[2], D[0], D[1], D[2], fscale, S, kept ? ctx->w64 : nullptr, ctx->err);
   return cudaGetLastError();
 }
 

@@ -107,7 +107,9 @@ struct erpp_kparams {
   double self_pref64;// -(dt/rho_f) (2 pi self_s2)^(-3/2)
   double basset_c;   // 12 mu sqrt(pi / (nu dt)) (ERPP_FULL_FORCE; 0 when dt = 0)
   double sig2;       // sigma_R^2
+  double gauss_hi, gauss_lo; // -1 / (2 sigma_R^2), rounded, and the rest
   double self_s2;    // variance of the self disturbance as gathered
+  double self_inv_2s2;  // 1 / (2 self_s2)
   float beta[3];     // log2(e) dx_a^2 / (2 sigma_R^2)
   float inv_rho_dV;  // 1 / (rho_f dV)
   float self_pref;   // -(dt/rho_f) (2 pi s2)^(-3/2)
@@ -181,6 +183,7 @@ struct erpp_ctx {
   float4* up_part;        // [entries_cap] x/y-halo tiles: each piece's gathered sums,
                           // at its place in the piece records
   float4* fscat;
+  double* w64;            // FP64 step: the gather's weights, for the source
   double* up64;           // FP64 mode or other weights: gathered velocity [3][cap]
   int32_t* w_key;         // other weights: sort key, place and order of each particle [cap]
   int32_t* w_slot;
@@ -367,10 +370,12 @@ cudaError_t launch_advance_full(erpp_ctx* ctx, const erpp_particles* P,
 cudaError_t launch_lag_store(erpp_ctx* ctx, int64_t n, const double* const x[3],
                              const double* const D[3], double* slot, cudaStream_t st);
 cudaError_t launch_gather_f64(erpp_ctx* ctx, const double* u, int64_t n,
-                              const double* const x[3], double* const up[3], cudaStream_t st);
+                              const double* const x[3], double* const up[3], bool keep,
+                              cudaStream_t st);  // keep: leave the weights in w64
 cudaError_t launch_scatter_f64(erpp_ctx* ctx, int64_t n, const double* const x[3],
-                               const double* const D[3], double fscale, double* S,
-                               cudaStream_t st);
+                               const double* const D[3], double fscale, double* S, bool kept,
+                               cudaStream_t st);  // kept: w64 holds the weights at x
+size_t w64_bytes(const erpp_kparams& kp, int64_t cap);
 // Per particle: outv = alpha sum_j F_j W (if outv), outx = alpha sum_j (F_j . v)
 // dW/dx + shear_coef v_x on y.
 cudaError_t launch_adjoint(erpp_ctx* ctx, int64_t n, const double* const x[3], const void* F,

@@ -77,33 +77,42 @@ __device__ void self_velocity_f32(const erpp_kparams& kp, const float r[3], cons
   for (int a = 0; a < 3; ++a) out[a] = kp.self_pref * (c1 * D[a] - c2 * rh[a]);
 }
 
+// F(eta) below eta = 1/2 in FP64: sum_k (-1)^k (eta^2)^k / (k! (2k + 3)) by
+// Horner's rule (fourteen terms: the first left out is below 2^-60 of the sum).
+// The coefficients are constants: evaluated term by term with FP64 divisions,
+// whose pipe is narrow, the sum took most of the FP64 advance (100 us for 100k
+// particles).
+__device__ __forceinline__ double self_series(double e2) {
+  double sum = 0.0;
+#pragma unroll
+  for (int k = 13; k >= 0; --k) {
+    double fact = 1.0;
+#pragma unroll
+    for (int j = 2; j <= k; ++j) fact *= (double)j;
+    sum = fma(sum, e2, (k & 1 ? -1.0 : 1.0) / (fact * (double)(2 * k + 3)));
+  }
+  return sum;
+}
+
 __device__ void self_velocity_f64(const erpp_kparams& kp, const double r[3], const double D[3],
                                   double out[3]) {
   const double pi = 3.141592653589793238462643;
-  double s2 = kp.self_s2;
-  double pref = kp.self_pref64;
-  double rr = sqrt(r[0] * r[0] + r[1] * r[1] + r[2] * r[2]);
-  double eta = rr / sqrt(2.0 * s2);
+  const double r2 = r[0] * r[0] + r[1] * r[1] + r[2] * r[2];
+  const double e2 = r2 * kp.self_inv_2s2;  // eta^2
+  const double e = exp(-e2);
   double F;
-  if (eta < 0.5) {
-    double e2 = eta * eta, term = 1.0, sum = 0.0;
-    for (int k = 0; k < 20; ++k) {
-      sum += term / (double)(2 * k + 3);
-      term = -term * e2 / (double)(k + 1);
-    }
-    F = sum;
+  if (e2 < 0.25) {
+    F = self_series(e2);
   } else {
-    double f = 0.5 * sqrt(pi) * erf(eta) - eta * exp(-eta * eta);
-    F = f / (2.0 * eta * eta * eta);
+    const double eta = sqrt(e2);
+    F = (0.5 * sqrt(pi) * erf(eta) - eta * e) / (2.0 * eta * e2);
   }
-  double e = exp(-eta * eta);
-  double rh[3] = {0.0, 0.0, 0.0};
-  double Ddr = 0.0;
-  if (rr > 0.0) {
-    for (int a = 0; a < 3; ++a) rh[a] = r[a] / rr;
-    Ddr = D[0] * rh[0] + D[1] * rh[1] + D[2] * rh[2];
-  }
-  for (int a = 0; a < 3; ++a) out[a] = pref * ((e - F) * D[a] - Ddr * (e - 3.0 * F) * rh[a]);
+  // (D . rh) rh = (D . r) r / r^2
+  const double c2 =
+      r2 > 0.0 ? (D[0] * r[0] + D[1] * r[1] + D[2] * r[2]) * (e - 3.0 * F) / r2 : 0.0;
+  const double pref = kp.self_pref64, c1 = e - F;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) out[a] = pref * (c1 * D[a] - c2 * r[a]);
 }
 
 // Laplacian in r of the disturbance above: the disturbance is the Leray
@@ -369,14 +378,15 @@ __device__ __forceinline__ void advance_one(const erpp_kparams& kp, int64_t i, c
     }
   } else {
     const double k_drag = 6.0 * pi * kp.mu * a_p;
-    const double m_p = (4.0 / 3.0) * pi * a_p * a_p * a_p * rho;
+    // divisions are slow on this part: one each for 1 / m_p and rho_f / rho_p
+    const double inv_m = 1.0 / ((4.0 / 3.0) * pi * a_p * a_p * a_p * rho);
     const double buoy = 1.0 - kp.rho_f / rho;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
       Dnf[a] = 0.f;
       double ut = up[a] - vs[a];
       Dn[a] = k_drag * (ut - v[a]);
-      P.v[a][i] = v[a] + kp.dt * (Dn[a] / m_p + buoy * kp.gravity[a]);
+      P.v[a][i] = v[a] + kp.dt * (Dn[a] * inv_m + buoy * kp.gravity[a]);
       P.x[a][i] = wrap_coord(x[a] + kp.dt * v[a], kp.L[a]);
       P.xp[a][i] = x[a];
       P.D[a][i] = Dn[a];
