@@ -174,6 +174,40 @@ __global__ void __launch_bounds__(256) k_brick_place(int64_t n, const int2* __re
   pbrick[pos] = k.x;
 }
 
+// A brick is dense that holds this many particles and more than an eighth of an
+// SM's share of all n: its regions take so long that the others are done before.
+// Uniform clouds of about 200 per brick, one source by whole regions and by
+// quarters: 64^3 292 and 198 us, 72^3 343 and 295, 80^3 356 and 341; where every
+// SM has its regions anyway 96^3 378 and 485, 128^3 565 and 848 us.
+constexpr int kDenseBrick = 192;
+__device__ __forceinline__ bool dense_brick(int members, int64_t n) {
+  return members >= kDenseBrick && members > n / (8 * 152);
+}
+// Lists the regions that the members of a dense brick can reach, each once.
+__device__ __noinline__ void mark_dense(const erpp_kparams& kp, const erpp_brick_dims& bd, int id,
+                                        int32_t* ndense, int32_t* dense, int32_t* dflag) {
+  int g = id >> 3;
+  const int br[3] = {2 * (g % bd.ng[0]) + (id & 1), 2 * ((g / bd.ng[0]) % bd.ng[1]) + ((id >> 1) & 1),
+                     2 * (g / (bd.ng[0] * bd.ng[1])) + ((id >> 2) & 1)};
+  int lst[3][4], cnt[3];
+  for (int a = 0; a < 3; ++a) {
+    const int n = kp.n[a], last = min(8 * br[a] + 8, n) + kp.hlo;
+    int k = 0;
+    for (int j = 8 * br[a] - kp.hlo; j <= last && k < 4;) {
+      const int w = j - erpp_floordiv(j, n) * n;
+      lst[a][k++] = w >> 4;
+      j += min(((w >> 4) + 1) * 16, n) - w;
+    }
+    cnt[a] = k;
+  }
+  for (int z = 0; z < cnt[2]; ++z)
+    for (int y = 0; y < cnt[1]; ++y)
+      for (int x = 0; x < cnt[0]; ++x) {
+        g = (lst[2][z] * bd.ng[1] + lst[1][y]) * bd.ng[0] + lst[0][x];
+        if (atomicExch(&dflag[g], 1) == 0) dense[atomicAdd(ndense, 1)] = g;
+      }
+}
+
 // Position j's particle moves to its rank (by index) among its brick's members.
 // The threads of a warp mostly share a brick, so its indices are read as
 // broadcasts, 16 bytes at a time (a dense cluster's bricks hold a thousand
@@ -188,7 +222,11 @@ __global__ void __launch_bounds__(256) k_brick_order(int64_t n, int nb,
                                                      int32_t* __restrict__ slot,
                                                      int32_t* __restrict__ ord, int tile_bricks,
                                                      int chunk, int32_t* __restrict__ nitems,
-                                                     int2* __restrict__ items) {
+                                                     int2* __restrict__ items,
+                                                     erpp_kparams kp, erpp_brick_dims bd,
+                                                     int32_t* __restrict__ ndense,
+                                                     int32_t* __restrict__ dense,
+                                                     int32_t* __restrict__ dflag) {
   erpp_pdl_enter();
   const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= n || j >= start[nb]) return;
@@ -212,6 +250,7 @@ __global__ void __launch_bounds__(256) k_brick_order(int64_t n, int nb,
   rec[s + r] = v;
   win[s + r] = __float_as_uint(v.w);
   slot[me] = s + r;
+  if (r == 0 && dense_brick(e - s, n)) mark_dense(kp, bd, b, ndense, dense, dflag);
   if (ord) {
     ord[s + r] = me;
     // the further chunks of an adjoint tile of more than `chunk` particles
@@ -292,11 +331,38 @@ __device__ __forceinline__ void ldmatrix_x4_trans(uint32_t (&r)[4], unsigned add
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                : "r"(addr));
 }
+// A pair of FP32 values in one register pair: one instruction works on both,
+// each rounded as by itself.
+struct Pair {
+  unsigned long long v;
+};
+__device__ __forceinline__ Pair pair_of(float a, float b) {
+  Pair p;
+  asm("mov.b64 %0, {%1, %2};\n" : "=l"(p.v) : "f"(a), "f"(b));
+  return p;
+}
+__device__ __forceinline__ float2 parts(Pair p) {
+  float2 f;
+  asm("mov.b64 {%0, %1}, %2;\n" : "=f"(f.x), "=f"(f.y) : "l"(p.v));
+  return f;
+}
+__device__ __forceinline__ Pair operator+(Pair a, Pair b) {
+  Pair p;
+  asm("add.rn.f32x2 %0, %1, %2;\n" : "=l"(p.v) : "l"(a.v), "l"(b.v));
+  return p;
+}
+__device__ __forceinline__ Pair operator*(Pair a, Pair b) {
+  Pair p;
+  asm("mul.rn.f32x2 %0, %1, %2;\n" : "=l"(p.v) : "l"(a.v), "l"(b.v));
+  return p;
+}
 // v = h + l in FP16 for a pair of values.
-__device__ __forceinline__ void split_pair(float v0, float v1, uint32_t& h, uint32_t& l) {
-  const __half2 hh = __floats2half2_rn(v0, v1);
+__device__ __forceinline__ void split_pair(Pair v, uint32_t& h, uint32_t& l) {
+  const float2 f = parts(v);
+  const __half2 hh = __floats2half2_rn(f.x, f.y);
   const float2 hf = __half22float2(hh);
-  const __half2 ll = __floats2half2_rn(v0 - hf.x, v1 - hf.y);
+  const float2 rest = parts(v + pair_of(-hf.x, -hf.y));
+  const __half2 ll = __floats2half2_rn(rest.x, rest.y);
   h = *reinterpret_cast<const uint32_t*>(&hh);
   l = *reinterpret_cast<const uint32_t*>(&ll);
 }
@@ -304,8 +370,46 @@ __device__ __forceinline__ void split_pair(float v0, float v1, uint32_t& h, uint
 struct ScatShared {
   int cnt[kScatWarps];  // members each warp found that touch the region
   int maxbits;          // largest |force component| of the bricks around
-  int pre[kMaxSegs + 1];// dense regions: touching members before each segment
 };
+
+// Dense regions: the segments one after the other as one range of candidates,
+// and how many of the candidates before every G-th touch the region.  In the
+// last rows' place (dense batches are shorter).
+constexpr int kDenseBatch = 272;
+constexpr int kMarks = 512;
+struct DenseTab {
+  int start[kMaxSegs];   // first record of the segment's brick, less the candidates before
+  uint32_t org[kMaxSegs];
+  int pre[kMaxSegs + 1]; // candidates before the segment
+  int mark[kMarks + 1];
+};
+static_assert(sizeof(DenseTab) <= (kListBatch - kDenseBatch) * kPitch, "dense table");
+
+// Largest k in [0, n) with v[k] <= x (v ascending, v[0] <= x).
+__device__ __forceinline__ int last_not_above(const int* v, int n, int x) {
+  int lo = 0, hi = n;
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) >> 1;
+    if (v[mid] <= x) lo = mid; else hi = mid;
+  }
+  return lo;
+}
+// Exclusive scan of v[0..n) in place by one warp, total at v[n].
+__device__ __forceinline__ void warp_scan(int* v, int n, int lane) {
+  int carry = 0;
+  for (int q0 = 0; q0 < n; q0 += 32) {
+    const int x = q0 + lane < n ? v[q0 + lane] : 0;
+    int incl = x;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int u = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += u;
+    }
+    if (q0 + lane < n) v[q0 + lane] = carry + incl - x;
+    carry += __shfl_sync(0xffffffffu, incl, 31);
+  }
+  if (lane == 0) v[n] = carry;
+}
 
 // A particle's window relative to a region, all axes at once in the bytes of
 // a word: first node + 64.
@@ -327,29 +431,32 @@ __device__ __forceinline__ bool touches(uint32_t w, uint32_t org, uint32_t ext1)
 // cells of the particles reaching the group's nodes (brick, first cell
 // relative to the group); the last entry of the eight holds their number and
 // 65536 / number, rounded up.
-template <int LP>
-__global__ void __launch_bounds__(kScatThreads, 2) k_brick_scatter(
-    erpp_kparams kp, erpp_brick_dims bd, const int2* __restrict__ axis,
-    const float4* __restrict__ rec, const uint32_t* __restrict__ win,
-    const float4* __restrict__ fs, const int32_t* __restrict__ bstart,
-    const int32_t* __restrict__ bmax, float* __restrict__ S) {
-  extern __shared__ __align__(128) unsigned char smem[];
-  __shared__ ScatShared sh;
+// ZS: planes of the region, 16, or 4 (planes z0 ..) of a dense one: there the
+// block's four output tiles of 2 planes x 8 rows take four warps each, which
+// share the tile's particles chunk by chunk and add their sums in order.
+template <int LP, int ZS>
+__device__ __forceinline__ void scatter_region(
+    const erpp_kparams& kp, const erpp_brick_dims& bd, const int gg[3], int z0,
+    const int2* __restrict__ axis, const float4* __restrict__ rec,
+    const uint32_t* __restrict__ win, const float4* __restrict__ fs,
+    const int32_t* __restrict__ bstart, const int32_t* __restrict__ bmax,
+    const int32_t* __restrict__ skip, float* __restrict__ S, unsigned char* smem,
+    ScatShared& sh) {
+  constexpr int kTiles = ZS, kParts = kScatWarps / kTiles;  // 2 x 8-row tiles; warps of each
   unsigned char* const row0 = smem;  // [kListBatch + 1][kPitch]
   uint32_t* const mask = reinterpret_cast<uint32_t*>(row0 + (kListBatch + 1) * kPitch);
   uint16_t* const wl = reinterpret_cast<uint16_t*>(mask + kListBatch);  // [warps][batch + 16]
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int b[3] = {(int)blockIdx.x * kRegion, (int)blockIdx.y * kRegion,
-                    (int)blockIdx.z * kRegion};
-  int ext[3];
-#pragma unroll
-  for (int a = 0; a < 3; ++a) ext[a] = min(kRegion, kp.n[a] - b[a]);
+  const int skipped = skip ? __ldg(skip) : 0;  // looked at after the segments' loads
+  const int b[3] = {gg[0] * kRegion, gg[1] * kRegion, gg[2] * kRegion + z0};
+  const int ext[3] = {min(kRegion, kp.n[0] - b[0]), min(kRegion, kp.n[1] - b[1]),
+                      min(ZS, kp.n[2] - b[2])};
   const uint32_t ext1 = 0x808080u | (uint32_t)(63 + ext[0]) | (uint32_t)(63 + ext[1]) << 8 |
                         (uint32_t)(63 + ext[2]) << 16;
-  const int2* axx = axis + (size_t)blockIdx.x * kMaxAxisSegs;
-  const int2* axy = axis + (size_t)(bd.ng[0] + blockIdx.y) * kMaxAxisSegs;
-  const int2* axz = axis + (size_t)(bd.ng[0] + bd.ng[1] + blockIdx.z) * kMaxAxisSegs;
+  const int2* axx = axis + (size_t)gg[0] * kMaxAxisSegs;
+  const int2* axy = axis + (size_t)(bd.ng[0] + gg[1]) * kMaxAxisSegs;
+  const int2* axz = axis + (size_t)(bd.ng[0] + bd.ng[1] + gg[2]) * kMaxAxisSegs;
   const int2 nsx = axx[kMaxAxisSegs - 1], nsy = axy[kMaxAxisSegs - 1],
              nsz = axz[kMaxAxisSegs - 1];
   const int ns = min(nsx.x * nsy.x * nsz.x, kMaxSegs);
@@ -366,7 +473,7 @@ __global__ void __launch_bounds__(kScatThreads, 2) k_brick_scatter(
     const int id = brick_id(bd.ng, ex_.x, ey_.x, ez_.x);
     start = bstart[id];
     count = bstart[id + 1] - start;
-    org = (uint32_t)(ex_.y + 56) | (uint32_t)(ey_.y + 56) << 8 | (uint32_t)(ez_.y + 56) << 16;
+    org = (uint32_t)(ex_.y + 56) | (uint32_t)(ey_.y + 56) << 8 | (uint32_t)(ez_.y + 56 - z0) << 16;
     return bmax[id];
   };
   // Lane k describes the warp's k-th segment (the warps take turns, shifted
@@ -375,6 +482,7 @@ __global__ void __launch_bounds__(kScatThreads, 2) k_brick_scatter(
   uint32_t seg_o = 0u;
   const int myq = lane * kScatWarps + ((warp + 5 * lane) & (kScatWarps - 1));
   if (lane < K && myq < ns) mx = describe(myq, seg_s, seg_c, seg_o);
+  if (skipped) return;
   uint16_t* const mylist = wl + warp * (kListBatch + 16);
   uint2* const queue = reinterpret_cast<uint2*>(mylist);  // until the warp's list is made
 
@@ -436,36 +544,48 @@ __global__ void __launch_bounds__(kScatThreads, 2) k_brick_scatter(
     at0 = __shfl_sync(0xffffffffu, incl - v, warp);
     dense = total > kListBatch || __any_sync(0xffffffffu, v > kQueue);
   }
+  DenseTab& tab = *reinterpret_cast<DenseTab*>(row0 + kDenseBatch * kPitch);
+  int marks = 0, G = 32;
+  // candidate idx of the range: its record, whether it touches, its window
+  auto candidate = [&](int idx, int& j, uint32_t& lo) {
+    if (idx >= tab.pre[ns]) return false;
+    const int q = last_not_above(tab.pre, ns, idx);
+    j = tab.start[q] + idx;
+    const uint32_t w = __ldg(&win[j]), o = tab.org[q];
+    lo = window_lo(w, o);
+    return touches(w, o, ext1);
+  };
   if (dense) {
     // more than one batch, or more than a warp can queue: the list is instead
-    // in segment order, and every warp stages an equal share of each batch
-    for (int k = 0; k < K; ++k) {
-      const int s0 = __shfl_sync(0xffffffffu, seg_s, k), c = __shfl_sync(0xffffffffu, seg_c, k);
-      const uint32_t o = __shfl_sync(0xffffffffu, seg_o, k);
-      const int q = __shfl_sync(0xffffffffu, myq, k);
-      int m = 0;
-      for (int m0 = 0; m0 < c; m0 += 32) {
-        const bool t = m0 + lane < c && touches(__ldg(&win[s0 + m0 + lane]), o, ext1);
-        m += __popc(__ballot_sync(0xffffffffu, t));
-      }
-      if (lane == 0 && q < ns) sh.pre[q] = m;
+    // in segment order, and every warp stages an equal share of each batch,
+    // which it finds from the marks
+    for (int q = tid; q < ns; q += kScatThreads) {
+      int st, c;
+      uint32_t o;
+      describe(q, st, c, o);
+      tab.start[q] = st;
+      tab.org[q] = o;
+      tab.pre[q] = c;
     }
     __syncthreads();
-    if (warp == 0) {
-      int carry = 0;
-      for (int q0 = 0; q0 < ns; q0 += 32) {
-        const int v = q0 + lane < ns ? sh.pre[q0 + lane] : 0;
-        int incl = v;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const int u = __shfl_up_sync(0xffffffffu, incl, o);
-          if (lane >= o) incl += u;
-        }
-        if (q0 + lane < ns) sh.pre[q0 + lane] = carry + incl - v;
-        carry += __shfl_sync(0xffffffffu, incl, 31);
+    if (warp == 0) warp_scan(tab.pre, ns, lane);
+    __syncthreads();
+    for (int q = tid; q < ns; q += kScatThreads) tab.start[q] -= tab.pre[q];
+    const int C = tab.pre[ns];
+    G = 32 * ((C + 32 * kMarks - 1) / (32 * kMarks));
+    marks = (C + G - 1) / G;
+    __syncthreads();
+    for (int k = warp; k < marks; k += kScatWarps) {
+      int m = 0;
+      for (int i = 0; i < G; i += 32) {
+        int j;
+        uint32_t lo;
+        m += __popc(__ballot_sync(0xffffffffu, candidate(k * G + i + lane, j, lo)));
       }
-      if (lane == 0) sh.pre[ns] = carry;
+      if (lane == 0) tab.mark[k] = m;
     }
+    __syncthreads();
+    if (warp == 0) warp_scan(tab.mark, marks, lane);
     __syncthreads();
   }
 
@@ -477,18 +597,20 @@ __global__ void __launch_bounds__(kScatThreads, 2) k_brick_scatter(
   ex = max(ex, -100);
   const float sB = ldexpf(1.f, 14 - ex);
 
-  const int zp = warp & 7, yh = warp >> 3;  // planes 2 zp, 2 zp + 1; rows 8 yh ..
+  const int tile = warp % kTiles, part = warp / kTiles;
+  const int zp = tile % (ZS / 2), yh = tile / (ZS / 2);  // planes 2 zp, 2 zp + 1; rows 8 yh ..
   const int gr = lane >> 2, tq = lane & 3;
-  float acc[3][2][4];
+  Pair acc[3][2][2];
 #pragma unroll
   for (int c = 0; c < 3; ++c)
 #pragma unroll
     for (int h = 0; h < 2; ++h)
 #pragma unroll
-      for (int k = 0; k < 4; ++k) acc[c][h][k] = 0.f;
+      for (int k = 0; k < 2; ++k) acc[c][h][k].v = 0ull;
 
   // batches of equal size, so that none leaves the warps a nearly empty chunk
-  const int nbatch = (total + kListBatch - 1) / kListBatch;
+  const int most = dense ? kDenseBatch : kListBatch;
+  const int nbatch = (total + most - 1) / most;
   const int bsize = nbatch > 0 ? (total + nbatch - 1) / nbatch : 1;
 
   // Stages the queue's nq members as rows p0, p0 + 1, ...: LP lanes a particle,
@@ -523,16 +645,17 @@ __global__ void __launch_bounds__(kScatThreads, 2) k_brick_scatter(
         const int q = at[a] - lo[a];  // -1 at the least
         const int nw = erpp_rec_nw(w, a);
         const float k = (float)(erpp_rec_off(kp, w, a) + q);
-        const float d = k - t[a], dn = (k + 1.f) - t[a];
-        v[a][0] = q >= 0 && q < nw ? erpp_ex2(-kp.beta[a] * d * d) : 0.f;
-        v[a][1] = q + 1 < nw ? erpp_ex2(-kp.beta[a] * dn * dn) : 0.f;
+        const Pair d = pair_of(k, k + 1.f) + pair_of(-t[a], -t[a]);
+        const float2 e2 = parts(pair_of(-kp.beta[a], -kp.beta[a]) * d * d);
+        v[a][0] = q >= 0 && q < nw ? erpp_ex2(e2.x) : 0.f;
+        v[a][1] = q + 1 < nw ? erpp_ex2(e2.y) : 0.f;
         in[a] = live && q < nw && (unsigned)at[a] < 16u;
       }
-      const float x0 = v[0][0] * sB, x1 = v[0][1] * sB;
+      const Pair x01 = pair_of(v[0][0], v[0][1]) * pair_of(sB, sB);
       uint32_t h[3], l[3];
-      split_pair(f.x * x0, f.x * x1, h[0], l[0]);
-      split_pair(f.y * x0, f.y * x1, h[1], l[1]);
-      split_pair(f.z * x0, f.z * x1, h[2], l[2]);
+      split_pair(pair_of(f.x, f.x) * x01, h[0], l[0]);
+      split_pair(pair_of(f.y, f.y) * x01, h[1], l[1]);
+      split_pair(pair_of(f.z, f.z) * x01, h[2], l[2]);
       if (in[0]) {
         uint32_t* col = reinterpret_cast<uint32_t*>(row + 2 * at[0]);
 #pragma unroll
@@ -547,11 +670,11 @@ __global__ void __launch_bounds__(kScatThreads, 2) k_brick_scatter(
             make_float2(v[1][0] * 16384.f, v[1][1] * 16384.f);
       if (in[2]) *reinterpret_cast<float2*>(wt + 16 + at[2]) = make_float2(v[2][0], v[2][1]);
       if (live && ql == 0) {
-        // the warps whose rows and planes the window reaches: bit 8 yh + zp
+        // the tiles whose rows and planes the window reaches: bit ZS / 2 yh + zp
         const int y1 = lo[1] + erpp_rec_nw(w, 1) - 1;
-        const int za = max(lo[2], 0) >> 1, zb = min(lo[2] + erpp_rec_nw(w, 2) - 1, 15) >> 1;
+        const int za = max(lo[2], 0) >> 1, zb = min(lo[2] + erpp_rec_nw(w, 2) - 1, ZS - 1) >> 1;
         const uint32_t zm = (2u << zb) - (1u << za);
-        mask[p0 + i] = (lo[1] < 8 ? zm : 0u) | (y1 >= 8 ? zm << 8 : 0u);
+        mask[p0 + i] = (lo[1] < 8 ? zm : 0u) | (y1 >= 8 ? zm << (ZS / 2) : 0u);
       }
     }
   };
@@ -566,32 +689,17 @@ __global__ void __launch_bounds__(kScatThreads, 2) k_brick_scatter(
       // the warp's share: list positions [ra, rb)
       const int share = (np + kScatWarps - 1) / kScatWarps;
       const int ra = l0 + min(warp * share, np), rb = l0 + min((warp + 1) * share, np);
-      for (int q0 = 0; q0 < ns && ra < rb; q0 += 32) {
-        const int q = q0 + lane;
-        const bool over = q < ns && sh.pre[q] < rb && sh.pre[q + 1] > ra;
-        uint32_t todo = __ballot_sync(0xffffffffu, over);
-        int ds = 0, dc = 0;
-        uint32_t dorg = 0u;
-        if (over) describe(q, ds, dc, dorg);
-        while (todo) {
-          const int k = __ffs(todo) - 1;
-          todo &= todo - 1u;
-          const int s0 = __shfl_sync(0xffffffffu, ds, k), c = __shfl_sync(0xffffffffu, dc, k);
-          const uint32_t o = __shfl_sync(0xffffffffu, dorg, k);
-          int at = sh.pre[q0 + k];
-          for (int m0 = 0; m0 < c && at < rb; m0 += 32) {
-            uint32_t w = 0u;
-            bool t = false;
-            if (m0 + lane < c) {
-              w = __ldg(&win[s0 + m0 + lane]);
-              t = touches(w, o, ext1);
-            }
-            const uint32_t bal = __ballot_sync(0xffffffffu, t);
-            const int p = at + __popc(bal & ((1u << lane) - 1u));
-            if (t && p >= ra && p < rb)
-              queue[p - ra] = make_uint2((uint32_t)(s0 + m0 + lane), window_lo(w, o));
-            at += __popc(bal);
-          }
+      if (ra < rb) {
+        const int k = last_not_above(tab.mark, marks, ra);
+        int at = tab.mark[k];
+        for (int idx = k * G; at < rb && idx < tab.pre[ns]; idx += 32) {
+          int j = 0;
+          uint32_t lo = 0u;
+          const bool t = candidate(idx + lane, j, lo);
+          const uint32_t bal = __ballot_sync(0xffffffffu, t);
+          const int p = at + __popc(bal & ((1u << lane) - 1u));
+          if (t && p >= ra && p < rb) queue[p - ra] = make_uint2((uint32_t)j, lo);
+          at += __popc(bal);
         }
       }
       __syncwarp();
@@ -603,7 +711,7 @@ __global__ void __launch_bounds__(kScatThreads, 2) k_brick_scatter(
     int cw = 0;
     for (int p0 = 0; p0 < np; p0 += 32) {
       const uint32_t m = p0 + lane < np ? mask[p0 + lane] : 0u;
-      const bool t = (m >> warp) & 1u;
+      const bool t = (m >> tile) & 1u;
       const unsigned bal = __ballot_sync(0xffffffffu, t);
       if (t)
         mylist[cw + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)((p0 + lane) * (kPitch / 16));
@@ -614,24 +722,21 @@ __global__ void __launch_bounds__(kScatThreads, 2) k_brick_scatter(
     const unsigned char* const wty = row0 + kRowW + 4 * (8 * yh + gr);
     const unsigned char* const wtz = row0 + kRowW + 4 * (16 + 2 * zp);
     const unsigned btab = (unsigned)__cvta_generic_to_shared(row0) + ((lane >> 4) << 4);
-    for (int c0 = 0; c0 < cw; c0 += 16) {
+    for (int c0 = 16 * part; c0 < cw; c0 += 16 * kParts) {
       const uint32_t pa = *reinterpret_cast<const uint32_t*>(mylist + c0 + 2 * tq);
       const uint32_t pb = *reinterpret_cast<const uint32_t*>(mylist + c0 + 8 + 2 * tq);
       const unsigned pk[4] = {(pa & 0xffffu) * 16u, (pa >> 16) * 16u, (pb & 0xffffu) * 16u,
                               (pb >> 16) * 16u};
-      float w0[4], w1[4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const float y = *reinterpret_cast<const float*>(wty + pk[k]);
-        const float2 z = *reinterpret_cast<const float2*>(wtz + pk[k]);
-        w0[k] = y * z.x;
-        w1[k] = y * z.y;
-      }
       uint32_t ah[4], al[4];
-      split_pair(w0[0], w0[1], ah[0], al[0]);
-      split_pair(w1[0], w1[1], ah[1], al[1]);
-      split_pair(w0[2], w0[3], ah[2], al[2]);
-      split_pair(w1[2], w1[3], ah[3], al[3]);
+#pragma unroll
+      for (int k = 0; k < 4; k += 2) {
+        const Pair y = pair_of(*reinterpret_cast<const float*>(wty + pk[k]),
+                               *reinterpret_cast<const float*>(wty + pk[k + 1]));
+        const float2 z0 = *reinterpret_cast<const float2*>(wtz + pk[k]);
+        const float2 z1 = *reinterpret_cast<const float2*>(wtz + pk[k + 1]);
+        split_pair(y * pair_of(z0.x, z1.x), ah[k], al[k]);
+        split_pair(y * pair_of(z0.y, z1.y), ah[k + 1], al[k + 1]);
+      }
       const unsigned addr = btab + 16u * mylist[c0 + (lane & 15)];
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
@@ -648,15 +753,33 @@ __global__ void __launch_bounds__(kScatThreads, 2) k_brick_scatter(
         mma_f16(d0, ah, bh[0], bh[1]);
         mma_f16(d1, ah, bh[2], bh[3]);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          acc[c][0][k] += d0[k];
-          acc[c][1][k] += d1[k];
+        for (int k = 0; k < 2; ++k) {
+          acc[c][0][k] = acc[c][0][k] + pair_of(d0[2 * k], d0[2 * k + 1]);
+          acc[c][1][k] = acc[c][1][k] + pair_of(d1[2 * k], d1[2 * k + 1]);
         }
       }
     }
     if (l0 + bsize < total) __syncthreads();  // the rows are staged again
   }
 
+  if (kParts > 1) {
+    // the parts' sums, added in order by the first
+    __syncthreads();
+    Pair* const sums = reinterpret_cast<Pair*>(smem);  // [parts - 1][tiles][12][32]
+    if (part > 0) {
+      Pair* dst = sums + ((part - 1) * kTiles + tile) * 12 * 32 + lane;
+#pragma unroll
+      for (int k = 0; k < 12; ++k) dst[32 * k] = acc[k / 4][(k / 2) & 1][k & 1];
+    }
+    __syncthreads();
+    if (part > 0) return;
+    for (int q = 0; q < kParts - 1; ++q) {
+      const Pair* src = sums + (q * kTiles + tile) * 12 * 32 + lane;
+#pragma unroll
+      for (int k = 0; k < 12; ++k)
+        acc[k / 4][(k / 2) & 1][k & 1] = acc[k / 4][(k / 2) & 1][k & 1] + src[32 * k];
+    }
+  }
   // a lane holds nodes (x, x + 1) of row gr of both planes
   const float inv = ldexpf(1.f, ex - 28);
   const size_t nxy = (size_t)kp.n[0] * kp.n[1], nn = nxy * kp.n[2];
@@ -672,16 +795,65 @@ __global__ void __launch_bounds__(kScatThreads, 2) k_brick_scatter(
         float* d = S + (size_t)(b[2] + 2 * zp + z) * nxy + (size_t)(b[1] + y) * kp.n[0] + b[0] + x;
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-          const float v0 = acc[c][h][2 * z] * inv, v1 = acc[c][h][2 * z + 1] * inv;
+          const float2 v = parts(acc[c][h][z] * pair_of(inv, inv));
           if (pair) {
-            *reinterpret_cast<float2*>(d + c * nn) = make_float2(v0, v1);
+            *reinterpret_cast<float2*>(d + c * nn) = v;
           } else {
-            d[c * nn] = v0;
-            if (x + 1 < ext[0]) d[c * nn + 1] = v1;
+            d[c * nn] = v.x;
+            if (x + 1 < ext[0]) d[c * nn + 1] = v.y;
           }
         }
       }
     }
+  }
+}
+
+// One block per region; the dense ones (the sort lists those near a dense brick)
+// are k_brick_scatter_dense's.
+template <int LP>
+__global__ void __launch_bounds__(kScatThreads, 2) k_brick_scatter(
+    erpp_kparams kp, erpp_brick_dims bd, const int32_t* __restrict__ dflag,
+    const int2* __restrict__ axis, const float4* __restrict__ rec,
+    const uint32_t* __restrict__ win, const float4* __restrict__ fs,
+    const int32_t* __restrict__ bstart, const int32_t* __restrict__ bmax, float* __restrict__ S) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  __shared__ ScatShared sh;
+  const int gg[3] = {(int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z};
+  scatter_region<LP, 16>(kp, bd, gg, 0, axis, rec, win, fs, bstart, bmax,
+                         &dflag[(gg[2] * bd.ng[1] + gg[1]) * bd.ng[0] + gg[0]], S, smem, sh);
+  // k_brick_scatter_dense, which this kernel runs beside, is done before this one is
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// The dense regions by quarters of four planes, which the blocks take from a
+// counter, ndense[1].  A kernel of its own, beside which k_brick_scatter starts
+// at once: one kernel with both forms made the regions of a 512 x 256 x 256 box
+// with 1M particles 1.6% slower (438 and 431 us), and taking the quarters by a fixed
+// stride left clusters of 100k particles in 128^3 nodes at 400 - 470 us instead
+// of 260 - 320.
+template <int LP>
+__global__ void __launch_bounds__(kScatThreads, 2) k_brick_scatter_dense(
+    erpp_kparams kp, erpp_brick_dims bd, int32_t* __restrict__ ndense,
+    const int32_t* __restrict__ dense, const int2* __restrict__ axis,
+    const float4* __restrict__ rec, const uint32_t* __restrict__ win,
+    const float4* __restrict__ fs, const int32_t* __restrict__ bstart,
+    const int32_t* __restrict__ bmax, float* __restrict__ S) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  __shared__ ScatShared sh;
+  __shared__ int item;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const int nd = 4 * *ndense;
+  for (;;) {
+    if (threadIdx.x == 0) item = atomicAdd(&ndense[1], 1);
+    __syncthreads();
+    const int it = item;
+    if (it >= nd) break;
+    const int g = dense[it >> 2], z0 = 4 * (it & 3);
+    const int gg[3] = {g % bd.ng[0], (g / bd.ng[0]) % bd.ng[1], g / (bd.ng[0] * bd.ng[1])};
+    if (gg[2] * kRegion + z0 < kp.n[2])
+      scatter_region<LP, 4>(kp, bd, gg, z0, axis, rec, win, fs, bstart, bmax, nullptr, S, smem,
+                            sh);
+    __syncthreads();
   }
 }
 
@@ -734,6 +906,10 @@ bool use_bricks(const erpp_ctx* c, int64_t n) {
   return regions >= 152 || (n >= 16384 && (double)n >= 0.25 * nodes);
 }
 
+static size_t table_bytes(int nbricks) {
+  return sizeof(int32_t) * (2 * (size_t)nbricks + 3 + (size_t)(nbricks / 8));
+}
+
 cudaError_t bricks_alloc_tables(erpp_ctx* c) {
   erpp_bricks& k = c->bk;
   if (!bricks_possible(c)) return cudaSuccess;
@@ -742,14 +918,18 @@ cudaError_t bricks_alloc_tables(erpp_ctx* c) {
     k.dims.ng[a] = (c->kp.n[a] + kRegion - 1) / kRegion;
     ng *= k.dims.ng[a];
   }
-  if (ng > (1 << 24) || k.dims.ng[1] > 65535 || k.dims.ng[2] > 65535) return cudaSuccess;
+  if (ng > (1 << 24) || k.dims.ng[1] > 65535 || k.dims.ng[2] > 65000) return cudaSuccess;
   k.nbricks = (int)(8 * ng);
-  // counts, force maxima and the number of further adjoint chunks, cleared together
-  cudaError_t e = cudaMalloc(&k.cnt, sizeof(int32_t) * (2 * (size_t)k.nbricks + 1));
+  // cleared together: counts, force maxima, the numbers of further adjoint
+  // chunks and of dense regions, the regions' dense flags
+  cudaError_t e = cudaMalloc(&k.cnt, table_bytes(k.nbricks));
   if (e == cudaSuccess) e = cudaMalloc(&k.start, sizeof(int32_t) * ((size_t)k.nbricks + 4));
   if (e == cudaSuccess) e = cudaMalloc(&k.scan_tmp, sizeof(int32_t) * (k.nbricks / 4096 + 1));
   k.bmax = k.cnt ? k.cnt + k.nbricks : nullptr;
   k.nitems = k.cnt ? k.cnt + 2 * (size_t)k.nbricks : nullptr;
+  k.ndense = k.cnt ? k.nitems + 1 : nullptr;
+  k.dflag = k.cnt ? k.nitems + 3 : nullptr;
+  if (e == cudaSuccess) e = cudaMalloc(&k.dense, sizeof(int32_t) * (size_t)(k.nbricks / 8));
   std::vector<int2> ax;
   for (int a = 0; a < 3; ++a)
     for (int g = 0; g < k.dims.ng[a]; ++g) {
@@ -768,7 +948,9 @@ void bricks_free_tables(erpp_ctx* c) {
   cudaFree(k.start);
   cudaFree(k.scan_tmp);
   cudaFree(k.axis);
+  cudaFree(k.dense);
   k.axis = nullptr;
+  k.dense = k.ndense = k.dflag = nullptr;
   k.cnt = k.start = k.scan_tmp = k.bmax = k.nitems = nullptr;
 }
 
@@ -814,7 +996,7 @@ cudaError_t brick_sort(erpp_ctx* c, int64_t n, const double* const x[3], bool fo
                        cudaStream_t st) {
   erpp_bricks& k = c->bk;
   const int nb = k.nbricks;
-  cudaError_t e = cudaMemsetAsync(k.cnt, 0, sizeof(int32_t) * (2 * (size_t)nb + 1), st);
+  cudaError_t e = cudaMemsetAsync(k.cnt, 0, table_bytes(nb), st);
   if (e != cudaSuccess) return e;
   const unsigned blocks = (unsigned)((n + 255) / 256);
   // the records in order of arrival: where the forces go later
@@ -840,7 +1022,8 @@ cudaError_t brick_sort(erpp_ctx* c, int64_t n, const double* const x[3], bool fo
                          (const int32_t*)k.pidx, (const int32_t*)k.pbrick, (const float4*)rec_tmp,
                          (const int32_t*)k.start, k.rec,
                          k.win, k.slot, for_adjoint ? k.ord : nullptr, brick_tile(c),
-                         brick_chunk(c), k.nitems, k.items);
+                         brick_chunk(c), k.nitems, k.items, c->kp, k.dims, k.ndense, k.dense,
+                         k.dflag);
 }
 
 cudaError_t brick_forces(erpp_ctx* c, int64_t n, const double* const D[3], float scale,
@@ -855,14 +1038,21 @@ cudaError_t brick_forces(erpp_ctx* c, int64_t n, const double* const D[3], float
 cudaError_t brick_scatter(erpp_ctx* c, float* S, cudaStream_t st) {
   erpp_bricks& k = c->bk;
   const size_t sm = scatter_smem();
-  auto kern = c->kp.xs <= 7 ? k_brick_scatter<4> : k_brick_scatter<8>;
+  const bool four = c->kp.xs <= 7;
+  auto kern = four ? k_brick_scatter<4> : k_brick_scatter<8>;
+  auto dkern = four ? k_brick_scatter_dense<4> : k_brick_scatter_dense<8>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(dkern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
-  ++c->launches;
+  c->launches += 2;
+  constexpr int kResident = 2 * 152;
+  dkern<<<kResident, kScatThreads, sm, st>>>(c->kp, k.dims, k.ndense, k.dense, k.axis, k.rec, k.win,
+                                       k.fs, k.start, k.bmax, S);
+  // started beside the dense regions' kernel: its blocks wait for that one last
   const dim3 grid((unsigned)k.dims.ng[0], (unsigned)k.dims.ng[1], (unsigned)k.dims.ng[2]);
-  kern<<<grid, kScatThreads, sm, st>>>(c->kp, k.dims, k.axis, k.rec, k.win, k.fs, k.start,
-                                                k.bmax, S);
-  return cudaGetLastError();
+  return erpp_launch_pdl(kern, grid, dim3(kScatThreads), sm, st, 0, c->kp, k.dims, k.dflag, k.axis,
+                         k.rec, k.win, k.fs, k.start, k.bmax, S);
 }
 
 }  // namespace erpp

@@ -147,6 +147,10 @@ struct erpp_bricks {
   int32_t* ord;     // [cap] in order: particle (sorts for the adjoint)
   int2* items;      // further chunks of dense adjoint tiles: tile, first record
   int32_t* nitems;  // their number (after bmax, cleared with it)
+  int32_t* ndense;  // regions near a dense brick: their number, the quarters taken so
+                    //   far, and a flag per region
+  int32_t* dflag;   //   (cleared with the counts)
+  int32_t* dense;   // [nbricks / 8] the regions
   float4* rec;      // [cap] records in order: fractional position, window word
   uint32_t* win;    // [cap] the window words alone
   float4* rec_in;   // [cap] records in input order (scratch of the sort)
@@ -204,7 +208,8 @@ struct erpp_ctx {
                           // chunks of dense tiles (tile, first record); their number
                           // follows tile_cnt and is cleared with it
   float* halo;            // scatter x-halo columns, [ntiles][3][T_z][T_y][xhlo + xhhi]
-  int32_t* tile_cnt;      // [32 ntiles + 1]: pieces per (tile, bucket) bin; gather_items' number
+  int32_t* tile_cnt;      // [32 ntiles + 2]: pieces per (tile, bucket) bin; gather_items'
+                          // number, and how many of them are taken
   int32_t* tile_start;    // [32 ntiles + 1]
   int32_t* piece_slot;    // [maxseg product][cap]: each piece's place in its bin
   int32_t* scan_tmp;      // [ceil(32 ntiles / 4096)] chunk totals of the scan

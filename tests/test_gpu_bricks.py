@@ -66,6 +66,9 @@ CASES = {
     "stretched_81x96x90": (work((81, 96, 90), 5000, stretch=(1.0, 0.8, 1.3)), {}),
     "dense_24x20x18": (work((24, 20, 18), 18000), {}),
     "dense_wide_33x31x30": (work((33, 31, 30), 20000, 1.5, "clusters"), {}),
+    # whole regions of several batches; dense regions, by quarters, among others
+    "several_batches_64x64x48": (work((64, 64, 48), 59000), {}),
+    "dense_and_not_64x50x39": (work((64, 50, 39), 32000, 1.0, "clusters", 0.15), {}),
     "one_brick_of_many_16x16x16": (work((16, 16, 16), 30000, 1.0, "clusters", 0.05), {}),
 }
 
