@@ -322,8 +322,10 @@ erpp_status derive_ctx(const erpp_params* p, erpp_ctx* c) {
   kp.self_pref64 = -(p->dt / p->rho_f) / pow(2.0 * kPi * kp.self_s2, 1.5);
   kp.self_pref = (float)kp.self_pref64;
   kp.raw_norm1 = 1.0 / sqrt(2.0 * kPi * sig2);
+  kp.inv_dt = 1.0 / p->dt;
   kp.basset_c = p->dt > 0.0 ? 12.0 * (p->rho_f * p->nu) * sqrt(kPi / (p->nu * p->dt)) : 0.0;
   kp.self_inv_w = (float)(1.0 / sqrt(2.0 * kp.self_s2));
+  kp.drag64 = 6.0 * kPi * kp.mu;
   kp.drag_f = (float)(6.0 * kPi * kp.mu);
   kp.rho_f_f = (float)p->rho_f;
   kp.dt_f = (float)p->dt;

@@ -105,6 +105,8 @@ struct erpp_kparams {
   double raw_norm3;  // (2 pi sigma_R^2)^(-3/2)
   double raw_norm1;  // (2 pi sigma_R^2)^(-1/2)
   double self_pref64;// -(dt/rho_f) (2 pi self_s2)^(-3/2)
+  double inv_dt;     // 1 / dt
+  double drag64;     // 6 pi mu
   double basset_c;   // 12 mu sqrt(pi / (nu dt)) (ERPP_FULL_FORCE; 0 when dt = 0)
   double sig2;       // sigma_R^2
   double gauss_hi, gauss_lo; // -1 / (2 sigma_R^2), rounded, and the rest
