@@ -302,7 +302,10 @@ constexpr int kRegion = 16;      // nodes of a region per axis
 constexpr int kListBatch = 296;  // particles staged at a time, at most
 constexpr int kScatThreads = 512;
 constexpr int kScatWarps = kScatThreads / 32;
-constexpr int kQueue = (kListBatch + 16) / 4;  // members a warp queues before staging them
+// A warp's own list area: offsets of the rows it works on, from its start; the
+// queue of the members that it found, 4 bytes each, from its end.
+constexpr int kArea = 896;
+constexpr int kQueueMost = 4096;  // members of a segment whose places an entry can hold
 // Staged row of a particle: 3 components x (h, l) x 16 columns of FP16, 16 y-
 // and 16 z-weights (FP32).  The pitch puts the rows that an ldmatrix (eight consecutive particles) or a
 // fragment load (four, every other one) reads together in different banks.
@@ -445,7 +448,7 @@ __device__ __forceinline__ void scatter_region(
   constexpr int kTiles = ZS, kParts = kScatWarps / kTiles;  // 2 x 8-row tiles; warps of each
   unsigned char* const row0 = smem;  // [kListBatch + 1][kPitch]
   uint32_t* const mask = reinterpret_cast<uint32_t*>(row0 + (kListBatch + 1) * kPitch);
-  uint16_t* const wl = reinterpret_cast<uint16_t*>(mask + kListBatch);  // [warps][batch + 16]
+  unsigned char* const areas = reinterpret_cast<unsigned char*>(mask + kListBatch);
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int skipped = skip ? __ldg(skip) : 0;  // looked at after the segments' loads
@@ -483,8 +486,11 @@ __device__ __forceinline__ void scatter_region(
   const int myq = lane * kScatWarps + ((warp + 5 * lane) & (kScatWarps - 1));
   if (lane < K && myq < ns) mx = describe(myq, seg_s, seg_c, seg_o);
   if (skipped) return;
-  uint16_t* const mylist = wl + warp * (kListBatch + 16);
-  uint2* const queue = reinterpret_cast<uint2*>(mylist);  // until the warp's list is made
+  uint16_t* const mylist = reinterpret_cast<uint16_t*>(areas + warp * kArea);
+  // queue[-1 - k]: the k-th member, its place in its segment (12 bits), the
+  // warp's segment (5), its window's first node + 16 per axis (5 each)
+  uint32_t* const queue = reinterpret_cast<uint32_t*>(areas + (warp + 1) * kArea);
+  uint2* const dqueue = reinterpret_cast<uint2*>(mylist);  // dense regions: (record, window)
 
   // The members of the warp's segments, four segments at a time as one range,
   // 32 members a step; those that touch go into the warp's queue (while they
@@ -505,45 +511,50 @@ __device__ __forceinline__ void scatter_region(
       }
       for (int m0 = 0; m0 < tot; m0 += 32) {
         const int idx = m0 + lane;
-        int j = s0[0];
+        int j = s0[0], at0 = 0, sg = k;
         uint32_t og = o[0];
 #pragma unroll
         for (int i = 1; i < 4; ++i) {
-          j = idx >= e[i - 1] ? s0[i] : j;
-          og = idx >= e[i - 1] ? o[i] : og;
+          const bool up = idx >= e[i - 1];
+          j = up ? s0[i] : j;
+          og = up ? o[i] : og;
+          at0 = up ? e[i - 1] : at0;
+          sg = up ? k + i : sg;
         }
         j += idx;
         const uint32_t w = idx < tot ? __ldg(&win[j]) : 0u;
         const bool t = idx < tot && touches(w, og, ext1);
         const uint32_t bal = __ballot_sync(0xffffffffu, t);
         const int at = mine + __popc(bal & ((1u << lane) - 1u));
-        if (t && at < kQueue) queue[at] = make_uint2((uint32_t)j, window_lo(w, og));
+        if (t && at < kArea / 4) {
+          const uint32_t lo = window_lo(w, og) - 0x303030u;
+          queue[-1 - at] = (uint32_t)(idx - at0) | (uint32_t)sg << 12 | (lo & 31u) << 17 |
+                           (lo & 0x1f00u) << 14 | (lo >> 16) << 27;
+        }
         mine += __popc(bal);
       }
     }
   }
   mx = __reduce_max_sync(0xffffffffu, (unsigned)mx);
+  constexpr int kLong = 1 << 30;
+  const bool seg_long = __any_sync(0xffffffffu, seg_c > kQueueMost);
   __syncthreads();  // maxbits is cleared
   if (lane == 0) {
-    sh.cnt[warp] = mine;
+    sh.cnt[warp] = mine | (seg_long ? kLong : 0);
     if (mx > 0) atomicMax(&sh.maxbits, mx);
   }
   __syncthreads();
-  // the list: warp by warp, segment by segment, in record order
-  int total, at0;
-  bool dense;
-  {
-    const int v = lane < kScatWarps ? sh.cnt[lane] : 0;
-    int incl = v;
-#pragma unroll
-    for (int o = 1; o < kScatWarps; o <<= 1) {
-      const int u = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += u;
-    }
-    total = __shfl_sync(0xffffffffu, incl, kScatWarps - 1);
-    at0 = __shfl_sync(0xffffffffu, incl - v, warp);
-    dense = total > kListBatch || __any_sync(0xffffffffu, v > kQueue);
-  }
+  // The list: in one batch, or in several to which every warp gives an equal
+  // part of its queue (a batch then holds total / nbatch + 16 at most).  Dense
+  // regions, whose queues don't hold their members beside a batch's rows'
+  // offsets, are listed again below.
+  const int v = lane < kScatWarps ? sh.cnt[lane] & (kLong - 1) : 0;
+  const int total = __reduce_add_sync(0xffffffffu, v);
+  int nbatch = total <= kListBatch ? 1 : (total + kListBatch - 17) / (kListBatch - 16);
+  const int room =
+      nbatch == 1 ? kArea / 4 : (kArea - 2 * (total / nbatch + 16 + 16)) / 4;
+  const bool dense =
+      __any_sync(0xffffffffu, v > room || (lane < kScatWarps && sh.cnt[lane] >= kLong));
   DenseTab& tab = *reinterpret_cast<DenseTab*>(row0 + kDenseBatch * kPitch);
   int marks = 0, G = 32;
   // candidate idx of the range: its record, whether it touches, its window
@@ -609,19 +620,26 @@ __device__ __forceinline__ void scatter_region(
       for (int k = 0; k < 2; ++k) acc[c][h][k].v = 0ull;
 
   // batches of equal size, so that none leaves the warps a nearly empty chunk
-  const int most = dense ? kDenseBatch : kListBatch;
-  const int nbatch = (total + most - 1) / most;
-  const int bsize = nbatch > 0 ? (total + nbatch - 1) / nbatch : 1;
+  if (dense) nbatch = (total + kDenseBatch - 1) / kDenseBatch;
+  const int bsize = (total + nbatch - 1) / nbatch;
 
-  // Stages the queue's nq members as rows p0, p0 + 1, ...: LP lanes a particle,
+  // Stages members q0, q0 + 1, ... of the queue as rows p0, p0 + 1, ...: LP lanes a particle,
   // a pair of neighbouring nodes per axis each; the row cleared, then the
   // weights at the region's nodes.
-  auto stage = [&](int p0, int nq) {
+  auto stage = [&](int q0, int p0, int nq) {
     const int ql = lane & (LP - 1);
     for (int i0 = 0; i0 < nq; i0 += 32 / LP) {
       const int i = i0 + lane / LP;
       const bool live = i < nq;
-      const uint2 e = queue[live ? i : i0];
+      const int qi = live ? i : i0;
+      uint2 e;
+      if (dense) {
+        e = dqueue[qi];
+      } else {
+        const uint32_t m = queue[-1 - q0 - qi];
+        e.x = (m & 4095u) + __shfl_sync(0xffffffffu, seg_s, (m >> 12) & 31u);
+        e.y = (((m >> 17) & 31u) | (m >> 14 & 0x1f00u) | (m >> 27) << 16) + 0x303030u;
+      }
       const float4 r = __ldg(&rec[e.x]);
       const float4 f = __ldg(&fs[e.x]);
       unsigned char* const row = row0 + (p0 + i) * kPitch;
@@ -679,12 +697,23 @@ __device__ __forceinline__ void scatter_region(
     }
   };
 
-  for (int l0 = 0; l0 < total; l0 += bsize) {
-    const int np = min(bsize, total - l0);
+  for (int ib = 0; ib < nbatch; ++ib) {
+    const int l0 = ib * bsize;
+    int np = min(bsize, total - l0);
     // the warp's members of the batch
     if (!dense) {
-      __syncwarp();
-      stage(at0, mine);
+      const int v = lane < kScatWarps ? sh.cnt[lane] : 0;
+      const int from = nbatch == 1 ? 0 : v * ib / nbatch;
+      const int share = (nbatch == 1 ? v : v * (ib + 1) / nbatch) - from;
+      int incl = share;
+#pragma unroll
+      for (int o = 1; o < kScatWarps; o <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += u;
+      }
+      np = __shfl_sync(0xffffffffu, incl, kScatWarps - 1);
+      stage(__shfl_sync(0xffffffffu, from, warp), __shfl_sync(0xffffffffu, incl - share, warp),
+            __shfl_sync(0xffffffffu, share, warp));
     } else {
       // the warp's share: list positions [ra, rb)
       const int share = (np + kScatWarps - 1) / kScatWarps;
@@ -698,12 +727,12 @@ __device__ __forceinline__ void scatter_region(
           const bool t = candidate(idx + lane, j, lo);
           const uint32_t bal = __ballot_sync(0xffffffffu, t);
           const int p = at + __popc(bal & ((1u << lane) - 1u));
-          if (t && p >= ra && p < rb) queue[p - ra] = make_uint2((uint32_t)j, lo);
+          if (t && p >= ra && p < rb) dqueue[p - ra] = make_uint2((uint32_t)j, lo);
           at += __popc(bal);
         }
       }
       __syncwarp();
-      stage(ra - l0, rb - ra);
+      stage(0, ra - l0, rb - ra);
     }
     __syncthreads();
     // the warp's own particles, those that reach its rows and planes: their
@@ -759,7 +788,7 @@ __device__ __forceinline__ void scatter_region(
         }
       }
     }
-    if (l0 + bsize < total) __syncthreads();  // the rows are staged again
+    if (ib + 1 < nbatch) __syncthreads();  // the rows are staged again
   }
 
   if (kParts > 1) {
@@ -859,7 +888,7 @@ __global__ void __launch_bounds__(kScatThreads, 2) k_brick_scatter_dense(
 
 size_t scatter_smem() {
   return (size_t)(kListBatch + 1) * kPitch + (size_t)kListBatch * 4 +
-         (size_t)kScatWarps * (kListBatch + 16) * 2;
+         (size_t)kScatWarps * kArea;
 }
 
 // The stretches of bricks along an axis of n cells whose particles (windows
