@@ -588,12 +588,12 @@ cudaError_t bin_particles(erpp_ctx* ctx, int64_t n, const double* const x[3], bo
   cudaError_t e = cudaMemsetAsync(ctx->tile_cnt, 0,
                                   sizeof(int32_t) * (nbins + (ctx->gather_items ? 1 : 0)), st);
   if (e != cudaSuccess) return e;
-  if (n > 0 && kp.design == 4 && !kp.full_force && nbins <= kHistBins && ms <= kHistPieces) {
+  if (n > 0 && kp.design == 4 && nbins <= kHistBins && ms <= kHistPieces) {
     // few tiles (a small box): count through block histograms
     ++ctx->launches;
-    float4* no_lapc = nullptr;
+    float4* lapc = kp.full_force ? ctx->lapc : nullptr;
     e = erpp_launch_pdl(k_bin_count_hist, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, st,
-                        0u, kp, n, x[0], x[1], x[2], ctx->geo_t, ctx->geo_c, ctx->d0x, no_lapc,
+                        0u, kp, n, x[0], x[1], x[2], ctx->geo_t, ctx->geo_c, ctx->d0x, lapc,
                         ctx->tile_cnt, ctx->piece_slot, ms, nbins, ctx->err);
     if (e != cudaSuccess) return e;
   } else if (n > 0) {

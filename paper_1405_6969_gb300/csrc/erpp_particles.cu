@@ -209,7 +209,7 @@ __device__ void self_laplacian_f32(const erpp_kparams& kp, const float r[3], con
 // particle, two thirds of the 51 us for 300k particles (about 150 and 82 us with
 // the force written term by term and conversions by that pipe).
 template <bool F32>
-__global__ void __launch_bounds__(256) k_advance_full(erpp_kparams kp, int64_t n, PartPtrs P,
+__global__ void __launch_bounds__(256, 4) k_advance_full(erpp_kparams kp, int64_t n, PartPtrs P,
                                                       UpPtrs U, const double* __restrict__ lap,
                                                       double* __restrict__ prev, int64_t stride,
                                                       int first_step) {
