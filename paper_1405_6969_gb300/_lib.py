@@ -63,6 +63,14 @@ class Particles(ctypes.Structure):
     ]
 
 
+# The addresses of a double*[3] and the words of a Particles: filled at once and
+# taken for them with from_buffer (with a cast per pointer a step's call spent 24 us more on them)
+addr3 = ctypes.c_uint64 * 3
+particles_words = ctypes.c_uint64 * 15
+assert ctypes.sizeof(addr3) == ctypes.sizeof(_dp3)
+assert ctypes.sizeof(particles_words) == ctypes.sizeof(Particles)
+
+
 class BoxDesc(ctypes.Structure):
     _fields_ = [("params", Params), ("u", ctypes.c_void_p), ("particles", Particles),
                 ("S", ctypes.c_void_p)]

@@ -17,10 +17,6 @@ import torch
 from . import _lib
 
 
-def _dptr(t):
-    return ctypes.cast(ctypes.c_void_p(t.data_ptr()), _lib._dp)
-
-
 def _require_host(t, dtype, ndim):
     if not isinstance(t, torch.Tensor) or t.is_cuda:
         raise TypeError("expected a host (CPU) tensor")
@@ -33,10 +29,8 @@ def _vec3(t, host=False):
     """[3, n] float64 CUDA (or, host=True, CPU) tensor -> double*[3]."""
     (_require_host if host else _require)(t, torch.float64, 2)
     assert t.shape[0] == 3
-    n = t.shape[1]
-    base = t.data_ptr()
-    return _lib._dp3(*[ctypes.cast(ctypes.c_void_p(base + 8 * n * c), _lib._dp)
-                       for c in range(3)])
+    base, row = t.data_ptr(), 8 * t.shape[1]
+    return _lib._dp3.from_buffer(_lib.addr3(base, base + row, base + 2 * row))
 
 
 def _require(t, dtype, ndim):
@@ -76,15 +70,17 @@ class ParticleState:
 
     def to_c(self, host=False):
         """erpp_particles of the arrays (CUDA tensors; CPU ones with host=True)."""
-        P = _lib.Particles()
-        P.n = self.n
-        P.x, P.v = _vec3(self.x, host), _vec3(self.v, host)
-        P.x_prev, P.D = _vec3(self.x_prev, host), _vec3(self.D, host)
         req = _require_host if host else _require
-        req(self.radius, torch.float64, 1)
-        req(self.rho_p, torch.float64, 1)
-        P.radius, P.rho_p = _dptr(self.radius), _dptr(self.rho_p)
-        return P
+        words = [self.n]
+        for t in (self.x, self.v, self.x_prev, self.D):
+            req(t, torch.float64, 2)
+            assert t.shape[0] == 3
+            base, row = t.data_ptr(), 8 * t.shape[1]
+            words += (base, base + row, base + 2 * row)
+        for t in (self.radius, self.rho_p):
+            req(t, torch.float64, 1)
+            words.append(t.data_ptr())
+        return _lib.Particles.from_buffer(_lib.particles_words(*words))
 
     def pinned(self):
         """Copy of the state in page-locked host memory."""
