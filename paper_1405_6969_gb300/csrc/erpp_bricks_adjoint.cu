@@ -4,11 +4,14 @@
 //
 // A block serves the particles of one tile of cells (one range of the sorted
 // records): it stages the tile's field with a halo as wide as a window on all
-// sides (one TMA box; bulk row copies where the box wraps around the periodic
-// box; word by word where rows are not 16-byte aligned) and, while that is on
-// its way, writes every particle's weights and derivative weights to shared
-// memory, 16 lanes to a particle and axis.  Then a warp takes a particle: each
-// lane a (y, z) row of the window, walked along x in 16-byte loads.
+// sides (one TMA box; 16-byte copies where the box wraps around the periodic
+// box; word by word where rows are not 16-byte aligned).  A warp takes two
+// particles at a time: their weights and derivative weights into shared memory,
+// 16 lanes to a particle, then each lane a (y, z) row of the window, walked along
+// x in 16-byte loads.  The warps meet for the field only: with the weights of 40
+// particles written by the whole block between two barriers the warps waited for
+// one another, and 100k particles with windows of 9 nodes in 128^3 nodes took
+// 207 us instead of 170.  Shared memory then bounds it, and two blocks per SM.
 //
 // The warp-per-particle kernel reads the field from global memory, each lane
 // its own row, so that every load touches 32 lines, wraps every node index by a
@@ -35,15 +38,16 @@ constexpr int kWarps = kThreads / 32;
 
 // Tile and staged box of a window class.  HL: nodes staged below the tile in y
 // and z (x: 4, so that the box starts on 16 bytes); NW: longest window.  A tile
-// is TB consecutive bricks of a group; kChunk particles of it per block, kRows
-// at a time (as many weight rows as leave room for two blocks per SM).
+// is TB consecutive bricks of a group; kChunk particles of it per block (100k
+// particles in 128^3 nodes, 49 a tile: 189 us with chunks of 48, 170 with 64 or
+// 96, which dense tiles then share among more blocks than with longer ones).
 struct Geo7 {  // windows of at most 7 nodes that start at most 3 below the cell
   static constexpr int TB = 4, PX = 24, NY = 23, NZ = 15, HL = 3, NW = 7;
-  static constexpr int kChunk = 80, kRows = 40;
+  static constexpr int kChunk = 96;
 };
 struct Geo10 {  // at most 10 nodes, 4 below the cell
   static constexpr int TB = 2, PX = 28, NY = 17, NZ = 17, HL = 4, NW = 10;
-  static constexpr int kChunk = 80, kRows = 40;
+  static constexpr int kChunk = 96;
 };
 
 // A particle's row in shared memory: x-weights by staged column from a multiple
@@ -90,30 +94,28 @@ __device__ __forceinline__ int wrap_mod(int j, int n) {
   const int r = j % n;
   return r < 0 ? r + n : r;
 }
+// The same without a division where j is at most one period off.
+__device__ __forceinline__ int wrap_near(int j, int n) {
+  const int r = j < 0 ? j + n : (j >= n ? j - n : j);
+  return (unsigned)r < (unsigned)n ? r : wrap_mod(j, n);
+}
 
-// Copies of the tile's box by the whole block where one TMA box cannot: rows
-// and their periodic segments by bulk copies (nx a multiple of 4, u 16-byte
-// aligned; bar already expects the bytes), else word by word.
+// Copies of the tile's box by the whole block where one TMA box cannot: 16 bytes
+// a thread (nx a multiple of 4, u 16-byte aligned; no four words straddle the
+// box's end), else word by word.
 template <class G>
 __device__ void stage_rows(const erpp_kparams& kp, const float* __restrict__ u, float* field,
-                           const int b[3], uint64_t* bar) {
+                           const int b[3]) {
   const size_t nn = (size_t)kp.n[0] * kp.n[1] * kp.n[2];
-  const unsigned fbase = smem_u32(field), mb = smem_u32(bar);
   const int gx0 = wrap_mod(b[0] - 4, kp.n[0]);
-  for (int r = threadIdx.x; r < 3 * G::NZ * G::NY; r += kThreads) {
+  constexpr int kQ = G::PX / 4;
+  for (int i = threadIdx.x; i < 3 * G::NZ * G::NY * kQ; i += kThreads) {
+    const int r = i / kQ, q = i - r * kQ;
     const int cz = r / G::NY, y = r - cz * G::NY;
     const int c = cz / G::NZ, z = cz - c * G::NZ;
-    const int gy = wrap_mod(b[1] - G::HL + y, kp.n[1]), gz = wrap_mod(b[2] - G::HL + z, kp.n[2]);
-    const float* grow = u + c * nn + ((size_t)gz * kp.n[1] + gy) * kp.n[0];
-    unsigned dst = fbase + 4u * (unsigned)(r * G::PX);
-    int gx = gx0, left = G::PX;
-    while (left > 0) {
-      const int seg = min(left, kp.n[0] - gx);
-      bulk_load_g2s(dst, grow + gx, 4u * (unsigned)seg, mb);
-      dst += 4u * (unsigned)seg;
-      left -= seg;
-      gx = 0;
-    }
+    const int gy = wrap_near(b[1] - G::HL + y, kp.n[1]), gz = wrap_near(b[2] - G::HL + z, kp.n[2]);
+    const int gx = wrap_near(gx0 + 4 * q, kp.n[0]);
+    cp_async16(field + 4 * i, u + c * nn + ((size_t)gz * kp.n[1] + gy) * kp.n[0] + gx);
   }
 }
 template <class G>
@@ -166,7 +168,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_brick_adjoint(
   __shared__ __align__(8) uint64_t stall_bar;  // debug_stall only: never completed
   float* const field = reinterpret_cast<float*>(smem);
   constexpr int kField = 3 * CS;
-  float* const table = field + kField + 16;
+  float* const tables = field + kField + 16;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   unsigned phase = 0;
   if (tid == 0) {
@@ -210,111 +212,117 @@ __global__ void __launch_bounds__(kThreads, 2) k_brick_adjoint(
     const int x0 = b[0] - 4, y0 = b[1] - G::HL, z0 = b[2] - G::HL;
     const bool tma = use_tma && x0 >= 0 && x0 + G::PX <= kp.n[0] && y0 >= 0 &&
                      y0 + G::NY <= kp.n[1] && z0 >= 0 && z0 + G::NZ <= kp.n[2];
-    const bool on_bar = tma || rows_ok;
-    if (on_bar && tid == 0) {
-      mbar_expect_tx(&bar, (unsigned)(kField * 4));
-      if (tma) tma_load_4d(field, &tmap, &bar, x0, y0, z0, 0);
-    }
-    if (!tma) {
-      if (rows_ok) {
-        __syncthreads();  // the barrier expects the bytes
-        stage_rows<G>(kp, u, field, b, &bar);
-      } else {
-        stage_words<G>(kp, u, field, b);
+    if (tma) {
+      if (tid == 0) {
+        mbar_expect_tx(&bar, (unsigned)(kField * 4));
+        tma_load_4d(field, &tmap, &bar, x0, y0, z0, 0);
       }
+    } else if (rows_ok) {
+      stage_rows<G>(kp, u, field, b);
+    } else {
+      stage_words<G>(kp, u, field, b);
     }
+    // A warp takes two particles at a time: their weights, then their sums.  The
+    // block meets only for the field.
     bool waited = false;
-    for (int p0 = 0; p0 < cnt; p0 += G::kRows) {
-      const int np = min(G::kRows, cnt - p0);
-      // the weights: 16 lanes to a particle and axis, a node of the window each
+    float* const table = tables + warp * 2 * T::kRow;
+    for (int p0 = 2 * warp;; p0 += 2 * kWarps) {
+      const int np = min(2, cnt - p0);
+      // the weights: 16 lanes to a particle, a node of the window each
       const int ql = lane & 15;
-      for (int i0 = warp * 2; i0 < 3 * np; i0 += kWarps * 2) {
-        const int i = min(i0 + (lane >> 4), 3 * np - 1);
-        const int a = i / np, p = i - a * np;
+      if (np > 0) {
+        const int p = min(lane >> 4, np - 1);
         const int j = j0 + p0 + p;
         const uint32_t w = __float_as_uint(__ldg(&rec[j].w));
         const int pi = ag.ord[j];
-        // first node of the window in the brick, and the brick in the tile (its
-        // place among the bricks' ranges)
+        double xp[3];
+        float vp[3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+          xp[a] = ag.x[a][pi];
+          vp[a] = (float)ag.v[a][pi];
+        }
+        // the brick in the tile (its place among the bricks' ranges)
         int brick = 0;
 #pragma unroll
         for (int k = 1; k < G::TB; ++k) brick += j >= bstart[tile * G::TB + k] ? 1 : 0;
-        const int lo = erpp_rec_lo(w, a), nw = erpp_rec_nw(w, a), off = erpp_rec_off(kp, w, a);
-        const double xa = a == 0 ? ag.x[0][pi] : (a == 1 ? ag.x[1][pi] : ag.x[2][pi]);
-        const double s = __dmul_rn(xa, a == 0 ? kp.inv_dx[0] : (a == 1 ? kp.inv_dx[1] : kp.inv_dx[2]));
-        const float sig2 = ag.sig2;
-        const float dxa = a == 0 ? ag.dx[0] : (a == 1 ? ag.dx[1] : ag.dx[2]);
-        float wv = 0.f, d = 0.f;
-        if (ql < nw) {
-          d = distance(s, off + ql) * dxa;  // signed distance x_j - x_p
-          wv = ag.raw1 * expf(-(d * d) / (2.f * sig2));
-        }
-        float dwv;
-        if (kp.normalize) {
-          const float sum = half_sum(wv);
-          wv = wv / (dxa * sum);
-          const float mean = dxa * half_sum(wv * d);  // dx sum_k w_k d_k
-          dwv = wv * (d - mean) / sig2;
-        } else {
-          dwv = wv * d / sig2;
-        }
         float* const row = table + p * T::kRow;
-        if (a == 0) {
-          const int sx = (lo + 4 + 8 * (brick & 1)) & 3;
+        const int sx = erpp_rec_lo(w, 0) + 4 + 8 * (brick & 1);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+          const int nw = erpp_rec_nw(w, a), off = erpp_rec_off(kp, w, a);
+          const double s = __dmul_rn(xp[a], kp.inv_dx[a]);
+          const float sig2 = ag.sig2, dxa = ag.dx[a];
+          float wv = 0.f, d = 0.f;
           if (ql < nw) {
-            row[T::kX + sx + ql] = wv;
-            row[T::kDX + sx + ql] = dwv;
+            d = distance(s, off + ql) * dxa;  // signed distance x_j - x_p
+            wv = ag.raw1 * expf(-(d * d) / (2.f * sig2));
           }
-        } else if (ql < nw) {
-          row[(a == 1 ? T::kY : T::kZ) + ql] = wv;
-          row[(a == 1 ? T::kDY : T::kDZ) + ql] = dwv;
+          // lanes beyond the window divide ones: a zero takes a division's slow way
+          const bool idle = ql >= nw;
+          float dwv;
+          if (kp.normalize) {
+            const float sum = half_sum(wv);
+            wv = (idle ? 1.f : wv) / (dxa * sum);
+            const float mean = dxa * half_sum(wv * d);  // dx sum_k w_k d_k
+            dwv = (idle ? 1.f : wv * (d - mean)) / sig2;
+          } else {
+            dwv = (idle ? 1.f : wv * d) / sig2;
+          }
+          if (!idle) {
+            row[(a == 0 ? T::kX + (sx & 3) : (a == 1 ? T::kY : T::kZ)) + ql] = wv;
+            row[(a == 0 ? T::kDX + (sx & 3) : (a == 1 ? T::kDY : T::kDZ)) + ql] = dwv;
+          }
         }
         if (ql == 0) {
-          row[T::kMeta + 4 + a] =
-              (float)(a == 0 ? ag.v[0][pi] : (a == 1 ? ag.v[1][pi] : ag.v[2][pi]));
-          if (a == 2) {
-            // the window's first staged word, its columns from a multiple of 4
-            const int sx = erpp_rec_lo(w, 0) + 4 + 8 * (brick & 1);
-            const int sy = erpp_rec_lo(w, 1) + G::HL + (G::TB == 4 ? 8 * (brick >> 1) : 0);
-            const int nwx = erpp_rec_nw(w, 0);
-            *reinterpret_cast<int4*>(row + T::kMeta) = make_int4(
-                ((lo + G::HL) * G::NY + sy) * G::PX + (sx & ~3),
-                (int)(((1u << nwx) - 1u) << (sx & 3)), erpp_rec_nw(w, 1), nw);
+          // the window's first staged word, its columns from a multiple of 4, and
+          // r / ny for r < 128 as r (65536 / ny + 1) / 65536
+          const int sy = erpp_rec_lo(w, 1) + G::HL + (G::TB == 4 ? 8 * (brick >> 1) : 0);
+          const int nwx = erpp_rec_nw(w, 0), ny = erpp_rec_nw(w, 1);
+          *reinterpret_cast<int4*>(row + T::kMeta) =
+              make_int4(((erpp_rec_lo(w, 2) + G::HL) * G::NY + sy) * G::PX + (sx & ~3),
+                        (int)(((1u << nwx) - 1u) << (sx & 3)), ny | (65536 / ny + 1) << 4,
+                        erpp_rec_nw(w, 2));
+#pragma unroll
+          for (int a = 0; a < 3; ++a) row[T::kMeta + 4 + a] = vp[a];
+        }
+      }
+      if (!waited) {
+        // one thread waits (bounded) for the field; the block goes on or gives up
+        // as a whole
+        if (!tma) cp_async_wait_all();
+        int timed_out = 0;
+        if (tma && tid == 0) {
+          bool ok = mbar_wait_ns(&bar, phase, kp.wait_ns);
+          if (!ok) {
+            mbar_wait_ns(&bar, phase, kp.wait_ns);  // once more for the copy in flight
+          } else if (kp.debug_stall) {
+            ok = mbar_wait_ns(&stall_bar, 0, kp.wait_ns);  // nothing arrives: runs out
+          }
+          if (!ok) {
+            erpp_set_err(err, ERPP_ERRBIT_TIMEOUT);
+            timed_out = 1;
           }
         }
-      }
-      // one thread waits (bounded) for the field; the block goes on or gives up
-      // as a whole
-      if (!on_bar) cp_async_wait_all();
-      int timed_out = 0;
-      if (on_bar && !waited && tid == 0) {
-        bool ok = mbar_wait_ns(&bar, phase, kp.wait_ns);
-        if (!ok) {
-          mbar_wait_ns(&bar, phase, kp.wait_ns);  // once more for the copy in flight
-        } else if (kp.debug_stall) {
-          ok = mbar_wait_ns(&stall_bar, 0, kp.wait_ns);  // nothing arrives: runs out
+        if (__syncthreads_or(timed_out)) return;
+        // the phase has completed: every thread observes it, which returns at once
+        if (tma) {
+          if (tid != 0) mbar_try_wait(&bar, phase);
+          phase ^= 1u;
         }
-        if (!ok) {
-          erpp_set_err(err, ERPP_ERRBIT_TIMEOUT);
-          timed_out = 1;
-        }
-      }
-      if (__syncthreads_or(timed_out)) return;
-      // the phase has completed: every thread observes it, which returns at once
-      if (on_bar && !waited) {
-        if (tid != 0) mbar_try_wait(&bar, phase);
-        phase ^= 1u;
         waited = true;
       }
-      for (int p = warp; p < np; p += kWarps) {
+      if (np <= 0) break;
+      __syncwarp();
+      for (int p = 0; p < np; ++p) {
         float* const row = table + p * T::kRow;
         const int4 meta = *reinterpret_cast<const int4*>(row + T::kMeta);
         const float v0 = row[T::kMeta + 4], v1 = row[T::kMeta + 5], v2 = row[T::kMeta + 6];
         const unsigned cols = (unsigned)meta.y;  // the window's columns, from the first load
-        const int ny = meta.z, rows = meta.z * meta.w;
+        const int ny = meta.z & 15, per = meta.z >> 4, rows = ny * meta.w;
         float g0 = 0.f, g1 = 0.f, g2 = 0.f, h0 = 0.f, h1 = 0.f, h2 = 0.f;
         for (int r = lane; r < rows; r += 32) {
-          const int kz = r / ny, ky = r - kz * ny;
+          const int kz = (r * per) >> 16, ky = r - kz * ny;
           const float* f = field + meta.x + kz * PL + ky * G::PX;
           float a0 = 0.f, a1 = 0.f, a2 = 0.f, b0 = 0.f, b1 = 0.f, b2 = 0.f;
 #pragma unroll
@@ -357,21 +365,23 @@ __global__ void __launch_bounds__(kThreads, 2) k_brick_adjoint(
         __syncwarp();
         if ((lane & 3) == 0) row[lane >> 2] = sum;
       }
-      __syncthreads();
-      if (tid < np) {
-        const float* const row = table + tid * T::kRow;
-        const int i = ag.ord[j0 + p0 + tid];
-        if (ag.val[0]) {
-          ag.val[0][i] = ag.alpha * (double)row[0];
-          ag.val[1][i] = ag.alpha * (double)row[1];
-          ag.val[2][i] = ag.alpha * (double)row[2];
+      __syncwarp();
+      if (lane < 6 * np) {
+        const int p = lane >= 6 ? 1 : 0, q = lane - 6 * p;
+        const float sum = table[p * T::kRow + q];
+        const int i = ag.ord[j0 + p0 + p];
+        if (q < 3) {
+          double* const to = q == 0 ? ag.val[0] : (q == 1 ? ag.val[1] : ag.val[2]);
+          if (to) to[i] = ag.alpha * (double)sum;
+        } else if (q == 4) {
+          ag.der[1][i] = ag.alpha * (double)sum + ag.shear * ag.v[0][i];
+        } else {
+          (q == 3 ? ag.der[0] : ag.der[2])[i] = ag.alpha * (double)sum;
         }
-        ag.der[0][i] = ag.alpha * (double)row[3];
-        ag.der[1][i] = ag.alpha * (double)row[4] + ag.shear * ag.v[0][i];
-        ag.der[2][i] = ag.alpha * (double)row[5];
       }
-      __syncthreads();  // the table (and the field) are written again
+      __syncwarp();  // the table is written again
     }
+    __syncthreads();  // and the field
   }
 }
 
@@ -381,7 +391,7 @@ cudaError_t launch(erpp_ctx* c, const float* u, int64_t n, const AdjArgs& ag, cu
   erpp_bricks& k = c->bk;
   auto kern = k_brick_adjoint<G>;
   const size_t sm = sizeof(float) * (3 * (size_t)G::NZ * G::NY * G::PX + 16 +
-                                     (size_t)G::kRows * Row<G>::kRow);
+                                     2 * kWarps * (size_t)Row<G>::kRow);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
   CUtensorMap map;
