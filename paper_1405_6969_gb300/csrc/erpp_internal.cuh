@@ -142,6 +142,7 @@ struct erpp_bricks {
   int32_t* start;   // [nbricks + 1]
   int32_t* scan_tmp;
   int2* axis;       // per axis and group: the stretches of bricks around it
+  unsigned char* block;  // the allocation that holds the arrays below, but for the tables
   int2* key;        // [cap] per particle: brick (-1: invalid position), place by arrival
   int32_t* pidx;    // [cap] in order of arrival: particle
   int32_t* pbrick;  // [cap] in order of arrival: brick
