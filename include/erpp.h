@@ -441,7 +441,7 @@ erpp_status erpp_set_tiling(erpp_ctx* ctx, int32_t tile_y, int32_t tile_z, int32
  * order of FP32 additions, and each is reproducible bit for bit):
  *   ERPP_SCATTER_MERGE (default): one block per tile writes its interior to S
  *     and its halo to strips in a context buffer; two merge kernels then add
- *     the strips onto the neighbouring tiles' rims.  Boxes of at least 152
+ *     the strips onto the neighbouring tiles' rims.  Boxes of at least 120
  *     regions of 16^3 nodes, or dense ones (16384 particles and a quarter per
  *     node), with windows of at most 10 nodes and without ERPP_KAHAN, take the
  *     source from particles sorted by 8^3-cell bricks instead: no tiles and no

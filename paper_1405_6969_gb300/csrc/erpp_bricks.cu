@@ -925,15 +925,18 @@ bool bricks_possible(const erpp_ctx* c) {
 }
 
 // The brick kernels serve a call when the context's scatter mode is the
-// default and the box gives every SM a region to work on (152 regions of
-// 16^3 nodes), or its particles are dense (a quarter of a particle per node,
-// 16384 at least: the x/y-halo tiles then hold thousands of pieces each).  Smaller boxes keep
-// the tile kernels, whose smaller blocks finish earlier there.
+// default and the box has regions of 16^3 nodes for most SMs, or its particles
+// are dense (a quarter of a particle per node, 16384 at least: the x/y-halo
+// tiles then hold thousands of pieces each).  One source by bricks and by tiles:
+// 64 regions, 16k particles (64^3) 51 and 44 us, but 64k 155 and 236 us; 125
+// regions, 20k (80^3) 36 and 46; 180, 20k (96 x 96 x 80) 32 and 43; 512, 30k
+// (128^3) 38 and 53 us.
+constexpr int64_t kRegionsLeast = 120;
 bool use_bricks(const erpp_ctx* c, int64_t n) {
   if (!c->bk.rec || c->scatter_mode != ERPP_SCATTER_MERGE || n <= 0) return false;
   const int64_t regions = c->bk.nbricks / 8;
   const double nodes = (double)c->kp.n[0] * c->kp.n[1] * c->kp.n[2];
-  return regions >= 152 || (n >= 16384 && (double)n >= 0.25 * nodes);
+  return regions >= kRegionsLeast || (n >= 16384 && (double)n >= 0.25 * nodes);
 }
 
 static size_t table_bytes(int nbricks) {

@@ -52,11 +52,12 @@ def work(n, particles, sigma=1.0, cloud="uniform", std=0.3, cutoff=3.0, stretch=
                                cutoff=cutoff)
 
 
-# at least 152 regions of 16^3 nodes, or a quarter of a particle per node
+# at least 120 regions of 16^3 nodes, or a quarter of a particle per node
 # and 16384 particles, so that the library's rule takes the brick kernels
 CASES = {
     "ragged_90x83x85": (work((90, 83, 85), 5000), {}),
     "even_96x96x80_raw": (work((96, 96, 80), 5000), dict(normalize=False)),
+    "few_regions_80x74x90": (work((80, 74, 90), 5000), {}),
     "rows_of_odd_length_91x97x81": (work((91, 97, 81), 9000, 1.5, "clusters"), {}),
     "thin_x_9x300x170": (work((9, 300, 170), 4000), {}),
     "one_past_a_region_17x289x81": (work((17, 289, 81), 4000), {}),
