@@ -1554,7 +1554,7 @@ inline double gather_lanes(const erpp_kparams& kp, int64_t n, int PB, int NT) {
 
 // LAP (the general force's gather) runs 256-thread blocks or, where two blocks
 // fit on an SM with half the pieces a batch and one otherwise, 384-thread blocks
-// with such batches (300k particles in 192^3 nodes: 187 -> 125 us; 137 us with 256
+// with such batches (300k particles in 192^3 nodes: 187 -> 146 us; 154 us with 256
 // threads, 166 us for one block of 512 threads with whole batches).
 template <int XM, int LMIN, int XW, bool LAP = false>
 cudaError_t gather4(erpp_ctx* ctx, const float* u, int64_t n, cudaStream_t st) {
