@@ -381,7 +381,10 @@ __global__ void __launch_bounds__(kThreads, 2) k_brick_adjoint(
       }
       __syncwarp();  // the table is written again
     }
-    __syncthreads();  // and the field
+    // a block that took a tile's first chunk is done (without further chunks' blocks,
+    // nextra = 0, the loop has no step)
+    if (!extra) break;
+    __syncthreads();  // the field is written again
   }
 }
 
