@@ -214,6 +214,10 @@ __global__ void __launch_bounds__(kThreads, 2) k_brick_adjoint(
                      y0 + G::NY <= kp.n[1] && z0 >= 0 && z0 + G::NZ <= kp.n[2];
     if (tma) {
       if (tid == 0) {
+        // a further chunk's box lands where the tile before was staged, by the
+        // generic proxy perhaps, and read: the block's barrier and this fence
+        // put those accesses before the copy's
+        fence_proxy_async_shared();
         mbar_expect_tx(&bar, (unsigned)(kField * 4));
         tma_load_4d(field, &tmap, &bar, x0, y0, z0, 0);
       }

@@ -69,3 +69,34 @@ def test_few_particles(erpp, oracle_lib, n, sigma, particles, cloud):
     assert rel(dD, rdD) < TOL and rel(dxs, rdx) < TOL
     rdu, rdx = oracle_lib.gather_backward(p, x, R.astype(np.float64), D)
     assert rel(dxg, rdx) < TOL and rel(du, rdu) < TOL
+
+
+@pytest.mark.parametrize("sigma", [1.0, 1.5])
+def test_blocks_of_many_chunks(erpp, oracle_lib, sigma):
+    """More further chunks than blocks for them (608): a block stages tiles at
+    the box's faces (copied row by row) and inside (one TMA box) in turn into the
+    same shared memory."""
+    import torch
+    n = (96, 80, 96)
+    w = dataclasses.replace(I.CFG_SMALL, n=n, L=tuple(v * DX for v in n), sigma_over_dx=sigma,
+                            shear_rate=0.5)
+    p = w.params()
+    rng = np.random.default_rng(2)
+    corners = np.array([[0, 0, 0], [40, 32, 40], [88, 72, 88], [24, 40, 56]]).T[:, :, None]
+    x = ((corners + 8 * rng.random((3, 4, 20000))) * DX * (1 - 1e-9)).reshape(3, -1)
+    assert sum(c // 96 for c in [20000] * 4) > 608
+    D = rng.standard_normal(x.shape)
+    R = rng.standard_normal((3,) + n[::-1]).astype(np.float32)
+    cu = lambda a: torch.as_tensor(np.ascontiguousarray(a)).cuda()  # noqa: E731
+    got = []
+    for mode in ("merge", "cluster"):
+        ctx = erpp.Context(p, precision="fp32")
+        ctx.set_scatter_mode(mode)
+        got.append(ctx.scatter_backward(cu(x), cu(D), cu(R)))
+        ctx.check()
+    for a, b in zip(*got):
+        assert torch.equal(a, b)
+    few = np.ascontiguousarray(x[:, ::40])
+    rdD, rdx = oracle_lib.scatter_backward(p, few, np.ascontiguousarray(D[:, ::40]),
+                                           R.astype(np.float64))
+    assert rel(got[0][0][:, ::40], rdD) < TOL and rel(got[0][1][:, ::40], rdx) < TOL
