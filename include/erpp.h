@@ -280,6 +280,14 @@ erpp_status erpp_check(erpp_ctx* ctx, erpp_stream stream);
 erpp_status erpp_debug_windows(erpp_ctx* ctx, int64_t n, const double* const x[3],
                                int32_t* jlo, int32_t* jhi, erpp_stream stream);
 
+/* Which parts of the most recent erpp_step, erpp_scatter_source,
+ * erpp_scatter_backward or erpp_gather_backward on ctx ran from particles sorted
+ * by bricks (a tracing and testing aid): ERPP_ROUTE_SOURCE the source (or du),
+ * ERPP_ROUTE_ADJOINT the contractions of a backward call; written to the HOST int
+ * *route. */
+enum { ERPP_ROUTE_SOURCE = 1, ERPP_ROUTE_ADJOINT = 2 };
+erpp_status erpp_debug_last_route(erpp_ctx* ctx, int32_t* route);
+
 /* Bounded device-side waits (a tracing and testing aid, not part of the
  * method).  The FP32 tile gather stages each tile by asynchronous copies
  * completed on a shared-memory barrier; one thread of the block waits for it

@@ -95,6 +95,7 @@ _SIGS = {
     "erpp_step_host_wait": (_st, [_vp, _vp]),
     "erpp_momentum": (_st, [_vp, _vp, _i64, _dp3, _dp3, _dp, _vp]),
     "erpp_check": (_st, [_vp, _vp]),
+    "erpp_debug_last_route": (_st, [_vp, ctypes.POINTER(ctypes.c_int32)]),
     "erpp_debug_windows": (_st, [_vp, _i64, _dp3, _vp, _vp, _vp]),
     "erpp_debug_set_wait": (_st, [_vp, _i64, ctypes.c_int32]),
     "erpp_interpolate_noalloc": (_st, [ctypes.POINTER(Params), _vp, _i64, _dp3, _dp3, _vp]),

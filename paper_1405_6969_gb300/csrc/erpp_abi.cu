@@ -195,8 +195,8 @@ erpp_status alloc_weight_tables(erpp_ctx* c) {
 // Whether an adjoint, which needs no scratch otherwise, takes the brick kernels:
 // where their scratch is there, or can be made without losing a step history
 // and outside a stream capture.
-bool adjoint_bricks(erpp_ctx* c, int64_t n, cudaStream_t st) {
-  if (c->fp64 || n <= 0 || !erpp::bricks_possible(c)) return false;
+bool adjoint_bricks(erpp_ctx* c, int64_t n, const void* F, cudaStream_t st) {
+  if (c->fp64 || !erpp::bricks_possible(c) || !erpp::bricks_pay_adjoint(c, n, F)) return false;
   if (n > c->cap) {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (c->kp.lag > 0 || c->kp.full_force ||
@@ -206,7 +206,9 @@ bool adjoint_bricks(erpp_ctx* c, int64_t n, cudaStream_t st) {
       return false;
     }
   }
-  return erpp::use_bricks(c, n);
+  if (!erpp::use_bricks(c, n)) return false;
+  c->route |= ERPP_ROUTE_ADJOINT;
+  return true;
 }
 
 erpp_status check_n(int64_t n) {
@@ -600,6 +602,7 @@ erpp_status erpp_scatter_source(erpp_ctx* c, int64_t n, const double* const x[3]
   cudaStream_t st = (cudaStream_t)stream;
   erpp_status s = erpp::ensure_capacity(c, n);
   if (s) return s;
+  c->route = 0;
   return set_cuda_err(erpp::scatter_source(c, n, x, D, S, st));
 }
 
@@ -612,8 +615,9 @@ erpp_status erpp_scatter_backward(erpp_ctx* c, int64_t n, const double* const x[
   if (dD && (!dD[0] || !dD[1] || !dD[2])) return ERPP_EINVAL;
   cudaStream_t st = (cudaStream_t)stream;
   cudaError_t e;
-  if (adjoint_bricks(c, n, st)) {
-    e = erpp::brick_sort(c, n, x, true, st);
+  c->route = 0;
+  if (adjoint_bricks(c, n, R, st)) {
+    e = erpp::brick_sort(c, n, x, false, true, st);
     if (e == cudaSuccess)
       e = erpp::brick_adjoint(c, n, x, (const float*)R, D, -1.0 / c->params.rho_f, 0.0, dD, dx,
                               st);
@@ -632,9 +636,14 @@ erpp_status erpp_gather_backward(erpp_ctx* c, int64_t n, const double* const x[3
   if (!du && !dx) return ERPP_EINVAL;
   cudaStream_t st = (cudaStream_t)stream;
   cudaError_t e = cudaSuccess;
+  c->route = 0;
   // one sort serves both parts
-  const bool adj = dx && adjoint_bricks(c, n, st);
-  if (adj) e = erpp::brick_sort(c, n, x, true, st);
+  const bool adj = dx && adjoint_bricks(c, n, u, st);
+  bool sorted = false;  // for the source too
+  if (adj) {
+    sorted = du && erpp::use_bricks(c, n);
+    e = erpp::brick_sort(c, n, x, sorted, true, st);
+  }
   if (e == cudaSuccess && dx && n > 0)
     e = adj ? erpp::brick_adjoint(c, n, x, (const float*)u, g, c->kp.dV, c->params.shear_rate,
                                   nullptr, dx, st)
@@ -646,7 +655,7 @@ erpp_status erpp_gather_backward(erpp_ctx* c, int64_t n, const double* const x[3
     if (c->fp64) {
       e = erpp::launch_scatter_f64(c, n, x, g, c->kp.dV, (double*)du, false, st);
     } else if (erpp::use_bricks(c, n)) {
-      if (!adj) e = erpp::brick_sort(c, n, x, false, st);
+      if (!sorted) e = erpp::brick_sort(c, n, x, true, false, st);
       if (e == cudaSuccess) e = erpp::brick_forces(c, n, g, 1.0f, st);
       if (e == cudaSuccess) e = erpp::brick_scatter(c, (float*)du, st);
     } else {
@@ -684,7 +693,7 @@ cudaError_t scatter_source(erpp_ctx* c, int64_t n, const double* const x[3],
     return erpp::launch_scatter_f64(c, n, x, D, -1.0 / c->params.rho_f, (double*)S, false, st);
   cudaError_t e;
   if (use_bricks(c, n)) {
-    e = brick_sort(c, n, x, false, st);
+    e = brick_sort(c, n, x, true, false, st);
     if (e == cudaSuccess) e = brick_forces(c, n, D, -c->kp.inv_rho_dV, st);
     if (e == cudaSuccess) e = brick_scatter(c, (float*)S, st);
     return e;
@@ -809,6 +818,7 @@ erpp_status step_device(erpp_ctx* c, const void* u, const erpp_particles* P, voi
   const int64_t n = P->n;
   erpp_status s = erpp::ensure_capacity(c, n);
   if (s) return s;
+  c->route = 0;
   if (c->kp.lag > 0) return step_lagged(c, u, P, S, first_step, st, after_advance);
   if (c->kp.full_force) return step_full_force(c, u, P, S, first_step, st, after_advance);
   const double* const xin[3] = {P->x[0], P->x[1], P->x[2]};
@@ -845,7 +855,7 @@ erpp_status step_device(erpp_ctx* c, const void* u, const erpp_particles* P, voi
     if (c->prof_on) ev = c->prof_ev + 5 * (c->prof_n++ % kProfSets);
     if (ev) cudaEventRecord(ev[0], st);
     const bool bricks = use_bricks(c, n);
-    e = bricks ? brick_sort(c, n, xin, false, st) : cudaSuccess;
+    e = bricks ? brick_sort(c, n, xin, true, false, st) : cudaSuccess;
     if (e == cudaSuccess) e = erpp::bin_particles(c, n, xin, true, st);
     if (ev) cudaEventRecord(ev[1], st);
     if (e == cudaSuccess) e = erpp::launch_gather_f32(c, (const float*)u, n, st);
@@ -869,6 +879,12 @@ extern "C" {
 erpp_status erpp_last_step_launches(erpp_ctx* c, int32_t* n) {
   if (!c || !n) return ERPP_EINVAL;
   *n = c->last_step_launches;
+  return ERPP_OK;
+}
+
+erpp_status erpp_debug_last_route(erpp_ctx* c, int32_t* route) {
+  if (!c || !route) return ERPP_EINVAL;
+  *route = c->route;
   return ERPP_OK;
 }
 

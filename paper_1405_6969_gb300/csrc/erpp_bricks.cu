@@ -154,13 +154,31 @@ __global__ void __launch_bounds__(1024) k_brick_scan(const int32_t* __restrict__
   if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) start[nb] = all + tot;
 }
 
+// Records of the adjoint's particles: the particle of each, and the further chunks
+// of tiles of more than `chunk` particles.
+struct AdjOrder {
+  int32_t* ord;  // null: not for the adjoint
+  int32_t* nitems;
+  int2* items;
+  int tile_bricks, chunk;
+  __device__ __forceinline__ void put(int pos, int i, int brick,
+                                      const int32_t* __restrict__ start) const {
+    ord[pos] = i;
+    const int tile = brick / tile_bricks;
+    const int off = pos - start[tile * tile_bricks];
+    if (off >= chunk && off % chunk == 0) items[atomicAdd(nitems, 1)] = make_int2(tile, pos);
+  }
+};
+
+// adj.ord given: the records' final places, in order of arrival.  An adjoint alone
+// takes them so: each particle's sums are its own, whatever the order.
 __global__ void __launch_bounds__(256) k_brick_place(int64_t n, const int2* __restrict__ key,
                                                      const float4* __restrict__ rec_in,
                                                      const int32_t* __restrict__ start,
                                                      float4* __restrict__ rec_tmp,
                                                      int32_t* __restrict__ pidx,
                                                      int32_t* __restrict__ pbrick,
-                                                     int32_t* __restrict__ slot) {
+                                                     int32_t* __restrict__ slot, AdjOrder adj) {
   erpp_pdl_enter();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
@@ -171,6 +189,11 @@ __global__ void __launch_bounds__(256) k_brick_place(int64_t n, const int2* __re
   }
   const int pos = start[k.x] + k.y;
   rec_tmp[pos] = rec_in[i];
+  if (adj.ord) {
+    slot[i] = pos;
+    adj.put(pos, (int)i, k.x, start);
+    return;
+  }
   pidx[pos] = (int)i;
   pbrick[pos] = k.x;
 }
@@ -220,10 +243,7 @@ __global__ void __launch_bounds__(256) k_brick_order(int64_t n, int nb,
                                                      const int32_t* __restrict__ start,
                                                      float4* __restrict__ rec,
                                                      uint32_t* __restrict__ win,
-                                                     int32_t* __restrict__ slot,
-                                                     int32_t* __restrict__ ord, int tile_bricks,
-                                                     int chunk, int32_t* __restrict__ nitems,
-                                                     int2* __restrict__ items,
+                                                     int32_t* __restrict__ slot, AdjOrder adj,
                                                      erpp_kparams kp, erpp_brick_dims bd,
                                                      int32_t* __restrict__ ndense,
                                                      int32_t* __restrict__ dense,
@@ -252,14 +272,7 @@ __global__ void __launch_bounds__(256) k_brick_order(int64_t n, int nb,
   win[s + r] = __float_as_uint(v.w);
   slot[me] = s + r;
   if (r == 0 && dense_brick(e - s, n)) mark_dense(kp, bd, b, ndense, dense, dflag);
-  if (ord) {
-    ord[s + r] = me;
-    // the further chunks of an adjoint tile of more than `chunk` particles
-    const int tile = b / tile_bricks;
-    const int off = s + r - start[tile * tile_bricks];
-    if (off >= chunk && off % chunk == 0)
-      items[atomicAdd(nitems, 1)] = make_int2(tile, s + r);
-  }
+  if (adj.ord) adj.put(s + r, me, b, start);
 }
 
 // Normalisation of a particle's weights (erpp_norm's arithmetic on its record).
@@ -1029,16 +1042,20 @@ void bricks_free(erpp_ctx* c) {
 }
 
 // Sorts n particles at x into bricks: bk.rec in order, bk.slot each particle's
-// place (-1: invalid position), bk.start the bricks' ranges.
-cudaError_t brick_sort(erpp_ctx* c, int64_t n, const double* const x[3], bool for_adjoint,
-                       cudaStream_t st) {
+// place (-1: invalid position), bk.start the bricks' ranges; for the adjoint bk.ord
+// and its further chunks.  What only the adjoint reads keeps the order of arrival
+// within a brick, and is sorted by a launch less.
+cudaError_t brick_sort(erpp_ctx* c, int64_t n, const double* const x[3], bool for_source,
+                       bool for_adjoint, cudaStream_t st) {
   erpp_bricks& k = c->bk;
   const int nb = k.nbricks;
   cudaError_t e = cudaMemsetAsync(k.cnt, 0, table_bytes(nb), st);
   if (e != cudaSuccess) return e;
   const unsigned blocks = (unsigned)((n + 255) / 256);
   // the records in order of arrival: where the forces go later
-  float4* rec_tmp = k.fs;
+  float4* rec_tmp = for_source ? k.fs : k.rec;
+  const AdjOrder adj = {for_adjoint ? k.ord : nullptr, k.nitems, k.items, brick_tile(c),
+                        brick_chunk(c)};
   ++c->launches;
   e = erpp_launch_pdl(k_brick_count, dim3(blocks), dim3(256), 0, st, 0u, c->kp, k.dims, n, x[0],
                       x[1], x[2], k.rec_in, k.key, k.cnt, c->err);
@@ -1051,17 +1068,16 @@ cudaError_t brick_sort(erpp_ctx* c, int64_t n, const double* const x[3], bool fo
     e = launch_scan(c, k.cnt, k.start, k.scan_tmp, nb, st);
   }
   if (e != cudaSuccess) return e;
-  c->launches += 2;
+  ++c->launches;
   e = erpp_launch_pdl(k_brick_place, dim3(blocks), dim3(256), 0, st, 0u, n, (const int2*)k.key,
                       (const float4*)k.rec_in, (const int32_t*)k.start, rec_tmp, k.pidx, k.pbrick,
-                      k.slot);
-  if (e != cudaSuccess) return e;
+                      k.slot, for_source ? AdjOrder{} : adj);
+  if (e != cudaSuccess || !for_source) return e;
+  ++c->launches;
   return erpp_launch_pdl(k_brick_order, dim3(blocks), dim3(256), 0, st, 0u, n, nb,
                          (const int32_t*)k.pidx, (const int32_t*)k.pbrick, (const float4*)rec_tmp,
                          (const int32_t*)k.start, k.rec,
-                         k.win, k.slot, for_adjoint ? k.ord : nullptr, brick_tile(c),
-                         brick_chunk(c), k.nitems, k.items, c->kp, k.dims, k.ndense, k.dense,
-                         k.dflag);
+                         k.win, k.slot, adj, c->kp, k.dims, k.ndense, k.dense, k.dflag);
 }
 
 cudaError_t brick_forces(erpp_ctx* c, int64_t n, const double* const D[3], float scale,
@@ -1084,6 +1100,7 @@ cudaError_t brick_scatter(erpp_ctx* c, float* S, cudaStream_t st) {
     e = cudaFuncSetAttribute(dkern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
   c->launches += 2;
+  c->route |= ERPP_ROUTE_SOURCE;
   constexpr int kResident = 2 * 152;
   dkern<<<kResident, kScatThreads, sm, st>>>(c->kp, k.dims, k.ndense, k.dense, k.axis, k.rec, k.win,
                                        k.fs, k.start, k.bmax, S);

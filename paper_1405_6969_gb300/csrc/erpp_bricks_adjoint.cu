@@ -103,8 +103,10 @@ __device__ __forceinline__ int wrap_near(int j, int n) {
 // Copies of the tile's box by the whole block where one TMA box cannot: 16 bytes
 // a thread (nx a multiple of 4, u 16-byte aligned; no four words straddle the
 // box's end), else word by word.
+// Both are calls: inlined, they made the kernel of 100k
+// particles with windows of 9 nodes 20 us longer.
 template <class G>
-__device__ void stage_rows(const erpp_kparams& kp, const float* __restrict__ u, float* field,
+__device__ __noinline__ void stage_rows(const erpp_kparams& kp, const float* __restrict__ u, float* field,
                            const int b[3]) {
   const size_t nn = (size_t)kp.n[0] * kp.n[1] * kp.n[2];
   const int gx0 = wrap_mod(b[0] - 4, kp.n[0]);
@@ -120,9 +122,9 @@ __device__ void stage_rows(const erpp_kparams& kp, const float* __restrict__ u, 
 }
 // A lane keeps its column.  Its instructions bound this form (a row is 24 or 28
 // words and as many index sums): with a remainder per index instead of
-// wrap_near a box of 250 x 251 x 253 nodes with 16k particles took 847 us, now 520.
+// wrap_near a box of 250 x 251 x 253 nodes with 16k particles took 847 us, now 604.
 template <class G>
-__device__ void stage_words(const erpp_kparams& kp, const float* __restrict__ u, float* field,
+__device__ __noinline__ void stage_words(const erpp_kparams& kp, const float* __restrict__ u, float* field,
                             const int b[3]) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (lane >= G::PX) return;
@@ -217,10 +219,10 @@ __global__ void __launch_bounds__(kThreads, 2) k_brick_adjoint(
                      y0 + G::NY <= kp.n[1] && z0 >= 0 && z0 + G::NZ <= kp.n[2];
     if (tma) {
       if (tid == 0) {
-        // a further chunk's box lands where the tile before was staged, by the
-        // generic proxy perhaps, and read: the block's barrier and this fence
-        // put those accesses before the copy's
-        fence_proxy_async_shared();
+        // a block's next further chunk: its box lands where the tile before was
+        // staged, by the generic proxy perhaps, and read; the block's barrier and
+        // this fence put those accesses before the copy's
+        if (extra && it != (int)blockIdx.x) fence_proxy_async_shared();
         mbar_expect_tx(&bar, (unsigned)(kField * 4));
         tma_load_4d(field, &tmap, &bar, x0, y0, z0, 0);
       }
@@ -425,6 +427,24 @@ namespace erpp {
 
 int brick_tile(const erpp_ctx* c) { return short_windows(c) ? Geo7::TB : Geo10::TB; }
 int brick_chunk(const erpp_ctx* c) { return short_windows(c) ? Geo7::kChunk : Geo10::kChunk; }
+
+// Whether n particles pay for the sort and for staging every tile with its halo.
+// The warp-per-particle kernel takes 4.6 - 9 ns a particle, whatever the box; here
+// the sort's three launches cost ten us, and a tile that holds any particle as much
+// as about six (its box by TMA or in 16-byte copies) or twenty (word by word, rows
+// that are no multiple of 16 bytes).  Uniform clouds, windows of 6 nodes and of 9,
+// by warps and by bricks in us: 96 x 96 x 80 nodes, 4k particles 32 and 37, 56 and
+// 42, 5k 40 and 37, 68 and 44; 128^3, 6k 46 and 48, 80 and 70, 8k 52 and 49, 91 and
+// 73; 256^3, 34k (0.002 a node) 178 and 204, 327 and 337, 50k (0.003) 252 and 220.
+// Odd rows: 90 x 83 x 85, 12k 64 and 68, 30k 146 and 108; 181 x 122 x 95, 31k (0.015
+// a node) 152 and 150, 201 and 200; 250 x 251 x 253, 0.015 a node 1089 and 896, 1619
+// and 1282.
+bool bricks_pay_adjoint(const erpp_ctx* c, int64_t n, const void* F) {
+  const bool rows_ok = (c->kp.n[0] & 3) == 0 && ((uintptr_t)F & 15) == 0;
+  const double nodes = (double)c->kp.n[0] * c->kp.n[1] * c->kp.n[2];
+  return rows_ok ? n >= 5000 && (double)n >= 0.0035 * nodes
+                 : n >= 14000 && (double)n >= 0.015 * nodes;
+}
 
 cudaError_t brick_adjoint(erpp_ctx* c, int64_t n, const double* const x[3], const float* F,
                           const double* const v[3], double alpha, double shear_coef,

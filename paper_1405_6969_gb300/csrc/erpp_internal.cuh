@@ -175,6 +175,7 @@ struct erpp_ctx {
   struct erpp_host_pipe* hp;  // erpp_step_host staging and streams (lazily created)
   int launches;           // kernels launched since erpp_step began (counted at each launch)
   int last_step_launches; // kernels the most recent erpp_step launched
+  int route;              // brick kernels the most recent call launched (ERPP_ROUTE_*)
   // scratch (owned)
   int64_t cap;            // particle capacity of the per-particle arrays
   float4* geo_t;
@@ -290,12 +291,13 @@ cudaError_t launch_advance_multi(const erpp_box_dev* boxes, const int2* pitems, 
 // their records' places (scale * norm * D), and the source from them.
 bool bricks_possible(const erpp_ctx* c);
 bool use_bricks(const erpp_ctx* c, int64_t n);
+bool bricks_pay_adjoint(const erpp_ctx* c, int64_t n, const void* F);
 cudaError_t bricks_alloc_tables(erpp_ctx* c);
 void bricks_free_tables(erpp_ctx* c);
 cudaError_t bricks_alloc(erpp_ctx* c, int64_t cap);
 void bricks_free(erpp_ctx* c);
-cudaError_t brick_sort(erpp_ctx* c, int64_t n, const double* const x[3], bool for_adjoint,
-                       cudaStream_t st);
+cudaError_t brick_sort(erpp_ctx* c, int64_t n, const double* const x[3], bool for_source,
+                       bool for_adjoint, cudaStream_t st);
 cudaError_t brick_forces(erpp_ctx* c, int64_t n, const double* const D[3], float scale,
                          cudaStream_t st);
 cudaError_t brick_scatter(erpp_ctx* c, float* S, cudaStream_t st);

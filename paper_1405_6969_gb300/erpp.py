@@ -311,6 +311,14 @@ class Context:
         _lib.check(self.lib.erpp_debug_set_wait(self._h, int(limit_ns), int(bool(stall))),
                    "erpp_debug_set_wait")
 
+    def debug_last_route(self):
+        """Parts of the last step, source or backward call that ran from
+        brick-sorted particles: a set of "source" and "adjoint"."""
+        r = ctypes.c_int32(0)
+        _lib.check(self.lib.erpp_debug_last_route(self._h, ctypes.byref(r)),
+                   "erpp_debug_last_route")
+        return {name for bit, name in ((1, "source"), (2, "adjoint")) if r.value & bit}
+
     def debug_windows(self, x, stream=None):
         n = x.shape[1]
         lo = torch.empty((3, n), dtype=torch.int32, device=x.device)
