@@ -28,6 +28,11 @@
  *   Streams: every call is asynchronous on the given CUDA stream (NULL = the
  *     legacy default stream) unless stated otherwise.  Calls that share one
  *     context share its scratch: issue them on one stream, in order.
+ *   Scratch: per-particle scratch is allocated (synchronously) by the first
+ *     call that needs it and remade by a call with more particles, after
+ *     which a captured graph of the context's calls with fewer is void.  The
+ *     backward calls do not remake it (erpp_gather_backward: for dx alone),
+ *     and what they sort stays in place for the graphs that hold it.
  *   Errors: argument errors are reported synchronously by the return value
  *     and nothing is launched.  Data errors found on the device (NaN or
  *     out-of-box positions) set a sticky device error word that

@@ -43,7 +43,6 @@ erpp_status set_cuda_err(cudaError_t e) {
 }
 
 void free_scratch(erpp_ctx* c) {
-  erpp::bricks_free(c);
   cudaFree(c->geo_t);
   cudaFree(c->geo_c);
   cudaFree(c->xw);
@@ -137,7 +136,6 @@ erpp_status ensure_capacity(erpp_ctx* c, int64_t n) {
     if (e == cudaSuccess && c->kp.design == 4)
       e = cudaMalloc(&c->gather_items, sizeof(int2) * (size_t)(ecap / ERPP_GATHER_CHUNK + 1));
     c->entries_cap = ecap;
-    if (e == cudaSuccess) e = bricks_alloc(c, cap);
   }
   if (e != cudaSuccess) {
     free_scratch(c);
@@ -174,6 +172,7 @@ void free_tile_tables(erpp_ctx* c) {
   cudaFree(c->halo);
   c->tile_cnt = c->tile_start = c->scan_tmp = nullptr;
   c->halo = nullptr;
+  erpp::bricks_free(c);
   erpp::bricks_free_tables(c);
 }
 
@@ -192,21 +191,9 @@ erpp_status alloc_weight_tables(erpp_ctx* c) {
   return set_cuda_err(e);
 }
 
-// Whether an adjoint, which needs no scratch otherwise, takes the brick kernels:
-// where their scratch is there, or can be made without losing a step history
-// and outside a stream capture.
+// Whether an adjoint takes the brick kernels.
 bool adjoint_bricks(erpp_ctx* c, int64_t n, const void* F, cudaStream_t st) {
-  if (c->fp64 || !erpp::bricks_possible(c) || !erpp::bricks_pay_adjoint(c, n, F)) return false;
-  if (n > c->cap) {
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (c->kp.lag > 0 || c->kp.full_force ||
-        cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone ||
-        erpp::ensure_capacity(c, n) != ERPP_OK) {
-      cudaGetLastError();
-      return false;
-    }
-  }
-  if (!erpp::use_bricks(c, n)) return false;
+  if (c->fp64 || !erpp::bricks_pay_adjoint(c, n, F) || !erpp::bricks_ready(c, n, st)) return false;
   c->route |= ERPP_ROUTE_ADJOINT;
   return true;
 }
@@ -641,7 +628,7 @@ erpp_status erpp_gather_backward(erpp_ctx* c, int64_t n, const double* const x[3
   const bool adj = dx && adjoint_bricks(c, n, u, st);
   bool sorted = false;  // for the source too
   if (adj) {
-    sorted = du && erpp::use_bricks(c, n);
+    sorted = du != nullptr;
     e = erpp::brick_sort(c, n, x, sorted, true, st);
   }
   if (e == cudaSuccess && dx && n > 0)
@@ -654,7 +641,7 @@ erpp_status erpp_gather_backward(erpp_ctx* c, int64_t n, const double* const x[3
     if (s) return s;
     if (c->fp64) {
       e = erpp::launch_scatter_f64(c, n, x, g, c->kp.dV, (double*)du, false, st);
-    } else if (erpp::use_bricks(c, n)) {
+    } else if (sorted || erpp::bricks_ready(c, n, st)) {
       if (!sorted) e = erpp::brick_sort(c, n, x, true, false, st);
       if (e == cudaSuccess) e = erpp::brick_forces(c, n, g, 1.0f, st);
       if (e == cudaSuccess) e = erpp::brick_scatter(c, (float*)du, st);
@@ -692,7 +679,7 @@ cudaError_t scatter_source(erpp_ctx* c, int64_t n, const double* const x[3],
   if (c->fp64)
     return erpp::launch_scatter_f64(c, n, x, D, -1.0 / c->params.rho_f, (double*)S, false, st);
   cudaError_t e;
-  if (use_bricks(c, n)) {
+  if (bricks_ready(c, n, st)) {
     e = brick_sort(c, n, x, true, false, st);
     if (e == cudaSuccess) e = brick_forces(c, n, D, -c->kp.inv_rho_dV, st);
     if (e == cudaSuccess) e = brick_scatter(c, (float*)S, st);
@@ -803,7 +790,7 @@ erpp_status step_full_force(erpp_ctx* c, const void* u, const erpp_particles* P,
   }
   if (e == cudaSuccess) e = erpp::launch_advance_full(c, P, upc, first_step, st);
   if (e == cudaSuccess && after_advance) e = cudaEventRecord(after_advance, st);
-  if (e == cudaSuccess && tiles && !use_bricks(c, n)) {
+  if (e == cudaSuccess && tiles && !bricks_ready(c, n, st)) {
     e = erpp::launch_prep_fscat(c, n, Dv, -c->kp.inv_rho_dV, st);
     if (e == cudaSuccess) e = erpp::launch_scatter_f32(c, (float*)S, st);
   } else if (e == cudaSuccess) {
@@ -854,7 +841,7 @@ erpp_status step_device(erpp_ctx* c, const void* u, const erpp_particles* P, voi
     cudaEvent_t* ev = nullptr;
     if (c->prof_on) ev = c->prof_ev + 5 * (c->prof_n++ % kProfSets);
     if (ev) cudaEventRecord(ev[0], st);
-    const bool bricks = use_bricks(c, n);
+    const bool bricks = bricks_ready(c, n, st);
     e = bricks ? brick_sort(c, n, xin, true, false, st) : cudaSuccess;
     if (e == cudaSuccess) e = erpp::bin_particles(c, n, xin, true, st);
     if (ev) cudaEventRecord(ev[1], st);

@@ -181,6 +181,7 @@ erpp_status erpp_batch_init(int32_t nbox, const erpp_box_desc* boxes, erpp_batch
     // scratch for the box's particles now: no allocation may happen while
     // the step is being captured
     if (s == ERPP_OK) s = erpp::ensure_capacity(b->ctx[i], b->boxes[i].particles.n);
+    if (s == ERPP_OK) erpp::bricks_reserve(b->ctx[i], b->boxes[i].particles.n);
   }
   cudaError_t e = cudaSuccess;
   if (s == ERPP_OK) e = cudaStreamCreateWithFlags(&b->origin, cudaStreamNonBlocking);
@@ -228,6 +229,7 @@ erpp_status erpp_batch_set_tiling(erpp_batch* b, int32_t box, int32_t tile_y, in
   // scratch again now (never during a capture), and the graphs hold the old
   // launch configuration
   if (s == ERPP_OK) s = erpp::ensure_capacity(b->ctx[box], b->boxes[box].particles.n);
+  if (s == ERPP_OK) erpp::bricks_reserve(b->ctx[box], b->boxes[box].particles.n);
   for (int k = 0; k < 2; ++k) {
     if (b->exec[k]) cudaGraphExecDestroy(b->exec[k]);
     b->exec[k] = nullptr;

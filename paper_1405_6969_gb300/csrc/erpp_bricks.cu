@@ -33,6 +33,7 @@
 // underflow.  The dropped l l' is below 2^-24 of its term.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
+#include <stdlib.h>
 
 #include <algorithm>
 #include <type_traits>
@@ -932,7 +933,7 @@ namespace erpp {
 // Whether the context's windows and options allow the brick kernels (windows
 // of at most 10 nodes that start at most 4 below the cell: the record's
 // fields; FP32, Gaussian source).
-bool bricks_possible(const erpp_ctx* c) {
+static bool bricks_possible(const erpp_ctx* c) {
   return !c->fp64 && c->kp.design == 4 && c->kp.weights != ERPP_W_PIC && !c->kp.kahan &&
          c->kp.xs <= 10 && c->kp.hlo <= 4;
 }
@@ -945,8 +946,8 @@ bool bricks_possible(const erpp_ctx* c) {
 // regions, 20k (80^3) 36 and 46; 180, 20k (96 x 96 x 80) 32 and 43; 512, 30k
 // (128^3) 38 and 53 us.
 constexpr int64_t kRegionsLeast = 120;
-bool use_bricks(const erpp_ctx* c, int64_t n) {
-  if (!c->bk.rec || c->scatter_mode != ERPP_SCATTER_MERGE || n <= 0) return false;
+static bool bricks_serve(const erpp_ctx* c, int64_t n) {
+  if (!c->bk.cnt || c->scatter_mode != ERPP_SCATTER_MERGE || n <= 0) return false;
   const int64_t regions = c->bk.nbricks / 8;
   const double nodes = (double)c->kp.n[0] * c->kp.n[1] * c->kp.n[2];
   return regions >= kRegionsLeast || (n >= 16384 && (double)n >= 0.25 * nodes);
@@ -1000,45 +1001,106 @@ void bricks_free_tables(erpp_ctx* c) {
   k.cnt = k.start = k.scan_tmp = k.bmax = k.nitems = nullptr;
 }
 
-cudaError_t bricks_alloc(erpp_ctx* c, int64_t cap) {
+bool stream_captures(cudaStream_t st) {
+  cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &s) == cudaSuccess) return s != cudaStreamCaptureStatusNone;
+  cudaGetLastError();
+  return true;
+}
+
+}  // namespace erpp
+
+// A former block: kept until the context's scratch goes, for the graphs that were
+// captured with it.
+struct erpp_brick_block {
+  unsigned char* block;
+  erpp_brick_block* next;
+};
+
+namespace erpp {
+
+// The per-particle arrays for n particles, apart from the context's other scratch:
+// made by the first call that sorts into bricks (76 bytes a particle, which a
+// context that interpolates only, or in another halo mode, has no use for), so that
+// an adjoint, which needs no scratch otherwise, leaves the other calls' alone.
+// Where there is no memory for them the calls take the kernels that need none.
+// Arrays that a capture has recorded stay in place when larger ones are made, of at
+// least twice the size, so that all former ones together are no larger.
+bool bricks_reserve(erpp_ctx* c, int64_t n) {
   erpp_bricks& k = c->bk;
-  if (!k.cnt) return cudaSuccess;
+  if (!bricks_serve(c, n)) return false;
+  if (n <= k.cap) return true;
+  if (k.refused > 0 && n >= k.refused) return false;
+  erpp_brick_block* former = nullptr;
+  size_t cap = (size_t)std::max<int64_t>(n, 1024);
+  if (k.captured) {
+    cap = std::max(cap, 2 * (size_t)k.cap);
+    former = static_cast<erpp_brick_block*>(malloc(sizeof(erpp_brick_block)));
+    if (!former) return false;
+  } else {
+    cudaFree(k.block);
+    k.block = nullptr;
+    k.cap = 0;
+  }
   // one allocation: eleven of their own made a context's first call on 1M
   // particles 0.3 ms longer
-  const size_t n = (size_t)cap;
+  unsigned char* block = nullptr;
   size_t at = 0;
   auto place = [&](auto*& p, size_t count) {
-    if (k.block) p = reinterpret_cast<std::remove_reference_t<decltype(p)>>(k.block + at);
+    if (block) p = reinterpret_cast<std::remove_reference_t<decltype(p)>>(block + at);
     at += (count * sizeof(*p) + 255) & ~(size_t)255;
   };
   for (int pass = 0; pass < 2; ++pass) {
     at = 0;
-    place(k.rec, n);
-    place(k.rec_in, n);
-    place(k.fs, n);
-    place(k.key, n);
-    place(k.items, n / brick_chunk(c) + 1);
-    place(k.pidx, n);
-    place(k.pbrick, n);
-    place(k.slot, n);
-    place(k.ord, n);
-    place(k.win, n);
+    place(k.rec, cap);
+    place(k.rec_in, cap);
+    place(k.fs, cap);
+    place(k.key, cap);
+    place(k.items, cap / brick_chunk(c) + 1);
+    place(k.pidx, cap);
+    place(k.pbrick, cap);
+    place(k.slot, cap);
+    place(k.ord, cap);
+    place(k.win, cap);
     if (pass == 1) break;
-    cudaError_t e = cudaMalloc(&k.block, at);
-    if (e != cudaSuccess) return e;
+    if (cudaMalloc(&block, at) != cudaSuccess) {
+      cudaGetLastError();
+      free(former);
+      k.refused = n;
+      return false;
+    }
   }
-  return cudaSuccess;
+  if (former) {
+    former->block = k.block;
+    former->next = k.retired;
+    k.retired = former;
+    k.captured = false;
+  }
+  k.block = block;
+  k.cap = (int64_t)cap;
+  return true;
+}
+
+bool bricks_ready(erpp_ctx* c, int64_t n, cudaStream_t st) {
+  if (!bricks_serve(c, n)) return false;
+  const bool recorded = stream_captures(st);
+  if (n > c->bk.cap && (recorded || !bricks_reserve(c, n))) return false;
+  c->bk.captured |= recorded;
+  return true;
 }
 
 void bricks_free(erpp_ctx* c) {
   erpp_bricks& k = c->bk;
   cudaFree(k.block);
+  while (k.retired) {
+    erpp_brick_block* r = k.retired;
+    k.retired = r->next;
+    cudaFree(r->block);
+    free(r);
+  }
   k.block = nullptr;
-  k.items = nullptr;
-  k.win = nullptr;
-  k.key = nullptr;
-  k.pidx = k.pbrick = k.slot = k.ord = nullptr;
-  k.rec_in = k.fs = k.rec = nullptr;
+  k.cap = k.refused = 0;
+  k.captured = false;
 }
 
 // Sorts n particles at x into bricks: bk.rec in order, bk.slot each particle's

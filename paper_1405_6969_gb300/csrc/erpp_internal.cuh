@@ -142,6 +142,10 @@ struct erpp_bricks {
   int32_t* start;   // [nbricks + 1]
   int32_t* scan_tmp;
   int2* axis;       // per axis and group: the stretches of bricks around it
+  int64_t cap;      // particles that the arrays below hold
+  int64_t refused;  // particles that there was no memory for (0: none)
+  bool captured;    // a stream capture has recorded the arrays' addresses
+  struct erpp_brick_block* retired;  // former blocks that a captured graph may still use
   unsigned char* block;  // the allocation that holds the arrays below, but for the tables
   int2* key;        // [cap] per particle: brick (-1: invalid position), place by arrival
   int32_t* pidx;    // [cap] in order of arrival: particle
@@ -287,14 +291,16 @@ cudaError_t launch_bin_multi(const erpp_box_dev* boxes, int nbox, const int2* pi
 cudaError_t launch_advance_multi(const erpp_box_dev* boxes, const int2* pitems, int npitems,
                                  int first_step, cudaStream_t st);
 
-// Particles sorted by brick (erpp_bricks.cu): scratch, the sort, the forces at
-// their records' places (scale * norm * D), and the source from them.
-bool bricks_possible(const erpp_ctx* c);
-bool use_bricks(const erpp_ctx* c, int64_t n);
+// Particles sorted by brick (erpp_bricks.cu): whether they serve a call on n
+// particles, with the scratch made then (bricks_ready; no allocation during a
+// capture of st) or before (bricks_reserve); the sort, the forces at their records'
+// places (scale * norm * D), and the source from them.
+bool bricks_ready(erpp_ctx* c, int64_t n, cudaStream_t st);
+bool bricks_reserve(erpp_ctx* c, int64_t n);
+bool stream_captures(cudaStream_t st);
 bool bricks_pay_adjoint(const erpp_ctx* c, int64_t n, const void* F);
 cudaError_t bricks_alloc_tables(erpp_ctx* c);
 void bricks_free_tables(erpp_ctx* c);
-cudaError_t bricks_alloc(erpp_ctx* c, int64_t cap);
 void bricks_free(erpp_ctx* c);
 cudaError_t brick_sort(erpp_ctx* c, int64_t n, const double* const x[3], bool for_source,
                        bool for_adjoint, cudaStream_t st);
