@@ -63,6 +63,7 @@ void free_scratch(erpp_ctx* c) {
   cudaFree(c->up64);
   cudaFree(c->w64);
   c->w64 = nullptr;
+  c->w64_refused = false;
   cudaFree(c->w_key);
   cudaFree(c->w_slot);
   cudaFree(c->w_perm);
@@ -101,9 +102,6 @@ erpp_status ensure_capacity(erpp_ctx* c, int64_t n) {
   cudaError_t e = cudaSuccess;
   if (c->fp64 || c->kp.weights != ERPP_W_GAUSS)
     e = cudaMalloc(&c->up64, sizeof(double) * 3 * (size_t)cap);
-  if (c->fp64 && c->kp.weights == ERPP_W_GAUSS && !c->kp.full_force && c->kp.lag == 0 &&
-      e == cudaSuccess)
-    e = cudaMalloc(&c->w64, w64_bytes(c->kp, cap));
   if (c->kp.full_force && e == cudaSuccess) {
     e = cudaMalloc(&c->ff_lap, sizeof(double) * 3 * (size_t)cap);
     if (e == cudaSuccess) e = cudaMalloc(&c->ff_prev, sizeof(double) * 6 * (size_t)cap);
@@ -142,6 +140,16 @@ erpp_status ensure_capacity(erpp_ctx* c, int64_t n) {
     return set_cuda_err(e);
   }
   c->cap = cap;
+  return ERPP_OK;
+}
+
+erpp_status step_reserve(erpp_ctx* c, int64_t n) {
+  erpp_status s = ensure_capacity(c, n);
+  if (s != ERPP_OK) return s;
+  if (c->fp64)
+    w64_reserve(c);
+  else
+    bricks_reserve(c, n);
   return ERPP_OK;
 }
 
@@ -831,12 +839,13 @@ erpp_status step_device(erpp_ctx* c, const void* u, const erpp_particles* P, voi
     }
   } else if (c->fp64) {
     double* up[3] = {c->up64, c->up64 + c->cap, c->up64 + 2 * c->cap};
-    e = erpp::launch_gather_f64(c, (const double*)u, n, xin, up, true, st);
+    const bool keep = w64_ready(c, st);
+    e = erpp::launch_gather_f64(c, (const double*)u, n, xin, up, keep, st);
     const double* const upc[3] = {up[0], up[1], up[2]};
     if (e == cudaSuccess) e = erpp::launch_advance(c, P, upc, false, false, first_step, st);
     if (e == cudaSuccess && after_advance) e = cudaEventRecord(after_advance, st);
     if (e == cudaSuccess)
-      e = erpp::launch_scatter_f64(c, n, xprev, Dv, -1.0 / c->params.rho_f, (double*)S, true, st);
+      e = erpp::launch_scatter_f64(c, n, xprev, Dv, -1.0 / c->params.rho_f, (double*)S, keep, st);
   } else {
     cudaEvent_t* ev = nullptr;
     if (c->prof_on) ev = c->prof_ev + 5 * (c->prof_n++ % kProfSets);

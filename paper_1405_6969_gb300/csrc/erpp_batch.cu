@@ -180,8 +180,7 @@ erpp_status erpp_batch_init(int32_t nbox, const erpp_box_desc* boxes, erpp_batch
     s = erpp_init(&b->boxes[i].params, &b->ctx[i]);
     // scratch for the box's particles now: no allocation may happen while
     // the step is being captured
-    if (s == ERPP_OK) s = erpp::ensure_capacity(b->ctx[i], b->boxes[i].particles.n);
-    if (s == ERPP_OK) erpp::bricks_reserve(b->ctx[i], b->boxes[i].particles.n);
+    if (s == ERPP_OK) s = erpp::step_reserve(b->ctx[i], b->boxes[i].particles.n);
   }
   cudaError_t e = cudaSuccess;
   if (s == ERPP_OK) e = cudaStreamCreateWithFlags(&b->origin, cudaStreamNonBlocking);
@@ -228,8 +227,7 @@ erpp_status erpp_batch_set_tiling(erpp_batch* b, int32_t box, int32_t tile_y, in
   erpp_status s = erpp_set_tiling(b->ctx[box], tile_y, tile_z, threads);
   // scratch again now (never during a capture), and the graphs hold the old
   // launch configuration
-  if (s == ERPP_OK) s = erpp::ensure_capacity(b->ctx[box], b->boxes[box].particles.n);
-  if (s == ERPP_OK) erpp::bricks_reserve(b->ctx[box], b->boxes[box].particles.n);
+  if (s == ERPP_OK) s = erpp::step_reserve(b->ctx[box], b->boxes[box].particles.n);
   for (int k = 0; k < 2; ++k) {
     if (b->exec[k]) cudaGraphExecDestroy(b->exec[k]);
     b->exec[k] = nullptr;

@@ -548,8 +548,23 @@ cudaError_t launch_gather_f64(erpp_ctx* ctx, const double* u, int64_t n,
   return cudaGetLastError();
 }
 
-size_t w64_bytes(const erpp_kparams& kp, int64_t cap) {
-  return sizeof(double) * kept_doubles(kp.xs) * (size_t)((cap + kPlainP - 1) / kPlainP);
+// The step's weights (24 (xs + 1) bytes a particle) are kept where there is memory
+// for them, made by the first step outside a capture; the source evaluates its own
+// otherwise, with the same values.
+bool w64_reserve(erpp_ctx* ctx) {
+  if (ctx->w64) return true;
+  if (ctx->w64_refused || ctx->cap <= 0) return false;
+  const size_t blocks = (size_t)((ctx->cap + kPlainP - 1) / kPlainP);
+  if (cudaMalloc(&ctx->w64, sizeof(double) * kept_doubles(ctx->kp.xs) * blocks) != cudaSuccess) {
+    cudaGetLastError();
+    ctx->w64 = nullptr;
+    ctx->w64_refused = true;
+  }
+  return ctx->w64 != nullptr;
+}
+
+bool w64_ready(erpp_ctx* ctx, cudaStream_t st) {
+  return ctx->w64 || (!stream_captures(st) && w64_reserve(ctx));
 }
 
 cudaError_t launch_scatter_f64(erpp_ctx* ctx, int64_t n, const double* const x[3],

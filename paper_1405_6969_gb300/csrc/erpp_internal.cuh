@@ -195,7 +195,8 @@ struct erpp_ctx {
   float4* up_part;        // [entries_cap] x/y-halo tiles: each piece's gathered sums,
                           // at its place in the piece records
   float4* fscat;
-  double* w64;            // FP64 step: the gather's weights, for the source
+  double* w64;            // FP64 step: the gather's weights, for the source [cap]
+  bool w64_refused;       // there was no memory for it
   double* up64;           // FP64 mode or other weights: gathered velocity [3][cap]
   int32_t* w_key;         // other weights: sort key, place and order of each particle [cap]
   int32_t* w_slot;
@@ -320,6 +321,8 @@ bool field_box_map(const erpp_kparams& kp, const float* u, const int box[3], voi
 
 erpp_status derive_ctx(const erpp_params* p, erpp_ctx* c);
 erpp_status ensure_capacity(erpp_ctx* c, int64_t n);  // may allocate (synchronous)
+// All scratch of the plain step for n particles now, before a capture.
+erpp_status step_reserve(erpp_ctx* c, int64_t n);
 int xw_len(const erpp_kparams& kp);
 inline int nbins(const erpp_kparams& kp) { return kp.design == 4 ? kp.ntiles : kp.ntiles * 32; }
 // The coupling step of erpp_step (arguments already checked); records
@@ -391,7 +394,8 @@ cudaError_t launch_gather_f64(erpp_ctx* ctx, const double* u, int64_t n,
 cudaError_t launch_scatter_f64(erpp_ctx* ctx, int64_t n, const double* const x[3],
                                const double* const D[3], double fscale, double* S, bool kept,
                                cudaStream_t st);  // kept: w64 holds the weights at x
-size_t w64_bytes(const erpp_kparams& kp, int64_t cap);
+bool w64_reserve(erpp_ctx* ctx);                  // w64 is there, or made now
+bool w64_ready(erpp_ctx* ctx, cudaStream_t st);   // the same outside a capture of st
 // Per particle: outv = alpha sum_j F_j W (if outv), outx = alpha sum_j (F_j . v)
 // dW/dx + shear_coef v_x on y.
 cudaError_t launch_adjoint(erpp_ctx* ctx, int64_t n, const double* const x[3], const void* F,

@@ -1,5 +1,5 @@
-"""Scratch of the brick kernels: made by the calls that use it, and left where
-captured graphs expect it.
+"""Scratch of the brick kernels and of the FP64 step: made by the calls that use
+it, and left where captured graphs expect it.
 
 Replays are compared bit for bit with the same call issued directly.
 """
@@ -166,3 +166,37 @@ def test_capture_without_it(erpp):
     assert ctx.debug_last_route() == {"source"}
     ctx.check()
     assert float((S - T).norm() / T.norm()) < 1e-5
+
+
+def test_fp64_step_keeps_weights_only(erpp, oracle_lib):
+    """An FP64 context that interpolates or forms sources holds the gathered
+    velocity alone (24 bytes a particle); the first step makes the array of the
+    weights (24 (xs + 1), xs = 7 here), and a step captured before that does
+    without it, with the same results."""
+    import torch
+    particles = 400_000
+    x, D = cloud(particles, 5)
+    u = torch.zeros((3,) + N[::-1], device="cuda", dtype=torch.float64)
+    S, up = torch.empty_like(u), torch.empty_like(x)
+    ctx = erpp.Context(box().params(), precision="fp64")
+    start = free_bytes()
+    ctx.interpolate(u, x, out=up)
+    ctx.scatter_source(x, D, S=S)
+    assert start - free_bytes() < 40 * particles
+    one = torch.ones(particles, device="cuda", dtype=torch.float64)
+    state = lambda: erpp.ParticleState(x.clone(), 0.01 * D, x.clone(), 1e-3 * D,  # noqa: E731
+                                       0.01 * one, 1000 * one)
+    P = state()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        ctx.step(u, P, S=S)
+    graph.replay()
+    start = free_bytes()
+    Q, T = state(), torch.empty_like(u)
+    start = free_bytes()
+    ctx.step(u, Q, S=T)
+    assert start - free_bytes() > 180 * particles
+    ctx.check()
+    assert torch.equal(P.D, Q.D) and torch.equal(P.v, Q.v) and torch.equal(P.x, Q.x)
+    assert float((S - T).norm() / T.norm()) < 1e-12  # atomics: the order of additions
