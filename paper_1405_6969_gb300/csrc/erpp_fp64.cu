@@ -55,46 +55,114 @@ __device__ int axis_weights_f64(const erpp_kparams& kp, int a, double x, double*
   return nw;
 }
 
-// Particles of a block of the plain kernels.
-constexpr int kPlainP = 32;
-constexpr int kPlainS = kPlainP + 1;  // stride of a weight's particles
+// Particles of a block of the plain kernels: 32, or 8 where there are few (plain_few).
+constexpr int kPlainMany = 32, kPlainFew = 8;
 
-// Doubles that keep a block's weights and windows between the gather and the
-// source of one step.
-__host__ __device__ constexpr size_t kept_doubles(int xs) { return (size_t)3 * (xs + 1) * kPlainP; }
+// Doubles that keep the weights and windows of a block of P particles between the
+// gather and the source of one step.
+__host__ __device__ constexpr size_t kept_doubles(int xs, int P) { return (size_t)3 * (xs + 1) * P; }
 
-// The weights of a block's particles into shared memory, a thread per particle
-// and axis: w[axis][k][particle], window starts and lengths beside (length 0:
-// invalid).
+// A block's particles: window starts and lengths per axis (length 0: invalid); where
+// they are few, the positions in units of the spacing and the weights' scales.  The
+// weights are w[axis][k][particle], P + 1 apart in k.
+template <int P>
+struct Plain {
+  int jlo[3][P], nw[3][P];
+  double s[3][P], scale[3][P];
+};
+
+// The weights of a block's particles, called by the whole block (it ends behind a
+// barrier).  Many particles: a thread evaluates an axis of a particle.  Few: the
+// exponentials by a thread each, between barriers, for a block would wait for xs of
+// them one after the other; the same products and sums in the same order.
+template <int P>
 __device__ __forceinline__ void plain_weights(const erpp_kparams& kp, int64_t p0, int np,
                                               const double* __restrict__ x0,
                                               const double* __restrict__ x1,
                                               const double* __restrict__ x2, double* w,
-                                              int (*jlo)[kPlainP], int (*nw)[kPlainP],
-                                              const double* __restrict__ kept, uint32_t* err) {
+                                              Plain<P>& sh, const double* __restrict__ kept,
+                                              uint32_t* err) {
+  constexpr int kS = P + 1;
   if (kept) {
     // evaluated by the step's gather at the same positions
-    const double* src = kept + (size_t)blockIdx.x * kept_doubles(kp.xs);
-    for (int i = threadIdx.x; i < 3 * kp.xs * kPlainP; i += blockDim.x)
-      w[(i / kPlainP) * kPlainS + (i & (kPlainP - 1))] = src[i];
-    const int2* win = reinterpret_cast<const int2*>(src + 3 * kp.xs * kPlainP);
-    for (int i = threadIdx.x; i < 3 * kPlainP; i += blockDim.x) {
-      const int a = i / kPlainP, p = i & (kPlainP - 1);
+    const double* src = kept + (size_t)blockIdx.x * kept_doubles(kp.xs, P);
+    for (int i = threadIdx.x; i < 3 * kp.xs * P; i += blockDim.x)
+      w[(i / P) * kS + (i & (P - 1))] = src[i];
+    const int2* win = reinterpret_cast<const int2*>(src + 3 * kp.xs * P);
+    for (int i = threadIdx.x; i < 3 * P; i += blockDim.x) {
+      const int a = i / P, p = i & (P - 1);
       const int2 v = win[i];
-      jlo[a][p] = v.x;
-      nw[a][p] = v.y;
+      sh.jlo[a][p] = v.x;
+      sh.nw[a][p] = v.y;
     }
+    __syncthreads();
     return;
   }
-  for (int i = threadIdx.x; i < 3 * kPlainP; i += blockDim.x) {
-    const int a = i / kPlainP, p = i & (kPlainP - 1);
-    if (p >= np) continue;
-    const double x = a == 0 ? x0[p0 + p] : (a == 1 ? x1[p0 + p] : x2[p0 + p]);
-    int lo = 0;
-    nw[a][p] =
-        axis_weights_f64(kp, a, x, w + a * kp.xs * kPlainS + p, kPlainS, &lo, err);
-    jlo[a][p] = lo;
+  if (P == kPlainMany) {
+    for (int i = threadIdx.x; i < 3 * P; i += blockDim.x) {
+      const int a = i / P, p = i & (P - 1);
+      if (p >= np) continue;
+      const double x = a == 0 ? x0[p0 + p] : (a == 1 ? x1[p0 + p] : x2[p0 + p]);
+      int lo = 0;
+      sh.nw[a][p] = axis_weights_f64(kp, a, x, w + a * kp.xs * kS + p, kS, &lo, err);
+      sh.jlo[a][p] = lo;
+    }
+    __syncthreads();
+    return;
   }
+  for (int i = threadIdx.x; i < 3 * P; i += blockDim.x) {
+    const int a = i / P, p = i & (P - 1);
+    int lo = 0, nw = 0;
+    double s = 0.0;
+    if (p < np) {
+      const double x = a == 0 ? x0[p0 + p] : (a == 1 ? x1[p0 + p] : x2[p0 + p]);
+      if (!(x >= 0.0 && x < kp.L[a])) {
+        erpp_set_err(err, ERPP_ERRBIT_RANGE);
+      } else {
+        const erpp_axis_win aw =
+            erpp_axis_window_lean(x, kp.inv_dx[a], kp.cp[a], kp.cp_int[a], kp.cp_frac[a]);
+        lo = aw.lo;
+        nw = aw.hi - aw.lo + 1;
+        if (nw > kp.xs || nw < 1) {
+          erpp_set_err(err, ERPP_ERRBIT_BOUNDS);
+          nw = 0;
+        }
+        s = __dmul_rn(x, kp.inv_dx[a]);
+      }
+    }
+    sh.jlo[a][p] = lo;
+    sh.nw[a][p] = nw;
+    sh.s[a][p] = s;
+  }
+  __syncthreads();
+  const int all = 3 * kp.xs * P;
+  for (int i = threadIdx.x; i < all; i += blockDim.x) {
+    const int r = i / P, p = i & (P - 1);
+    const int a = r >= 2 * kp.xs ? 2 : (r >= kp.xs ? 1 : 0), k = r - a * kp.xs;
+    if (k >= sh.nw[a][p]) continue;
+    const double d = ((double)(sh.jlo[a][p] + k) - sh.s[a][p]) * kp.dx[a];
+    const double q = d * d;
+    // -q / (2 sigma_R^2) by the reciprocal's high and low parts
+    w[r * kS + p] = exp(fma(q, kp.gauss_hi, q * kp.gauss_lo));
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < 3 * P; i += blockDim.x) {
+    const int a = i / P, p = i & (P - 1);
+    double scale = kp.raw_norm1;
+    if (kp.normalize) {
+      double sum = 0.0;
+      for (int k = 0; k < sh.nw[a][p]; ++k) sum += w[(a * kp.xs + k) * kS + p];
+      scale = 1.0 / (kp.dx[a] * sum);
+    }
+    sh.scale[a][p] = scale;
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < all; i += blockDim.x) {
+    const int r = i / P, p = i & (P - 1);
+    const int a = r >= 2 * kp.xs ? 2 : (r >= kp.xs ? 1 : 0);
+    if (r - a * kp.xs < sh.nw[a][p]) w[r * kS + p] *= sh.scale[a][p];
+  }
+  __syncthreads();
 }
 
 __device__ __forceinline__ int wrap_idx(int j, int n) {
@@ -105,10 +173,12 @@ __device__ __forceinline__ int wrap_idx(int j, int n) {
 // row and 32 / nwx rows at a time; wyz[] holds the products of the rows'
 // weights (written here), f(lane's weight e_x, row weight, node) sees every node
 // of the window once.
-template <typename F>
+template <int P, typename F>
 __device__ __forceinline__ void plain_walk(const erpp_kparams& kp, const double* w,
-                                           const int (*jlo)[kPlainP], const int (*nw)[kPlainP],
-                                           int p, double* wyz, F f) {
+                                           const Plain<P>& sh, int p, double* wyz, F f) {
+  constexpr int kPlainS = P + 1;
+  const int (*jlo)[P] = sh.jlo;
+  const int (*nw)[P] = sh.nw;
   const int lane = threadIdx.x & 31;
   const int nx = nw[0][p], ny = nw[1][p], nz = nw[2][p], rows = ny * nz;
   const double* wy = w + kp.xs * kPlainS + p;
@@ -141,14 +211,14 @@ __device__ __forceinline__ void plain_walk(const erpp_kparams& kp, const double*
   }
 }
 
-// A block takes kPlainP particles: their weights first, a thread per particle
-// and axis, then a warp per particle.  The FP64 pipe bounds both kernels (2
+// A block takes P particles: their weights first, then a warp per particle.  The FP64 pipe bounds both kernels (2
 // lanes a clock on an SM, whatever the number of active lanes of an
 // instruction): per particle the exponentials are evaluated once per node and
 // axis instead of by all 32 lanes of a warp, the row weights once per row, and
 // a node costs one operation per component.  100k particles, 216 nodes each, on
 // 128^3: gather 1585 -> 302 us (100 us of it the weights), source 1480 -> 210 us
 // with the weights that the step's gather leaves in w64, 290 us without.
+template <int P>
 __global__ void __launch_bounds__(kWarps * 32) k_gather_f64(erpp_kparams kp, int64_t n,
                                                             const double* __restrict__ x0,
                                                             const double* __restrict__ x1,
@@ -158,28 +228,28 @@ __global__ void __launch_bounds__(kWarps * 32) k_gather_f64(erpp_kparams kp, int
                                                             double* __restrict__ keep,
                                                             uint32_t* err) {
   extern __shared__ double plain_smem[];
-  __shared__ int jlo[3][kPlainP], nw[3][kPlainP];
+  __shared__ Plain<P> sh;
+  constexpr int kPlainS = P + 1;
   double* const w = plain_smem;  // [3][xs][kPlainS]
   double* const rowbuf = w + 3 * kp.xs * kPlainS;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t p0 = (int64_t)blockIdx.x * kPlainP;
-  const int np = (int)min((int64_t)kPlainP, n - p0);
-  plain_weights(kp, p0, np, x0, x1, x2, w, jlo, nw, nullptr, err);
-  __syncthreads();
+  const int64_t p0 = (int64_t)blockIdx.x * P;
+  const int np = (int)min((int64_t)P, n - p0);
+  plain_weights<P>(kp, p0, np, x0, x1, x2, w, sh, nullptr, err);
   if (keep) {
-    double* dst = keep + (size_t)blockIdx.x * kept_doubles(kp.xs);
-    for (int i = threadIdx.x; i < 3 * kp.xs * kPlainP; i += blockDim.x)
-      dst[i] = w[(i / kPlainP) * kPlainS + (i & (kPlainP - 1))];
-    int2* win = reinterpret_cast<int2*>(dst + 3 * kp.xs * kPlainP);
-    for (int i = threadIdx.x; i < 3 * kPlainP; i += blockDim.x)
-      win[i] = make_int2(jlo[i / kPlainP][i & (kPlainP - 1)], nw[i / kPlainP][i & (kPlainP - 1)]);
+    double* dst = keep + (size_t)blockIdx.x * kept_doubles(kp.xs, P);
+    for (int i = threadIdx.x; i < 3 * kp.xs * P; i += blockDim.x)
+      dst[i] = w[(i / P) * kPlainS + (i & (P - 1))];
+    int2* win = reinterpret_cast<int2*>(dst + 3 * kp.xs * P);
+    for (int i = threadIdx.x; i < 3 * P; i += blockDim.x)
+      win[i] = make_int2(sh.jlo[i / P][i & (P - 1)], sh.nw[i / P][i & (P - 1)]);
   }
   const size_t nn = (size_t)kp.n[0] * kp.n[1] * kp.n[2];
   for (int p = warp; p < np; p += kWarps) {
     double a0 = 0.0, a1 = 0.0, a2 = 0.0;
-    if (nw[0][p] > 0 && nw[1][p] > 0 && nw[2][p] > 0) {
+    if (sh.nw[0][p] > 0 && sh.nw[1][p] > 0 && sh.nw[2][p] > 0) {
       double wx = 0.0;
-      plain_walk(kp, w, jlo, nw, p, rowbuf + warp * kRowBuf,
+      plain_walk<P>(kp, w, sh, p, rowbuf + warp * kRowBuf,
                  [&](double wl, double wr, size_t node) {
                    wx = wl;
                    a0 = fma(wr, __ldg(u + node), a0);
@@ -206,6 +276,7 @@ __global__ void __launch_bounds__(kWarps * 32) k_gather_f64(erpp_kparams kp, int
   }
 }
 
+template <int P>
 __global__ void __launch_bounds__(kWarps * 32) k_scatter_f64(erpp_kparams kp, int64_t n,
                                                              const double* __restrict__ x0,
                                                              const double* __restrict__ x1,
@@ -217,21 +288,21 @@ __global__ void __launch_bounds__(kWarps * 32) k_scatter_f64(erpp_kparams kp, in
                                                              const double* __restrict__ kept,
                                                              uint32_t* err) {
   extern __shared__ double plain_smem[];
-  __shared__ int jlo[3][kPlainP], nw[3][kPlainP];
+  __shared__ Plain<P> sh;
+  constexpr int kPlainS = P + 1;
   double* const w = plain_smem;  // [3][xs][kPlainS]
   double* const rowbuf = w + 3 * kp.xs * kPlainS;
   const int warp = threadIdx.x >> 5;
-  const int64_t p0 = (int64_t)blockIdx.x * kPlainP;
-  const int np = (int)min((int64_t)kPlainP, n - p0);
-  plain_weights(kp, p0, np, x0, x1, x2, w, jlo, nw, kept, err);
-  __syncthreads();
+  const int64_t p0 = (int64_t)blockIdx.x * P;
+  const int np = (int)min((int64_t)P, n - p0);
+  plain_weights<P>(kp, p0, np, x0, x1, x2, w, sh, kept, err);
   const size_t nn = (size_t)kp.n[0] * kp.n[1] * kp.n[2];
   for (int p = warp; p < np; p += kWarps) {
-    if (!(nw[0][p] > 0 && nw[1][p] > 0 && nw[2][p] > 0)) continue;
-    const double wl = w[((threadIdx.x & 31) % nw[0][p]) * kPlainS + p];
+    if (!(sh.nw[0][p] > 0 && sh.nw[1][p] > 0 && sh.nw[2][p] > 0)) continue;
+    const double wl = w[((threadIdx.x & 31) % sh.nw[0][p]) * kPlainS + p];
     const double f0 = fscale * D0[p0 + p] * wl, f1 = fscale * D1[p0 + p] * wl,
                  f2 = fscale * D2[p0 + p] * wl;
-    plain_walk(kp, w, jlo, nw, p, rowbuf + warp * kRowBuf, [&](double, double wr, size_t node) {
+    plain_walk<P>(kp, w, sh, p, rowbuf + warp * kRowBuf, [&](double, double wr, size_t node) {
       atomicAdd(S + node, f0 * wr);
       atomicAdd(S + nn + node, f1 * wr);
       atomicAdd(S + 2 * nn + node, f2 * wr);
@@ -239,9 +310,17 @@ __global__ void __launch_bounds__(kWarps * 32) k_scatter_f64(erpp_kparams kp, in
   }
 }
 
-size_t plain_smem_bytes(const erpp_kparams& kp) {
-  return sizeof(double) * ((size_t)3 * kp.xs * kPlainS + (size_t)kWarps * kRowBuf);
+size_t plain_smem_bytes(const erpp_kparams& kp, int P) {
+  return sizeof(double) * ((size_t)3 * kp.xs * (P + 1) + (size_t)kWarps * kRowBuf);
 }
+
+// Few particles: a warp for each, so that no warp walks one window after another
+// while SMs are idle.  Interpolation with blocks of 32 and of 8 in us, windows of 6
+// nodes: 1000 particles 27 and 14.5, 10k 48 and 39, 30k 108 and 97, 100k 301 and 311;
+// of 9: 54 and 19, 99 and 80, 232 and 212, 667 and 685; of 31: 1131 and 294, 2150 and
+// 1635, 5104 and 4486, 15086 and 14801.
+constexpr int64_t kFewMost = 50000;
+bool plain_few(int64_t n) { return n <= kFewMost; }
 
 // Weights of one axis and their second derivatives in the particle
 // coordinate (raw or normalised like axis_weights_f64), evaluated in FP64 and
@@ -541,9 +620,10 @@ cudaError_t launch_gather_f64(erpp_ctx* ctx, const double* u, int64_t n,
                               const double* const x[3], double* const up[3], bool keep,
                               cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  const unsigned blocks = (unsigned)((n + kPlainP - 1) / kPlainP);
+  const int P = plain_few(n) ? kPlainFew : kPlainMany;
+  auto kern = plain_few(n) ? k_gather_f64<kPlainFew> : k_gather_f64<kPlainMany>;
   ++ctx->launches;
-  k_gather_f64<<<blocks, kWarps * 32, plain_smem_bytes(ctx->kp), st>>>(
+  kern<<<(unsigned)((n + P - 1) / P), kWarps * 32, plain_smem_bytes(ctx->kp, P), st>>>(
       ctx->kp, n, x[0], x[1], x[2], u, up[0], up[1], up[2], keep ? ctx->w64 : nullptr, ctx->err);
   return cudaGetLastError();
 }
@@ -554,8 +634,10 @@ cudaError_t launch_gather_f64(erpp_ctx* ctx, const double* u, int64_t n,
 bool w64_reserve(erpp_ctx* ctx) {
   if (ctx->w64) return true;
   if (ctx->w64_refused || ctx->cap <= 0) return false;
-  const size_t blocks = (size_t)((ctx->cap + kPlainP - 1) / kPlainP);
-  if (cudaMalloc(&ctx->w64, sizeof(double) * kept_doubles(ctx->kp.xs) * blocks) != cudaSuccess) {
+  // whole blocks of either size
+  const size_t blocks = (size_t)((ctx->cap + kPlainMany - 1) / kPlainMany);
+  if (cudaMalloc(&ctx->w64, sizeof(double) * kept_doubles(ctx->kp.xs, kPlainMany) * blocks) !=
+      cudaSuccess) {
     cudaGetLastError();
     ctx->w64 = nullptr;
     ctx->w64_refused = true;
@@ -575,9 +657,10 @@ cudaError_t launch_scatter_f64(erpp_ctx* ctx, int64_t n, const double* const x[3
   cudaError_t e = cudaMemsetAsync(S, 0, sizeof(double) * 3 * nn, st);
   if (e != cudaSuccess) return e;
   if (n <= 0) return cudaSuccess;
-  const unsigned blocks = (unsigned)((n + kPlainP - 1) / kPlainP);
+  const int P = plain_few(n) ? kPlainFew : kPlainMany;
+  auto kern = plain_few(n) ? k_scatter_f64<kPlainFew> : k_scatter_f64<kPlainMany>;
   ++ctx->launches;
-  k_scatter_f64<<<blocks, kWarps * 32, plain_smem_bytes(kp), st>>>(
+  kern<<<(unsigned)((n + P - 1) / P), kWarps * 32, plain_smem_bytes(kp, P), st>>>(
       kp, n, x[0], x[1], x[2], D[0], D[1], D[2], fscale, S, kept ? ctx->w64 : nullptr, ctx->err);
   return cudaGetLastError();
 }
