@@ -303,13 +303,14 @@ __device__ __forceinline__ void bin_fill_one(const erpp_kparams& kp, int64_t i, 
     jlo[a] = c[a] + erpp_geo_off(pack, a);
     nw[a] = erpp_geo_nw(pack, a);
   }
-  int k = 0;
+  int k = 0, off = 0;  // off: the piece's place in its bin
   // x/y-halo tiles: each piece's place replaces its place in its bin, for the
   // gather's per-piece sums
   auto place = [&](int bin) -> int64_t {
     int64_t pos = cap;
     if (k < ms) {
-      pos = (int64_t)start[bin] + slot[(int64_t)k * n + i];
+      off = slot[(int64_t)k * n + i];
+      pos = (int64_t)start[bin] + off;
       if (kp.design == 4) slot[(int64_t)k * n + i] = pos < cap ? (int32_t)pos : 0;
     }
     ++k;
@@ -335,8 +336,7 @@ __device__ __forceinline__ void bin_fill_one(const erpp_kparams& kp, int64_t i, 
       if (pos < cap) {
         entries[pos] = make_int4((int)i, (int)pk, __float_as_int(d0y), __float_as_int(d0z));
         // the first piece of a further chunk of the gather's tile
-        const int off = (int)pos - start[tile];
-        if (items && off > 0 && off % ERPP_GATHER_CHUNK == 0)
+        if (off > 0 && (off & (ERPP_GATHER_CHUNK - 1)) == 0 && items)
           items[atomicAdd(nitems, 1)] = make_int2(tile, (int)pos);
       } else {
         erpp_set_err(err, ERPP_ERRBIT_BOUNDS);

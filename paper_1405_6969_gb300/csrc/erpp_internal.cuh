@@ -54,7 +54,7 @@
 #define ERPP_GEO_VALID 0x80000000u
 
 // Pieces of a tile that one block of the x/y-halo tile gather takes; a denser
-// tile's further chunks are listed by the binning.
+// tile's further chunks are listed by the binning (a power of two).
 #define ERPP_GATHER_CHUNK 1024
 
 // Particle indices are 31-bit; the packed piece base is 17 bits.

@@ -835,7 +835,12 @@ __device__ __forceinline__ int gather_tile4(
 // The first nextra blocks take the further chunks of dense tiles in turn (the
 // binning lists the pieces kGatherChunk, 2 kGatherChunk, ... of every tile), the
 // others a tile's first chunk each: a tile that holds a cluster is gathered by
-// many blocks (100k particles in 50 clusters: 700 us in one block per tile).
+// many blocks (100k particles in 50 clusters: 700 us in one block per tile).  The
+// other tiles pay for the blocks that find no chunk, so there is one per SM: 100k
+// particles in 50 clusters, a step 587 us with 608, 584 with 304, 564 with 152, 562
+// with 76 (but 100k in 80^3 68, 67, 67, 84 for a gather).  And they run straight
+// through code of their own: in the chunks' loop the gather of 100k particles in
+// 256^3 nodes took 94.3 us, now 90.6 (93.8 without further chunks).
 template <int XM, int LMIN, int XW, int NT, bool LAP, int PB>
 __global__ void __launch_bounds__(NT, LAP ? 2 : 768 / NT) k_gather4(
     erpp_kparams kp, const float* __restrict__ u, const __grid_constant__ CUtensorMap tmap,
@@ -847,17 +852,22 @@ __global__ void __launch_bounds__(NT, LAP ? 2 : 768 / NT) k_gather4(
   __shared__ SchedState ss;
   __shared__ __align__(8) uint64_t tma_bar;
   __shared__ __align__(8) uint64_t stall_bar;  // debug_stall only: never completed
-  const bool extra = (int)blockIdx.x < nextra;
-  const int nit = extra ? *nitems : 1;
-  for (int it = extra ? (int)blockIdx.x : 0; it < nit; it += nextra) {
-    const int tile = extra ? items[it].x : (int)blockIdx.x - nextra;
-    const int e0 = extra ? items[it].y : start[tile];
+  auto chunk = [&](int tile, int e0) {
     int e1 = (int)min((int64_t)start[tile + 1], ecap);
     if (nextra > 0) e1 = min(e1, e0 + ERPP_GATHER_CHUNK);
-    const int r = gather_tile4<XM, LMIN, XW, NT, LAP, PB>(kp, tile, u, &tmap, use_tma, e0, e1,
-                                                          entries, d0x, lapc, up_part, lap_part,
-                                                          err, smem_raw, ss, tma_bar, stall_bar);
-    if (!extra || (r & 1)) break;
+    return gather_tile4<XM, LMIN, XW, NT, LAP, PB>(kp, tile, u, &tmap, use_tma, e0, e1, entries,
+                                                   d0x, lapc, up_part, lap_part, err, smem_raw,
+                                                   ss, tma_bar, stall_bar);
+  };
+  if ((int)blockIdx.x >= nextra) {
+    const int tile = (int)blockIdx.x - nextra;
+    chunk(tile, start[tile]);
+    return;
+  }
+  const int nit = *nitems;
+  for (int it = (int)blockIdx.x; it < nit; it += nextra) {
+    const int r = chunk(items[it].x, items[it].y);
+    if (r & 1) break;
     __syncthreads();  // every thread is done with the tile and its barriers
     if (threadIdx.x == 0 && (r & 2)) {
       mbar_inval(&tma_bar);
@@ -1521,7 +1531,7 @@ cudaError_t gather4_nt(erpp_ctx* ctx, const float* u, cudaStream_t st) {
   const int use_tma = field_tensor_map(kp, u, &map) ? 1 : 0;
   ++ctx->launches;
   const int nextra =
-      ctx->gather_items ? (int)std::min<int64_t>(ctx->entries_cap / ERPP_GATHER_CHUNK, 608) : 0;
+      ctx->gather_items ? (int)std::min<int64_t>(ctx->entries_cap / ERPP_GATHER_CHUNK, 152) : 0;
   kern<<<kp.ntiles + nextra, NT, sm, st>>>(kp, u, map, use_tma, ctx->tile_start, ctx->entries,
                                            ctx->entries_cap, ctx->d0x, ctx->lapc, ctx->up_part,
                                            ctx->lap_part, nextra, ctx->tile_cnt + kp.ntiles,
