@@ -131,7 +131,7 @@ erpp_status ensure_capacity(erpp_ctx* c, int64_t n) {
     if (e == cudaSuccess && c->kp.design == 4 && c->kp.full_force)
       e = cudaMalloc(&c->lap_part, sizeof(float4) * (size_t)ecap);
     if (e == cudaSuccess) e = cudaMalloc(&c->piece_slot, sizeof(int32_t) * (size_t)ecap);
-    if (e == cudaSuccess && c->kp.design == 4)
+    if (e == cudaSuccess && c->kp.design == 4 && c->kp.weights == ERPP_W_GAUSS)
       e = cudaMalloc(&c->gather_items, sizeof(int2) * (size_t)(ecap / ERPP_GATHER_CHUNK + 1));
     c->entries_cap = ecap;
   }
