@@ -635,7 +635,8 @@ __device__ __forceinline__ void scatter_region(
       for (int k = 0; k < 2; ++k) acc[c][h][k].v = 0ull;
 
   // batches of equal size, so that none leaves the warps a nearly empty chunk
-  if (dense) nbatch = (total + kDenseBatch - 1) / kDenseBatch;
+  // (one, of none, where a brick around is long but nothing reaches these planes)
+  if (dense) nbatch = max(1, (total + kDenseBatch - 1) / kDenseBatch);
   const int bsize = (total + nbatch - 1) / nbatch;
 
   // Stages members q0, q0 + 1, ... of the queue as rows p0, p0 + 1, ...: LP lanes a particle,
