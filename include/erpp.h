@@ -206,7 +206,11 @@ erpp_status erpp_particle_advance(erpp_ctx* ctx, const double* const u_p[3],
 
 /* Regularised momentum source of forces D at positions x (Eq.
  * ns_regularized_filtered): S[c][j] = -(1/rho_f) sum_i D[c][i] W_i(j).
- * S (grid field) is overwritten entirely. */
+ * S (grid field) is overwritten entirely.
+ * A component of D that is NaN or infinite makes S so at the nodes of its
+ * particle's window in FP64 and in dense FP32 boxes; where they are sparse
+ * (tiles of up to 1024 pieces, which sum in fixed point, and regions of as few
+ * particles) it gives nothing. */
 erpp_status erpp_scatter_source(erpp_ctx* ctx, int64_t n, const double* const x[3],
                                 const double* const D[3], void* S, erpp_stream stream);
 

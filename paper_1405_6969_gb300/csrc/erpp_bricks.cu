@@ -388,6 +388,7 @@ __device__ __forceinline__ void split_pair(Pair v, uint32_t& h, uint32_t& l) {
 struct ScatShared {
   int cnt[kScatWarps];  // members each warp found that touch the region
   int maxbits;          // largest |force component| of the bricks around
+  int odd;              // a staged particle's force is not finite
 };
 
 // Dense regions: the segments one after the other as one range of candidates,
@@ -443,6 +444,58 @@ __device__ __forceinline__ bool touches(uint32_t w, uint32_t org, uint32_t ext1)
   return (((ext1 - lo) & hi) & 0x808080u) == 0x808080u;
 }
 
+// A region of more than this many particles (a quarter of one, kOddQuarter) passes
+// forces that are not finite on to the nodes in their windows; elsewhere such a
+// component gives nothing.  The tiles do the same: a tile of 64 x 16 x 4 nodes sums
+// up to 1024 pieces in fixed point, which has no such values, and more in FP32; a
+// region and a tile of the same density hold as many, a quarter 0.43 times.
+constexpr int kOddRegion = 1024, kOddQuarter = 440;
+
+// Adds them, after S has its finite sums: the whole block, a thread per particle of
+// the bricks around (seldom called, so that it keeps out of scatter_region's registers).
+__device__ __noinline__ void add_odd_forces(const erpp_kparams& kp, const erpp_brick_dims& bd,
+                                            const int gg0, const int gg1, const int gg2, int z0,
+                                            int zs, const int2* __restrict__ axis,
+                                            const uint32_t* __restrict__ win,
+                                            const float4* __restrict__ fs,
+                                            const int32_t* __restrict__ bstart, float* S) {
+  const int b[3] = {gg0 * kRegion, gg1 * kRegion, gg2 * kRegion + z0};
+  const int ext[3] = {min(kRegion, kp.n[0] - b[0]), min(kRegion, kp.n[1] - b[1]),
+                      min(zs, kp.n[2] - b[2])};
+  const int2* ax[3] = {axis + (size_t)gg0 * kMaxAxisSegs,
+                       axis + (size_t)(bd.ng[0] + gg1) * kMaxAxisSegs,
+                       axis + (size_t)(bd.ng[0] + bd.ng[1] + gg2) * kMaxAxisSegs};
+  const int ns[3] = {ax[0][kMaxAxisSegs - 1].x, ax[1][kMaxAxisSegs - 1].x,
+                     ax[2][kMaxAxisSegs - 1].x};
+  const size_t nxy = (size_t)kp.n[0] * kp.n[1], nn = nxy * kp.n[2];
+  for (int q = 0; q < ns[0] * ns[1] * ns[2]; ++q) {
+    const int2 e[3] = {ax[0][q % ns[0]], ax[1][q / ns[0] % ns[1]], ax[2][q / (ns[0] * ns[1])]};
+    const int id = brick_id(bd.ng, e[0].x, e[1].x, e[2].x);
+    for (int j = bstart[id] + threadIdx.x; j < bstart[id + 1]; j += blockDim.x) {
+      const uint32_t odd = __float_as_uint(fs[j].w);
+      if (odd == 0u) continue;
+      const uint32_t w = win[j];
+      int lo[3], from[3], to[3];
+      for (int a = 0; a < 3; ++a) {
+        lo[a] = erpp_rec_lo(w, a) + e[a].y - (a == 2 ? z0 : 0);
+        from[a] = max(lo[a], 0);
+        to[a] = min(lo[a] + erpp_rec_nw(w, a), ext[a]);
+      }
+      for (int c = 0; c < 3; ++c) {
+        const uint32_t k = (odd >> (3 * c)) & 7u;
+        if (k == 0u) continue;
+        const float v = k == 1u ? __int_as_float(0x7fffffff)
+                                : __int_as_float(k == 2u ? 0x7f800000 : (int)0xff800000);
+        for (int z = from[2]; z < to[2]; ++z)
+          for (int y = from[1]; y < to[1]; ++y)
+            for (int x = from[0]; x < to[0]; ++x)
+              atomicAdd(S + c * nn + (b[2] + z) * nxy + (size_t)(b[1] + y) * kp.n[0] + b[0] + x,
+                        v);
+      }
+    }
+  }
+}
+
 // LP: lanes that stage a particle, each two neighbouring nodes per axis: 4 for
 // windows of at most 7 nodes (at most 4 aligned pairs of nodes), else 8.
 // axis: per axis a and group g the stretches of bricks that hold the home
@@ -480,7 +533,10 @@ __device__ __forceinline__ void scatter_region(
   const int ns = min(nsx.x * nsy.x * nsz.x, kMaxSegs);
   const int K = (ns + kScatWarps - 1) / kScatWarps;  // segments per warp, at most 22
 
-  if (tid == 0) sh.maxbits = 0;
+  if (tid == 0) {
+    sh.maxbits = 0;
+    sh.odd = 0;
+  }
   if (tid < kPitch / 16)
     reinterpret_cast<uint4*>(row0 + kListBatch * kPitch)[tid] = make_uint4(0u, 0u, 0u, 0u);
   // Segment q: its brick's records, its first cell; returns the brick's
@@ -704,6 +760,7 @@ __device__ __forceinline__ void scatter_region(
             make_float2(v[1][0] * 16384.f, v[1][1] * 16384.f);
       if (in[2]) *reinterpret_cast<float2*>(wt + 16 + at[2]) = make_float2(v[2][0], v[2][1]);
       if (live && ql == 0) {
+        if (__float_as_uint(f.w) != 0u) sh.odd = 1;
         // the tiles whose rows and planes the window reaches: bit ZS / 2 yh + zp
         const int y1 = lo[1] + erpp_rec_nw(w, 1) - 1;
         const int za = max(lo[2], 0) >> 1, zb = min(lo[2] + erpp_rec_nw(w, 2) - 1, ZS - 1) >> 1;
@@ -817,8 +874,7 @@ __device__ __forceinline__ void scatter_region(
       for (int k = 0; k < 12; ++k) dst[32 * k] = acc[k / 4][(k / 2) & 1][k & 1];
     }
     __syncthreads();
-    if (part > 0) return;
-    for (int q = 0; q < kParts - 1; ++q) {
+    for (int q = 0; q < kParts - 1 && part == 0; ++q) {
       const Pair* src = sums + (q * kTiles + tile) * 12 * 32 + lane;
 #pragma unroll
       for (int k = 0; k < 12; ++k)
@@ -830,7 +886,7 @@ __device__ __forceinline__ void scatter_region(
   const size_t nxy = (size_t)kp.n[0] * kp.n[1], nn = nxy * kp.n[2];
   const int y = 8 * yh + gr;
   const bool pair = (kp.n[0] & 1) == 0 && (((uintptr_t)S) & 7) == 0;
-  if (y < ext[1]) {
+  if (y < ext[1] && part == 0) {
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int x = 8 * h + 2 * tq;
@@ -850,6 +906,10 @@ __device__ __forceinline__ void scatter_region(
         }
       }
     }
+  }
+  if (sh.odd && total > (ZS == kRegion ? kOddRegion : kOddQuarter)) {
+    __syncthreads();  // S has the block's finite sums
+    add_odd_forces(kp, bd, gg[0], gg[1], gg[2], z0, ZS, axis, win, fs, bstart, S);
   }
 }
 

@@ -551,15 +551,24 @@ __device__ __forceinline__ int erpp_rec_off(const erpp_kparams& kp, uint32_t w, 
 }
 
 // A particle's force for the source from sorted particles, stored at its
-// record's place (a component that is not finite gives no force), and the
-// brick's largest |component| (as the bits of a non-negative float).
+// record's place, and the brick's largest |component| (as the bits of a
+// non-negative float).  A component that is not finite is stored as zero; the
+// last word then says which they are (three bits a component: NaN, +inf, -inf).
 __device__ __forceinline__ void erpp_put_force(float4* __restrict__ fs,
                                                int32_t* __restrict__ bmax, int slot, int brick,
                                                float f0, float f1, float f2) {
-  f0 = isfinite(f0) ? f0 : 0.f;
-  f1 = isfinite(f1) ? f1 : 0.f;
-  f2 = isfinite(f2) ? f2 : 0.f;
-  fs[slot] = make_float4(f0, f1, f2, 0.f);
+  uint32_t odd = 0u;
+  if (!(isfinite(f0) && isfinite(f1) && isfinite(f2))) {
+    auto take = [&](float& f, int a) {
+      if (isfinite(f)) return;
+      odd |= (isnan(f) ? 1u : (f > 0.f ? 2u : 4u)) << (3 * a);
+      f = 0.f;
+    };
+    take(f0, 0);
+    take(f1, 1);
+    take(f2, 2);
+  }
+  fs[slot] = make_float4(f0, f1, f2, __uint_as_float(odd));
   const int m = __float_as_int(fmaxf(fabsf(f0), fmaxf(fabsf(f1), fabsf(f2))));
   if (m > bmax[brick]) atomicMax(&bmax[brick], m);
 }
