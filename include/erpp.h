@@ -455,15 +455,17 @@ erpp_status erpp_set_tiling(erpp_ctx* ctx, int32_t tile_y, int32_t tile_z, int32
 
 /* How the FP32 scatter (x/y-halo tiles) adds each tile's halo to its
  * neighbours (a tuning option: every mode computes the same sums up to the
- * order of FP32 additions, and each is reproducible bit for bit):
+ * order of FP32 additions, and each is reproducible bit for bit but for dense
+ * places, as MERGE says):
  *   ERPP_SCATTER_MERGE (default): one block per tile writes its interior to S
  *     and its halo to strips in a context buffer; two merge kernels then add
  *     the strips onto the neighbouring tiles' rims.  Boxes of at least 120
  *     regions of 16^3 nodes, or dense ones (16384 particles and a quarter per
  *     node), with windows of at most 10 nodes and without ERPP_KAHAN, take the
  *     source from particles sorted by 8^3-cell bricks instead: no tiles and no
- *     merges (bricks of more than 4096 particles are summed in the order in
- *     which the sort's counting arrived, as tiles of more than 1024 pieces are).
+ *     merges.  Bricks of more than 4096 particles are summed in the order in
+ *     which the sort's counting arrived, and tiles of more than 1024 pieces in
+ *     the order of their atomic additions, in every mode.
  *   ERPP_SCATTER_CLUSTER: the x-tiles of each (y, z) tile row run as one
  *     thread-block cluster, and every tile adds its x-neighbours' halo columns
  *     to its own rim straight from their shared memory (fixed order: own,

@@ -24,13 +24,18 @@
 // added by atomics, the region needs no halo, and S is written once.
 //
 // Precision.  Both factors are split into two FP16 numbers, v = h + l (h the
-// rounded value, l the rounded rest: 22 bits and the sign of the rest, an error
-// of at most 2^-24 |v|), and the three products h h', h l', l h' are summed in
-// FP32, 16 particles at a time; the chunks' sums are added in FP32 with
-// rounding (the tensor core truncates: accumulating through it, 125 chunks of
-// a dense cluster left an error of 1.5e-5).  The factors are scaled by powers
-// of two so that a term of 2^-17 of the largest is still split without
-// underflow.  The dropped l l' is below 2^-24 of its term.
+// rounded value, l the rounded rest: off by at most 2^-23 |v|, 2^-24.5 rms), and the
+// three products h h', h l', l h' are summed in FP32, 16 particles at a time; the
+// chunks' sums are added in FP32 with rounding (the tensor core truncates:
+// accumulating through it, 125 chunks of a dense cluster left an error of 1.5e-5).
+// The dropped l l' is at most 2^-22 of its term (|l| <= 2^-11 |v|), 2^-24.6 rms.  The
+// factors are scaled by powers of two so that a term of 2^-17 of the largest is
+// still split without underflow; a smaller one keeps an error of 2^-39 of the largest
+// (a tile's fixed point: 2^-31 of the sum of its forces).  Against 64 bits, S is at
+// most as far off as from the tiles, relative to the whole and to each node's own
+// terms: 100k particles in clusters 2.0e-7 of the whole and 4.8e-8 of a node's in the
+// median, tiles 1.5e-6 and 1.2e-7; 800k uniform ones 1.9e-7 and 3.6e-8, tiles 2.2e-7
+// and 4.1e-8; the same with forces spread over nine decades.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <stdlib.h>
@@ -206,7 +211,7 @@ __global__ void __launch_bounds__(256) k_brick_place(int64_t n, const int2* __re
 // SM has its regions anyway 96^3 378 and 485, 128^3 565 and 848 us.
 constexpr int kDenseBrick = 192;
 __device__ __forceinline__ bool dense_brick(int members, int64_t n) {
-  return members >= kDenseBrick && members > n / (8 * 152);
+  return members >= kDenseBrick && members > n / (8 * ERPP_SMS);
 }
 // Lists the regions that the members of a dense brick can reach, each once.
 __device__ __noinline__ void mark_dense(const erpp_kparams& kp, const erpp_brick_dims& bd, int id,
@@ -1224,7 +1229,7 @@ cudaError_t brick_scatter(erpp_ctx* c, float* S, cudaStream_t st) {
   if (e != cudaSuccess) return e;
   c->launches += 2;
   c->route |= ERPP_ROUTE_SOURCE;
-  constexpr int kResident = 2 * 152;
+  constexpr int kResident = 2 * ERPP_SMS;
   dkern<<<kResident, kScatThreads, sm, st>>>(c->kp, k.dims, k.ndense, k.dense, k.axis, k.rec, k.win,
                                        k.fs, k.start, k.bmax, S);
   // started beside the dense regions' kernel: its blocks wait for that one last

@@ -411,7 +411,7 @@ cudaError_t launch(erpp_ctx* c, const float* u, int64_t n, const AdjArgs& ag, cu
   const int rows_ok = (kp.n[0] & 3) == 0 && (((uintptr_t)u) & 15) == 0;
   const int box[3] = {G::PX, G::NY, G::NZ};
   const int use_tma = rows_ok && erpp::field_box_map(kp, u, box, &map) ? 1 : 0;
-  const int nextra = (int)std::min<int64_t>(n / G::kChunk, 608);
+  const int nextra = (int)std::min<int64_t>(n / G::kChunk, 4 * ERPP_SMS);
   ++c->launches;
   kern<<<(unsigned)(k.nbricks / G::TB + nextra), kThreads, sm, st>>>(
       kp, k.dims, u, map, use_tma, rows_ok, nextra, k.rec, k.start, k.nitems, k.items, ag, n,

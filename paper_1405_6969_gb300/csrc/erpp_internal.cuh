@@ -53,6 +53,9 @@
 // 22-26 = window length on x / y / z, bit 31 = valid.
 #define ERPP_GEO_VALID 0x80000000u
 
+// SMs of the part, for the sizes of grids (nothing else depends on it).
+#define ERPP_SMS 152
+
 // Pieces of a tile that one block of the x/y-halo tile gather takes; a denser
 // tile's further chunks are listed by the binning (a power of two).
 #define ERPP_GATHER_CHUNK 1024
@@ -217,8 +220,8 @@ struct erpp_ctx {
                           // chunks of dense tiles (tile, first record); their number
                           // follows tile_cnt and is cleared with it
   float* halo;            // scatter x-halo columns, [ntiles][3][T_z][T_y][xhlo + xhhi]
-  int32_t* tile_cnt;      // [32 ntiles + 2]: pieces per (tile, bucket) bin; gather_items'
-                          // number, and how many of them are taken
+  int32_t* tile_cnt;      // [nbins + 1]: pieces per bin (x/y-halo tiles: per tile, else
+                          // per tile and bucket); then gather_items' number
   int32_t* tile_start;    // [32 ntiles + 1]
   int32_t* piece_slot;    // [maxseg product][cap]: each piece's place in its bin
   int32_t* scan_tmp;      // [ceil(32 ntiles / 4096)] chunk totals of the scan

@@ -1531,7 +1531,9 @@ cudaError_t gather4_nt(erpp_ctx* ctx, const float* u, cudaStream_t st) {
   const int use_tma = field_tensor_map(kp, u, &map) ? 1 : 0;
   ++ctx->launches;
   const int nextra =
-      ctx->gather_items ? (int)std::min<int64_t>(ctx->entries_cap / ERPP_GATHER_CHUNK, 152) : 0;
+      ctx->gather_items
+          ? (int)std::min<int64_t>(ctx->entries_cap / ERPP_GATHER_CHUNK, ERPP_SMS)
+          : 0;
   kern<<<kp.ntiles + nextra, NT, sm, st>>>(kp, u, map, use_tma, ctx->tile_start, ctx->entries,
                                            ctx->entries_cap, ctx->d0x, ctx->lapc, ctx->up_part,
                                            ctx->lap_part, nextra, ctx->tile_cnt + kp.ntiles,
