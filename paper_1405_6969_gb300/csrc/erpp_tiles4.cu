@@ -308,18 +308,17 @@ struct Carve {
 // slots may reach past the last staged row.
 constexpr int kFieldPad = 16;
 
-// Schedule entries of up to NU units: whole rounds of 256, 384 or 512 threads.
-__host__ __device__ constexpr int sched_slots(int NU) {
-  return (NU + 511) / 512 * 512 > (NU + 383) / 384 * 384 ? (NU + 511) / 512 * 512
-                                                         : (NU + 383) / 384 * 384;
+// Schedule entries of up to NU units: whole rounds of NT threads (256 as 512).
+__host__ __device__ constexpr int sched_slots(int NU, int NT) {
+  return NT == 384 ? (NU + 383) / 384 * 384 : (NU + 511) / 512 * 512;
 }
 
 // The unit words, the schedule and the gather's piece accumulators are sized
 // for the tile's tz planes (a piece has at most tz units).
-template <int PB>
+template <int PB, int NT>
 __host__ __device__ inline size_t carve_bytes(int plane, int tz, int copies, bool gather,
                                               bool lap = false) {
-  const int NU = PB * tz, NS = sched_slots(NU);
+  const int NU = PB * tz, NS = sched_slots(NU, NT);
   size_t b = ((size_t)copies * plane + kFieldPad) * 4;
   b += (size_t)PB * 16;          // rec
   if (!gather) b += (size_t)PB * 16;  // fsb
@@ -333,10 +332,10 @@ __host__ __device__ inline size_t carve_bytes(int plane, int tz, int copies, boo
   return b;
 }
 
-template <int PB>
+template <int PB, int NT>
 __device__ inline Carve<PB> carve(unsigned char* base, int plane, int tz, int copies, bool gather,
                                   bool lap = false) {
-  const int NU = PB * tz, NS = sched_slots(NU);
+  const int NU = PB * tz, NS = sched_slots(NU, NT);
   Carve<PB> c;
   size_t o = 0;
   c.field = reinterpret_cast<float*>(base);
@@ -609,7 +608,7 @@ __device__ __forceinline__ int gather_tile4(
   static_assert(PB <= 1024, "unit words hold the piece index in 10 bits");
   if (e0 >= e1) return 0;
   const int tzs = kp.T[2];  // planes per tile: units per piece, at most
-  const Carve<PB> cv = carve<PB>(smem_raw, kp.plane, tzs, 3, true, LAP);
+  const Carve<PB> cv = carve<PB, NT>(smem_raw, kp.plane, tzs, 3, true, LAP);
   int b[3], ext[3], tt[3];
   tile_origin4(kp, tile, b, ext, tt);
   // one TMA box when the staged rows need no periodic wrap
@@ -836,11 +835,11 @@ __device__ __forceinline__ int gather_tile4(
 // binning lists the pieces kGatherChunk, 2 kGatherChunk, ... of every tile), the
 // others a tile's first chunk each: a tile that holds a cluster is gathered by
 // many blocks (100k particles in 50 clusters: 700 us in one block per tile).  The
-// other tiles pay for the blocks that find no chunk, so there is one per SM: 100k
-// particles in 50 clusters, a step 587 us with 608, 584 with 304, 564 with 152, 562
-// with 76 (but 100k in 80^3 68, 67, 67, 84 for a gather).  And they run straight
-// through code of their own: in the chunks' loop the gather of 100k particles in
-// 256^3 nodes took 94.3 us, now 90.6 (93.8 without further chunks).
+// other tiles pay for the blocks that find no chunk, so there are two per SM: with
+// 76, 152, 304 and 608, 100k particles in 50 clusters 370, 280, 272 and 269 us, 218k
+// in 50 others 278, 188, 158 and 161, 100k uniform ones in 256^3 nodes 91, 91, 92 and
+// 92.  And the tiles run straight through code of their own: in the chunks' loop those
+// last took 94 us (93.8 without further chunks).
 template <int XM, int LMIN, int XW, int NT, bool LAP, int PB>
 __global__ void __launch_bounds__(NT, LAP ? 2 : 768 / NT) k_gather4(
     erpp_kparams kp, const float* __restrict__ u, const __grid_constant__ CUtensorMap tmap,
@@ -1118,7 +1117,7 @@ __device__ __forceinline__ void scatter_tile4(const erpp_kparams& kp, int tile,
   constexpr int NW = NT / 32;
   constexpr int PB = Batch<XW>::kPB;
   static_assert(PB <= NT, "a batch holds at most one piece per thread");
-  const Carve<PB> cv = carve<PB>(smem_raw, kp.plane, kp.T[2], MODE == 1 ? 6 : 3, false);
+  const Carve<PB> cv = carve<PB, NT>(smem_raw, kp.plane, kp.T[2], MODE == 1 ? 6 : 3, false);
   float* smem = cv.field;
   const TileAcc ta =
       scatter_tile<XM, LMIN, XW, MODE, NT>(kp, tile, cv, ss, red, start, entries, ecap, d0x,
@@ -1522,7 +1521,7 @@ template <int XM, int LMIN, int XW, int NT, bool LAP, int PB>
 cudaError_t gather4_nt(erpp_ctx* ctx, const float* u, cudaStream_t st) {
   const erpp_kparams& kp = ctx->kp;
   if (LAP && (!ctx->lapc || !ctx->lap_part)) return cudaErrorInvalidValue;
-  const size_t sm = carve_bytes<PB>(kp.plane, kp.T[2], 3, true, LAP);
+  const size_t sm = carve_bytes<PB, NT>(kp.plane, kp.T[2], 3, true, LAP);
   auto kern = k_gather4<XM, LMIN, XW, NT, LAP, PB>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
@@ -1532,7 +1531,7 @@ cudaError_t gather4_nt(erpp_ctx* ctx, const float* u, cudaStream_t st) {
   ++ctx->launches;
   const int nextra =
       ctx->gather_items
-          ? (int)std::min<int64_t>(ctx->entries_cap / ERPP_GATHER_CHUNK, ERPP_SMS)
+          ? (int)std::min<int64_t>(ctx->entries_cap / ERPP_GATHER_CHUNK, 2 * ERPP_SMS)
           : 0;
   kern<<<kp.ntiles + nextra, NT, sm, st>>>(kp, u, map, use_tma, ctx->tile_start, ctx->entries,
                                            ctx->entries_cap, ctx->d0x, ctx->lapc, ctx->up_part,
@@ -1573,21 +1572,27 @@ cudaError_t gather4(erpp_ctx* ctx, const float* u, int64_t n, cudaStream_t st) {
   constexpr int PB = Batch<XW>::kPB;
   if constexpr (LAP) {
     const erpp_kparams& kp = ctx->kp;
-    if (gather_blocks_per_sm(carve_bytes<PB>(kp.plane, kp.T[2], 3, true, true)) < 2 &&
-        gather_blocks_per_sm(carve_bytes<PB / 2>(kp.plane, kp.T[2], 3, true, true)) >= 2)
+    if (gather_blocks_per_sm(carve_bytes<PB, 256>(kp.plane, kp.T[2], 3, true, true)) < 2 &&
+        gather_blocks_per_sm(carve_bytes<PB / 2, 384>(kp.plane, kp.T[2], 3, true, true)) >= 2)
       return gather4_nt<XM, LMIN, XW, 384, true, PB / 2>(ctx, u, st);
     return gather4_nt<XM, LMIN, XW, 256, true, PB>(ctx, u, st);
   } else {
     if (ctx->kp.nthreads == 512) return gather4_nt<XM, LMIN, XW, 512, false, PB>(ctx, u, st);
     const erpp_kparams& kp = ctx->kp;
-    if (gather_big_batch(carve_bytes<PB>(kp.plane, kp.T[2], 3, true),
-                         carve_bytes<2 * PB>(kp.plane, kp.T[2], 3, true)))
+    const size_t one = carve_bytes<PB, 256>(kp.plane, kp.T[2], 3, true);
+    // One block per SM only, two with half the pieces a batch (tiles of 64 x 18 x 4
+    // nodes with windows of 6: 138k particles in 128 x 274 x 76 nodes 86 -> 64 us;
+    // 63 us with 384 threads)
+    if (gather_blocks_per_sm(one) < 2 &&
+        gather_blocks_per_sm(carve_bytes<PB / 2, 256>(kp.plane, kp.T[2], 3, true)) >= 2)
+      return gather4_nt<XM, LMIN, XW, 256, false, PB / 2>(ctx, u, st);
+    if (gather_big_batch(one, carve_bytes<2 * PB, 256>(kp.plane, kp.T[2], 3, true)))
       return gather4_nt<XM, LMIN, XW, 256, false, 2 * PB>(ctx, u, st);
     // Shared memory for two blocks per SM only: 384 threads each where that
     // leaves fewer lanes idle in a batch's last round (512x256x256, 1M
     // particles, 64x16x4 tiles: 366 units a batch, 346 -> 329 us; 256^3, 1M:
     // 490 units, 306 us with 256 threads, 334 us with 384).
-    if (gather_blocks_per_sm(carve_bytes<PB>(kp.plane, kp.T[2], 3, true)) <= 2 &&
+    if (gather_blocks_per_sm(carve_bytes<PB, 384>(kp.plane, kp.T[2], 3, true)) == 2 &&
         gather_lanes(kp, n, PB, 384) < gather_lanes(kp, n, PB, 256))
       return gather4_nt<XM, LMIN, XW, 384, false, PB>(ctx, u, st);
     return gather4_nt<XM, LMIN, XW, 256, false, PB>(ctx, u, st);
@@ -1600,7 +1605,8 @@ cudaError_t gather4(erpp_ctx* ctx, const float* u, int64_t n, cudaStream_t st) {
 template <int XM, int LMIN, int XW, int MODE, int NT, bool CL>
 cudaError_t scatter4_mode(erpp_ctx* ctx, float* S, cudaStream_t st) {
   const erpp_kparams& kp = ctx->kp;
-  const size_t sm = carve_bytes<Batch<XW>::kPB>(kp.plane, kp.T[2], MODE == 1 ? 6 : 3, false);
+  const size_t sm =
+      carve_bytes<Batch<XW>::kPB, NT>(kp.plane, kp.T[2], MODE == 1 ? 6 : 3, false);
   auto kern = k_scatter4<XM, LMIN, XW, MODE, NT, CL>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
@@ -1638,10 +1644,15 @@ cudaError_t scatter4_mode(erpp_ctx* ctx, float* S, cudaStream_t st) {
 
 template <int XM, int LMIN, int XW, bool CL>
 cudaError_t scatter4(erpp_ctx* ctx, float* S, cudaStream_t st) {
-  const bool big = ctx->kp.nthreads == 512;
-  if (ctx->kp.kahan)
-    return big ? scatter4_mode<XM, LMIN, XW, 1, 512, CL>(ctx, S, st)
-               : scatter4_mode<XM, LMIN, XW, 1, 256, CL>(ctx, S, st);
+  const erpp_kparams& kp = ctx->kp;
+  const bool big = kp.nthreads == 512;
+  if (kp.kahan) {
+    // 512 threads also where the staged sums leave one block per SM (tiles of 32 x 16
+    // x 4 nodes with windows of 6, 393k particles in 32 x 367 x 467 nodes: 349 -> 303 us)
+    const size_t sm = carve_bytes<Batch<XW>::kPB, 256>(kp.plane, kp.T[2], 6, false);
+    return big || gather_blocks_per_sm(sm) < 2 ? scatter4_mode<XM, LMIN, XW, 1, 512, CL>(ctx, S, st)
+                                               : scatter4_mode<XM, LMIN, XW, 1, 256, CL>(ctx, S, st);
+  }
   return big ? scatter4_mode<XM, LMIN, XW, 0, 512, CL>(ctx, S, st)
              : scatter4_mode<XM, LMIN, XW, 0, 256, CL>(ctx, S, st);
 }
@@ -1794,10 +1805,10 @@ size_t smem_bytes4(const erpp_kparams& kp, int copies, bool gather) {
   const bool lap = gather && kp.full_force;
   const int tz = kp.plane / kp.pxy;
   if (gather)  // the smaller batch: the launch takes the larger only when it fits as well
-    return xw4(kp) == 8 ? carve_bytes<Batch<8>::kPB>(kp.plane, tz, copies, true, lap)
-                        : carve_bytes<Batch<16>::kPB>(kp.plane, tz, copies, true, lap);
-  return xw4(kp) == 8 ? carve_bytes<Batch<8>::kPB>(kp.plane, tz, copies, false, lap)
-                      : carve_bytes<Batch<16>::kPB>(kp.plane, tz, copies, false, lap);
+    return xw4(kp) == 8 ? carve_bytes<Batch<8>::kPB, 256>(kp.plane, tz, copies, true, lap)
+                        : carve_bytes<Batch<16>::kPB, 256>(kp.plane, tz, copies, true, lap);
+  return xw4(kp) == 8 ? carve_bytes<Batch<8>::kPB, 256>(kp.plane, tz, copies, false, lap)
+                      : carve_bytes<Batch<16>::kPB, 256>(kp.plane, tz, copies, false, lap);
 }
 
 template <bool LAP>
