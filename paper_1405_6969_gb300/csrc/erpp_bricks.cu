@@ -239,7 +239,13 @@ __device__ __noinline__ void mark_dense(const erpp_kparams& kp, const erpp_brick
     if (j > last) return;  // fewer regions than that
   }
   g = (at[2] * bd.ng[1] + at[1]) * bd.ng[0] + at[0];
-  if (atomicExch(&dflag[g], 1) == 0) dense[atomicAdd(ndense, 1)] = g;
+  if (atomicExch(&dflag[g], 1) != 0) return;
+  // a brick's own region, which takes longest, from the list's front, the others
+  // from its end
+  if (at[0] == br[0] >> 1 && at[1] == br[1] >> 1 && at[2] == br[2] >> 1)
+    dense[atomicAdd(&ndense[0], 1)] = g;
+  else
+    dense[bd.ng[0] * bd.ng[1] * bd.ng[2] - 1 - atomicAdd(&ndense[1], 1)] = g;
 }
 
 // Position j's particle moves to its rank (by index) among its brick's members.
@@ -940,7 +946,7 @@ __global__ void __launch_bounds__(kScatThreads, 2) k_brick_scatter(
 }
 
 // The dense regions by quarters of four planes, which the blocks take from a
-// counter, ndense[1].  A kernel of its own, beside which k_brick_scatter starts
+// counter, ndense[2].  A kernel of its own, beside which k_brick_scatter starts
 // at once: one kernel with both forms made the regions of a 512 x 256 x 256 box
 // with 1M particles 1.6% slower (438 and 431 us), and taking the quarters by a fixed
 // stride left clusters of 100k particles in 128^3 nodes at 400 - 470 us instead
@@ -956,13 +962,15 @@ __global__ void __launch_bounds__(kScatThreads, 2) k_brick_scatter_dense(
   __shared__ ScatShared sh;
   __shared__ int item;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  const int nd = 4 * *ndense;
+  const int front = ndense[0], nd = 4 * (front + ndense[1]);
+  const int last = bd.ng[0] * bd.ng[1] * bd.ng[2] - 1;
   for (;;) {
-    if (threadIdx.x == 0) item = atomicAdd(&ndense[1], 1);
+    if (threadIdx.x == 0) item = atomicAdd(&ndense[2], 1);
     __syncthreads();
     const int it = item;
     if (it >= nd) break;
-    const int g = dense[it >> 2], z0 = 4 * (it & 3);
+    const int k = it >> 2, z0 = 4 * (it & 3);
+    const int g = dense[k < front ? k : last - (k - front)];
     const int gg[3] = {g % bd.ng[0], (g / bd.ng[0]) % bd.ng[1], g / (bd.ng[0] * bd.ng[1])};
     if (gg[2] * kRegion + z0 < kp.n[2])
       scatter_region<LP, 4>(kp, bd, gg, z0, axis, rec, win, fs, bstart, bmax, nullptr, S, smem,
@@ -1014,7 +1022,12 @@ static bool bricks_possible(const erpp_ctx* c) {
 // tiles then hold thousands of pieces each).  One source by bricks and by tiles:
 // 64 regions, 16k particles (64^3) 51 and 44 us, but 64k 155 and 236 us; 125
 // regions, 20k (80^3) 36 and 46; 180, 20k (96 x 96 x 80) 32 and 43; 512, 30k
-// (128^3) 38 and 53 us.
+// (128^3) 38 and 53 us.  One stretch inside is the tiles': uniform clouds with windows
+// of 6 nodes at 0.06 to 0.11 particles per node, where tiles still sum up to 1024
+// pieces in fixed point; a step by tiles and by bricks in 96^3 nodes, 53k particles
+// 115 and 120 us, 88k 146 and 163 (128^3, 210k 247 and 276; 35k in 96^3 99 and 91, 133k
+// 271 and 215).  The same number in clusters takes the tiles 914 us and the bricks 280
+// (60k in 96^3), and the number alone doesn't tell which it is.
 constexpr int64_t kRegionsLeast = 120;
 static bool bricks_serve(const erpp_ctx* c, int64_t n) {
   if (!c->bk.cnt || c->scatter_mode != ERPP_SCATTER_MERGE || n <= 0) return false;
@@ -1024,7 +1037,7 @@ static bool bricks_serve(const erpp_ctx* c, int64_t n) {
 }
 
 static size_t table_bytes(int nbricks) {
-  return sizeof(int32_t) * (2 * (size_t)nbricks + 3 + (size_t)(nbricks / 8));
+  return sizeof(int32_t) * (2 * (size_t)nbricks + 4 + (size_t)(nbricks / 8));
 }
 
 cudaError_t bricks_alloc_tables(erpp_ctx* c) {
@@ -1045,7 +1058,7 @@ cudaError_t bricks_alloc_tables(erpp_ctx* c) {
   k.bmax = k.cnt ? k.cnt + k.nbricks : nullptr;
   k.nitems = k.cnt ? k.cnt + 2 * (size_t)k.nbricks : nullptr;
   k.ndense = k.cnt ? k.nitems + 1 : nullptr;
-  k.dflag = k.cnt ? k.nitems + 3 : nullptr;
+  k.dflag = k.cnt ? k.nitems + 4 : nullptr;
   if (e == cudaSuccess) e = cudaMalloc(&k.dense, sizeof(int32_t) * (size_t)(k.nbricks / 8));
   std::vector<int2> ax;
   for (int a = 0; a < 3; ++a)

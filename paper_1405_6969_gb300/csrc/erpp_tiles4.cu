@@ -835,11 +835,12 @@ __device__ __forceinline__ int gather_tile4(
 // binning lists the pieces kGatherChunk, 2 kGatherChunk, ... of every tile), the
 // others a tile's first chunk each: a tile that holds a cluster is gathered by
 // many blocks (100k particles in 50 clusters: 700 us in one block per tile).  The
-// other tiles pay for the blocks that find no chunk, so there are two per SM: with
-// 76, 152, 304 and 608, 100k particles in 50 clusters 370, 280, 272 and 269 us, 218k
-// in 50 others 278, 188, 158 and 161, 100k uniform ones in 256^3 nodes 91, 91, 92 and
-// 92.  And the tiles run straight through code of their own: in the chunks' loop those
-// last took 94 us (93.8 without further chunks).
+// other tiles pay little for the blocks that find no chunk, so that there are more than
+// fit on the SMs: with 76, 152, 304 and 608, 100k particles in 50 clusters 370, 280, 272
+// and 269 us, 218k in 50 others 278, 188, 158 and 161, 400k with windows of 9 where three
+// blocks fit on an SM 860 us with 304 and 730 with 608 (the whole call), 100k uniform ones
+// in 256^3 nodes 91, 91, 92 and 92.  And the tiles run straight through code of their own:
+// in the chunks' loop those last took 94 us (93.8 without further chunks).
 template <int XM, int LMIN, int XW, int NT, bool LAP, int PB>
 __global__ void __launch_bounds__(NT, LAP ? 2 : 768 / NT) k_gather4(
     erpp_kparams kp, const float* __restrict__ u, const __grid_constant__ CUtensorMap tmap,
@@ -1531,7 +1532,7 @@ cudaError_t gather4_nt(erpp_ctx* ctx, const float* u, cudaStream_t st) {
   ++ctx->launches;
   const int nextra =
       ctx->gather_items
-          ? (int)std::min<int64_t>(ctx->entries_cap / ERPP_GATHER_CHUNK, 2 * ERPP_SMS)
+          ? (int)std::min<int64_t>(ctx->entries_cap / ERPP_GATHER_CHUNK, 4 * ERPP_SMS)
           : 0;
   kern<<<kp.ntiles + nextra, NT, sm, st>>>(kp, u, map, use_tma, ctx->tile_start, ctx->entries,
                                            ctx->entries_cap, ctx->d0x, ctx->lapc, ctx->up_part,
@@ -1582,17 +1583,20 @@ cudaError_t gather4(erpp_ctx* ctx, const float* u, int64_t n, cudaStream_t st) {
     const size_t one = carve_bytes<PB, 256>(kp.plane, kp.T[2], 3, true);
     // One block per SM only, two with half the pieces a batch (tiles of 64 x 18 x 4
     // nodes with windows of 6: 138k particles in 128 x 274 x 76 nodes 86 -> 64 us;
-    // 63 us with 384 threads)
-    if (gather_blocks_per_sm(one) < 2 &&
-        gather_blocks_per_sm(carve_bytes<PB / 2, 256>(kp.plane, kp.T[2], 3, true)) >= 2)
-      return gather4_nt<XM, LMIN, XW, 256, false, PB / 2>(ctx, u, st);
+    // 63 us with 384 threads).  Longer windows' batches are half as long already, and
+    // halved leave lanes idle (windows of 9, the same box, clusters: 321 -> 369 us).
+    if constexpr (XW <= 8) {
+      if (gather_blocks_per_sm(one) < 2 &&
+          gather_blocks_per_sm(carve_bytes<PB / 2, 256>(kp.plane, kp.T[2], 3, true)) >= 2)
+        return gather4_nt<XM, LMIN, XW, 256, false, PB / 2>(ctx, u, st);
+    }
     if (gather_big_batch(one, carve_bytes<2 * PB, 256>(kp.plane, kp.T[2], 3, true)))
       return gather4_nt<XM, LMIN, XW, 256, false, 2 * PB>(ctx, u, st);
     // Shared memory for two blocks per SM only: 384 threads each where that
     // leaves fewer lanes idle in a batch's last round (512x256x256, 1M
     // particles, 64x16x4 tiles: 366 units a batch, 346 -> 329 us; 256^3, 1M:
     // 490 units, 306 us with 256 threads, 334 us with 384).
-    if (gather_blocks_per_sm(carve_bytes<PB, 384>(kp.plane, kp.T[2], 3, true)) == 2 &&
+    if (gather_blocks_per_sm(carve_bytes<PB, 384>(kp.plane, kp.T[2], 3, true)) <= 2 &&
         gather_lanes(kp, n, PB, 384) < gather_lanes(kp, n, PB, 256))
       return gather4_nt<XM, LMIN, XW, 384, false, PB>(ctx, u, st);
     return gather4_nt<XM, LMIN, XW, 256, false, PB>(ctx, u, st);
