@@ -218,7 +218,9 @@ __device__ __forceinline__ bool dense_brick(int members, int64_t n) {
 // of its first 64 members the r-th of up to 4 x 4 x 4 (one member listed them all, one
 // atomic after the other, while the rest of the sort had long been done: 10.5k
 // particles in 50 clusters, k_brick_order 21.5 us, now 8.8).
-__device__ __noinline__ void mark_dense(const erpp_kparams& kp, const erpp_brick_dims& bd, int id,
+// Called instead of inlined it cost the ranking's registers: 400k particles in clusters
+// 112 us instead of 84.
+__device__ __forceinline__ void mark_dense(const erpp_kparams& kp, const erpp_brick_dims& bd, int id,
                                         int r, int32_t* ndense, int32_t* dense, int32_t* dflag) {
   int g = id >> 3;
   const int br[3] = {2 * (g % bd.ng[0]) + (id & 1), 2 * ((g / bd.ng[0]) % bd.ng[1]) + ((id >> 1) & 1),
@@ -239,13 +241,7 @@ __device__ __noinline__ void mark_dense(const erpp_kparams& kp, const erpp_brick
     if (j > last) return;  // fewer regions than that
   }
   g = (at[2] * bd.ng[1] + at[1]) * bd.ng[0] + at[0];
-  if (atomicExch(&dflag[g], 1) != 0) return;
-  // a brick's own region, which takes longest, from the list's front, the others
-  // from its end
-  if (at[0] == br[0] >> 1 && at[1] == br[1] >> 1 && at[2] == br[2] >> 1)
-    dense[atomicAdd(&ndense[0], 1)] = g;
-  else
-    dense[bd.ng[0] * bd.ng[1] * bd.ng[2] - 1 - atomicAdd(&ndense[1], 1)] = g;
+  if (atomicExch(&dflag[g], 1) == 0) dense[atomicAdd(ndense, 1)] = g;
 }
 
 // Position j's particle moves to its rank (by index) among its brick's members.
@@ -946,7 +942,7 @@ __global__ void __launch_bounds__(kScatThreads, 2) k_brick_scatter(
 }
 
 // The dense regions by quarters of four planes, which the blocks take from a
-// counter, ndense[2].  A kernel of its own, beside which k_brick_scatter starts
+// counter, ndense[1].  A kernel of its own, beside which k_brick_scatter starts
 // at once: one kernel with both forms made the regions of a 512 x 256 x 256 box
 // with 1M particles 1.6% slower (438 and 431 us), and taking the quarters by a fixed
 // stride left clusters of 100k particles in 128^3 nodes at 400 - 470 us instead
@@ -962,15 +958,13 @@ __global__ void __launch_bounds__(kScatThreads, 2) k_brick_scatter_dense(
   __shared__ ScatShared sh;
   __shared__ int item;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  const int front = ndense[0], nd = 4 * (front + ndense[1]);
-  const int last = bd.ng[0] * bd.ng[1] * bd.ng[2] - 1;
+  const int nd = 4 * *ndense;
   for (;;) {
-    if (threadIdx.x == 0) item = atomicAdd(&ndense[2], 1);
+    if (threadIdx.x == 0) item = atomicAdd(&ndense[1], 1);
     __syncthreads();
     const int it = item;
     if (it >= nd) break;
-    const int k = it >> 2, z0 = 4 * (it & 3);
-    const int g = dense[k < front ? k : last - (k - front)];
+    const int g = dense[it >> 2], z0 = 4 * (it & 3);
     const int gg[3] = {g % bd.ng[0], (g / bd.ng[0]) % bd.ng[1], g / (bd.ng[0] * bd.ng[1])};
     if (gg[2] * kRegion + z0 < kp.n[2])
       scatter_region<LP, 4>(kp, bd, gg, z0, axis, rec, win, fs, bstart, bmax, nullptr, S, smem,
@@ -1037,7 +1031,7 @@ static bool bricks_serve(const erpp_ctx* c, int64_t n) {
 }
 
 static size_t table_bytes(int nbricks) {
-  return sizeof(int32_t) * (2 * (size_t)nbricks + 4 + (size_t)(nbricks / 8));
+  return sizeof(int32_t) * (2 * (size_t)nbricks + 3 + (size_t)(nbricks / 8));
 }
 
 cudaError_t bricks_alloc_tables(erpp_ctx* c) {
@@ -1058,7 +1052,7 @@ cudaError_t bricks_alloc_tables(erpp_ctx* c) {
   k.bmax = k.cnt ? k.cnt + k.nbricks : nullptr;
   k.nitems = k.cnt ? k.cnt + 2 * (size_t)k.nbricks : nullptr;
   k.ndense = k.cnt ? k.nitems + 1 : nullptr;
-  k.dflag = k.cnt ? k.nitems + 4 : nullptr;
+  k.dflag = k.cnt ? k.nitems + 3 : nullptr;
   if (e == cudaSuccess) e = cudaMalloc(&k.dense, sizeof(int32_t) * (size_t)(k.nbricks / 8));
   std::vector<int2> ax;
   for (int a = 0; a < 3; ++a)

@@ -157,11 +157,10 @@ struct erpp_bricks {
   int32_t* ord;     // [cap] in order: particle (sorts for the adjoint)
   int2* items;      // further chunks of dense adjoint tiles: tile, first record
   int32_t* nitems;  // their number (after bmax, cleared with it)
-  int32_t* ndense;  // regions near a dense brick: how many hold one, how many others, the
-                    //   quarters taken so far, and a flag per region
+  int32_t* ndense;  // regions near a dense brick: their number, the quarters taken so
+                    //   far, and a flag per region
   int32_t* dflag;   //   (cleared with the counts)
-  int32_t* dense;   // [nbricks / 8] the regions: those that hold a dense brick, and from
-                    //   the end the others
+  int32_t* dense;   // [nbricks / 8] the regions
   float4* rec;      // [cap] records in order: fractional position, window word
   uint32_t* win;    // [cap] the window words alone
   float4* rec_in;   // [cap] records in input order (scratch of the sort)
