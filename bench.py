@@ -637,9 +637,9 @@ def main():
     # the scatter phase against the measured rate of the shared-memory add it
     # accumulates with: each stencil node of each particle receives one
     # contribution per force component (one 32-bit add, two with the split
-    # words of the compensated form)
+    # words of the compensated form); the source from bricks has no such adds
     atomics = None
-    if nsteps > 0 and args.weights == "gaussian":
+    if nsteps > 0 and args.weights == "gaussian" and "source" not in ctx.debug_last_route():
         from paper_1405_6969_gb300 import shared_add_rate
         peak_s32 = shared_add_rate("s32")
         updates = 3 * (nodes_per_step // 2)
