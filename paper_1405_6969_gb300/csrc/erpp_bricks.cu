@@ -220,8 +220,9 @@ __device__ __forceinline__ bool dense_brick(int members, int64_t n) {
 // particles in 50 clusters, k_brick_order 21.5 us, now 8.8).
 // Called instead of inlined it cost the ranking's registers: 400k particles in clusters
 // 112 us instead of 84.
-__device__ __forceinline__ void mark_dense(const erpp_kparams& kp, const erpp_brick_dims& bd, int id,
-                                        int r, int32_t* ndense, int32_t* dense, int32_t* dflag) {
+__device__ __forceinline__ void mark_dense(const erpp_kparams& kp, const erpp_brick_dims& bd,
+                                           int id, int r, int32_t* ndense, int32_t* dense,
+                                           int32_t* dflag) {
   int g = id >> 3;
   const int br[3] = {2 * (g % bd.ng[0]) + (id & 1), 2 * ((g / bd.ng[0]) % bd.ng[1]) + ((id >> 1) & 1),
                      2 * (g / (bd.ng[0] * bd.ng[1])) + ((id >> 2) & 1)};

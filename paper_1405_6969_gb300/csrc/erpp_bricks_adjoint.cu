@@ -102,12 +102,11 @@ __device__ __forceinline__ int wrap_near(int j, int n) {
 
 // Copies of the tile's box by the whole block where one TMA box cannot: 16 bytes
 // a thread (nx a multiple of 4, u 16-byte aligned; no four words straddle the
-// box's end), else word by word.
-// Both are calls: inlined, they made the kernel of 100k
-// particles with windows of 9 nodes 20 us longer.
+// box's end), else word by word.  Both are calls: inlined, they made the kernel of
+// 100k particles with windows of 9 nodes 20 us longer.
 template <class G>
-__device__ __noinline__ void stage_rows(const erpp_kparams& kp, const float* __restrict__ u, float* field,
-                           const int b[3]) {
+__device__ __noinline__ void stage_rows(const erpp_kparams& kp, const float* __restrict__ u,
+                                         float* field, const int b[3]) {
   const size_t nn = (size_t)kp.n[0] * kp.n[1] * kp.n[2];
   const int gx0 = wrap_mod(b[0] - 4, kp.n[0]);
   constexpr int kQ = G::PX / 4;
